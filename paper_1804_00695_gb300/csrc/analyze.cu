@@ -227,8 +227,9 @@ int launch_compress(const spgemm_csr &M, int2 *pairs, int32_t *ccnt, int2 *minma
 constexpr int AN_G = 8;
 __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
                           const int64_t *__restrict__ arp, const int32_t *__restrict__ acol,
-                          const int2 *__restrict__ ana, int64_t *__restrict__ flops,
-                          uint8_t *__restrict__ bins, int64_t *__restrict__ crp, DevState *st) {
+                          const int2 *__restrict__ ana, const int2 *__restrict__ bmm, int64_t *__restrict__ flops,
+                          uint8_t *__restrict__ bins, int64_t *__restrict__ crp, int2 *__restrict__ rspan,
+                          DevState *st) {
     __shared__ unsigned long long hist[NBINS];
     __shared__ unsigned long long fsum;
     __shared__ unsigned long long alen_max;
@@ -246,18 +247,23 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
         const int64_t i = i0 + threadIdx.x / AN_G;
         const bool live = i < nrows;
         long long f = 0, cp = 0;
+        int lo = INT_MAX, hi = -1;
         if (live) {
             for (int64_t p = arp[i] + lane; p < arp[i + 1]; p += AN_G) {
                 int k = acol[p];
                 if (k < 0 || (int64_t)k >= nrows_b) { bad = true; continue; }
-                const int2 d = ana[k];
+                const int2 d = ana[k], m = bmm[k];
                 f += d.x;
                 cp += d.y;
+                lo = min(lo, m.x);
+                hi = max(hi, m.y);
             }
         }
         for (int d = AN_G / 2; d > 0; d >>= 1) {
             f += __shfl_xor_sync(gmask, f, d, AN_G);
             cp += __shfl_xor_sync(gmask, cp, d, AN_G);
+            lo = min(lo, __shfl_xor_sync(gmask, lo, d, AN_G));
+            hi = max(hi, __shfl_xor_sync(gmask, hi, d, AN_G));
         }
         int b = BIN_EMPTY;
         const bool lead = live && lane == 0;
@@ -266,6 +272,7 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
             b = sym_bin(keys, cp);
             flops[i] = f;
             bins[i] = (uint8_t)b;
+            rspan[i] = make_int2(lo, hi >= lo ? hi - lo + 1 : 0);
             if (b == BIN_EMPTY) crp[i + 1] = 0;
             if (b == BIN_HUGE) crp[i + 1] = -1;
             wf += f;
@@ -292,8 +299,8 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
     }
 }
 
-int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, int64_t *flops,
-                   uint8_t *bins, int64_t *crp, DevState *st, Ctx &c) {
+int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, const int2 *bmm, int64_t *flops,
+                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     int64_t threads = A.nrows * AN_G;
     int64_t blocks = (threads + 255) / 256;
@@ -301,40 +308,7 @@ int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, in
     int64_t nwords = (B.ncols + 31) / 32;
     c.begin("analyze", A.nrows);
     k_analyze<<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, B.nrows, nwords, A.row_ptr, A.col_idx,
-                                                   ana, flops, bins, crp, st);
-    c.end();
-    SG_CUDA(cudaGetLastError());
-    return SPGEMM_OK;
-}
-
-__global__ void k_list_spans(const int64_t *__restrict__ arp, const int32_t *__restrict__ acol,
-                             const int2 *__restrict__ bmm, const int32_t *__restrict__ rows, int64_t count,
-                             int2 *__restrict__ spans) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < count; t += warps) {
-        const int i = rows[t];
-        int lo = INT_MAX, hi = -1;
-        for (int64_t p = arp[i] + lane; p < arp[i + 1]; p += 32) {
-            const int2 m = bmm[acol[p]];
-            lo = min(lo, m.x);
-            hi = max(hi, m.y);
-        }
-        for (int d = 16; d > 0; d >>= 1) {
-            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-        }
-        if (lane == 0) spans[t] = make_int2(lo, hi >= lo ? hi - lo + 1 : 0);
-    }
-}
-
-int launch_list_spans(const spgemm_csr &A, const int2 *bmm, const int32_t *rows, int64_t count, int2 *spans,
-                      Ctx &c) {
-    if (count <= 0) return SPGEMM_OK;
-    int64_t blocks = (count + 7) / 8;
-    blocks = std::min<int64_t>(blocks, (int64_t)c.nsm * 16);
-    c.begin("list_spans", count);
-    k_list_spans<<<(unsigned)blocks, 256, 0, c.s>>>(A.row_ptr, A.col_idx, bmm, rows, count, spans);
+                                                   ana, bmm, flops, bins, crp, rspan, st);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
@@ -376,9 +350,12 @@ int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, i
 // ---------------------------------------------------------------- numeric bins
 __global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
                                   const int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
-                                  DevState *st, const int32_t *__restrict__ nlo) {
+                                  uint8_t *__restrict__ cls, const int2 *__restrict__ rspan, DevState *st,
+                                  const int32_t *__restrict__ nlo) {
     __shared__ unsigned long long hist[NBINS];
+    __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS];
     if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
+    if (threadIdx.x < NCLS) ccnt[threadIdx.x] = cnnz[threadIdx.x] = cwords[threadIdx.x] = 0;
     __syncthreads();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int b = BIN_EMPTY;
@@ -389,70 +366,92 @@ __global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
         if (b != BIN_EMPTY && nlo && nlo[i] >= 0 && c <= NARROW_NMAX && f <= NARROW_FLOPS) b = BIN_NARROW;
         bins[i] = (uint8_t)b;
         if (b == BIN_HUGE) atomicMax((unsigned long long *)&st->max_row_nnz, (unsigned long long)c);
+        int k = CLS_NONE;
+        if (b >= 2 && b <= BIN_HUGE) {
+            const int words = rspan[i].y;
+            k = num_cls(b, c, f, words);
+            atomicAdd(&ccnt[k], 1);
+            if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
+            if (words > cwords[k]) atomicMax(&cwords[k], words);
+        }
+        cls[i] = (uint8_t)k;
     }
     warp_hist(hist, i < n, b);
     __syncthreads();
     if (threadIdx.x < NBINS && hist[threadIdx.x])
         atomicAdd((unsigned long long *)&st->bin_count[1][threadIdx.x], hist[threadIdx.x]);
+    if (threadIdx.x < NCLS && ccnt[threadIdx.x]) {
+        atomicAdd((unsigned long long *)&st->cls_count[threadIdx.x], (unsigned long long)ccnt[threadIdx.x]);
+        if (cnnz[threadIdx.x] > *(volatile int *)&st->cls_nnz[threadIdx.x])
+            atomicMax(&st->cls_nnz[threadIdx.x], cnnz[threadIdx.x]);
+        if (cwords[threadIdx.x] > *(volatile int *)&st->cls_words[threadIdx.x])
+            atomicMax(&st->cls_words[threadIdx.x], cwords[threadIdx.x]);
+    }
 }
 
-int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins,
-                           DevState *st, Ctx &c, const int32_t *nlo) {
+int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
+                           const int2 *rspan, DevState *st, Ctx &c, const int32_t *nlo) {
     if (n == 0) return SPGEMM_OK;
     c.begin("numeric_binning", n);
-    k_numeric_binning<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, crp, flops, bins, st, nlo);
+    k_numeric_binning<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, crp, flops, bins, cls, rspan, st, nlo);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
-// Row lists for the list-driven kernels.  phase 0 (symbolic second pass):
+// Row lists for the list-driven kernels.  CLS false (symbolic second pass):
 // rows marked -1 in crp[i+1] (overflowed the first pass, or bin 6), listed by
-// max(bins[i], 2).  phase 1 (numeric): rows of bins first_bin..6.  Within a warp the
-// lanes with the same bin reserve their slots with one atomic
-// (__match_any_sync), so rows stay in ascending order inside each warp.
-__global__ void k_scatter_bins(int64_t n, const uint8_t *__restrict__ bins,
-                               const int64_t *__restrict__ crp, int32_t *__restrict__ rows,
-                               DevState *st, int phase, int first_bin) {
-    __shared__ long long off[NBINS];
+// max(key[i], 2), key the bins.  CLS true (numeric): rows of the classes
+// `first` and up, key the classes.  Within a warp the lanes with the same
+// list reserve their slots with one atomic (__match_any_sync), so rows stay
+// in ascending order inside each warp.
+template <bool CLS>
+__global__ void k_scatter_rows(int64_t n, const uint8_t *__restrict__ key, const int64_t *__restrict__ crp,
+                               int32_t *__restrict__ rows, DevState *st, int first) {
+    constexpr int NL = CLS ? (int)NCLS : (int)NBINS;
+    __shared__ long long off[NL];
+    long long *cursor = CLS ? st->cls_cursor : st->bin_cursor;
     if (threadIdx.x == 0) {
         long long o = 0;
-        for (int b = 0; b < NBINS; b++) {
+        for (int b = 0; b < NL; b++) {
             off[b] = o;
-            if (b >= (phase == 0 ? 2 : first_bin) && b <= BIN_HUGE) o += st->bin_count[phase][b];
+            if (b >= first && (CLS || b <= BIN_HUGE)) o += CLS ? st->cls_count[b] : st->bin_count[0][b];
         }
     }
     __syncthreads();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int b = BIN_EMPTY;
+    int b = 0;   // none
     if (i < n) {
-        if (phase == 0) {
-            if (crp[i + 1] < 0) b = max((int)bins[i], 2);
-        } else {
-            int x = bins[i];
-            if (x >= first_bin && x <= BIN_HUGE) b = x;
-        }
+        if (CLS) b = key[i] >= first ? key[i] : 0;
+        else if (crp[i + 1] < 0) b = max((int)key[i], first);
     }
-    unsigned act = __ballot_sync(0xffffffffu, b != BIN_EMPTY);
-    if (b == BIN_EMPTY) return;
+    unsigned act = __ballot_sync(0xffffffffu, b != 0);
+    if (b == 0) return;
     unsigned peers = __match_any_sync(act, b);
     int lane = threadIdx.x & 31;
     int leader = __ffs(peers) - 1;
     long long base = 0;
-    if (lane == leader) base = atomicAdd((unsigned long long *)&st->bin_cursor[b],
-                                         (unsigned long long)__popc(peers));
+    if (lane == leader) base = atomicAdd((unsigned long long *)&cursor[b], (unsigned long long)__popc(peers));
     base = __shfl_sync(peers, base, leader);
     int rank = __popc(peers & ((1u << lane) - 1));
     rows[off[b] + base + rank] = (int32_t)i;
 }
 
-int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows,
-                        DevState *st, int phase, Ctx &c, int first_bin) {
+int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows, DevState *st, Ctx &c) {
     if (n == 0) return SPGEMM_OK;
     SG_CUDA(cudaMemsetAsync(st->bin_cursor, 0, sizeof(st->bin_cursor), c.s));
     c.begin("scatter_bins", n);
-    k_scatter_bins<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, bins, crp, rows, st, phase,
-                                                                   first_bin);
+    k_scatter_rows<false><<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, bins, crp, rows, st, 2);
+    c.end();
+    SG_CUDA(cudaGetLastError());
+    return SPGEMM_OK;
+}
+
+int launch_scatter_cls(int64_t n, const uint8_t *cls, int32_t *rows, DevState *st, int first_cls, Ctx &c) {
+    if (n == 0) return SPGEMM_OK;
+    SG_CUDA(cudaMemsetAsync(st->cls_cursor, 0, sizeof(st->cls_cursor), c.s));
+    c.begin("scatter_cls", n);
+    k_scatter_rows<true><<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, cls, nullptr, rows, st, first_cls);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;

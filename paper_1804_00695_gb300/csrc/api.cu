@@ -71,8 +71,9 @@ struct spgemm_handle_s {
     long long sym_counts[NBINS] = {0};
     long long num_counts[NBINS] = {0};
     int64_t max_row_nnz = 0;
+    ClsInfo cls;              // numeric rows by class (symbolic)
     size_t num_gws = 0;   // bytes of the second-level maps numeric needs
-    int num_lists = 0;        // first bin of the numeric row lists built (0 = none)
+    int num_lists = 0;        // first class of the numeric row lists built (0 = none)
     bool b_sorted = false;    // every row of B strictly ascending (symbolic)
     int64_t max_alen = 0;     // longest row of A
     int small_cap = 32, slot_factor = 2;
@@ -300,19 +301,20 @@ static int lanes_for(double x, int lo = 8) {
     return g;
 }
 
-// Workspace offsets.  [bins | rows | B descriptors | B block ranges | spans
-// of the listed rows | first window block of every row | window words of
-// the narrow rows (count, list)] persist from symbolic to numeric; after
+// Workspace offsets.  [bins | classes | rows | B descriptors | B block ranges |
+// column-block span of every row | first window block of every row | window
+// words of the narrow rows (count, list)] persist from symbolic to numeric; after
 // them the symbolic scratch, or (later) the numeric scratch, which may
 // overlap it.
 struct WsLayout {
-    size_t bins, rows, desc, mm, spans, nlo, nwords, ulist, persist;   // persistent
+    size_t bins, cls, rows, desc, mm, spans, nlo, nwords, ulist, persist;   // persistent
     size_t ana, flops, pairs, ccnt, tmp, gws;                          // symbolic scratch
 };
 static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     WsLayout L;
     L.bins = 0;
-    L.rows = L.bins + align_up((size_t)n);
+    L.cls = L.bins + align_up((size_t)n);
+    L.rows = L.cls + align_up((size_t)n);
     L.desc = L.rows + align_up((size_t)n * 4);
     L.mm = L.desc + align_up((size_t)nb * 16);
     L.spans = L.mm + align_up((size_t)nb * 8);
@@ -362,6 +364,8 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         int2 *minmax = (int2 *)(w + L.mm);
         int4 *desc = (int4 *)(w + L.desc);
         int2 *ana = (int2 *)(w + L.ana);
+        uint8_t *cls = (uint8_t *)(w + L.cls);
+        int2 *rspan = (int2 *)(w + L.spans);
         int32_t *nlo = (int32_t *)(w + L.nlo);
         uint8_t *nwords = (uint8_t *)(w + L.nwords);
         uint2 *ulist = (uint2 *)(w + L.ulist);
@@ -378,10 +382,10 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
             // pass below takes the other rows
             // lanes per row: rows of A longer than 32 entries take 8
             const int gn = h->g_narrow_sym ? h->g_narrow_sym : (mean_alen <= 32.0 ? 4 : 8);
-            SG_TRY(launch_sym_narrow(*A, *B, desc, minmax, pairs, flops, bins, C_row_ptr, nlo, nwords, ulist,
-                                     h->dstate, gn, c));
+            SG_TRY(launch_sym_narrow(*A, *B, desc, minmax, pairs, flops, bins, C_row_ptr, rspan, nlo, nwords,
+                                     ulist, h->dstate, gn, c));
         } else {
-            SG_TRY(launch_analyze(*A, *B, ana, flops, bins, C_row_ptr, h->dstate, c));
+            SG_TRY(launch_analyze(*A, *B, ana, minmax, flops, bins, C_row_ptr, rspan, h->dstate, c));
         }
         SG_TRY(launch_symbolic_first(*A, bins, desc, pairs, C_row_ptr, h->dstate, gs, c));
         SG_TRY(fetch_state(h, s));
@@ -395,26 +399,26 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         for (int b = 2; b < NBINS; b++) h->sym_counts[b] = h->hstate->bin_count[0][b];
         h->sym_counts[BIN_NARROW] = h->hstate->sym_hist[BIN_NARROW];
         if (second > 0) {
-            SG_TRY(launch_scatter_bins(n, bins, C_row_ptr, rows, h->dstate, 0, c));
-            // spans of the rows of bins 2..5 (the lists come in bin order)
-            int2 *spans = (int2 *)(w + L.spans);
-            long long spanned = 0;
-            for (int b = 2; b < BIN_HUGE; b++) spanned += h->hstate->bin_count[0][b];
-            SG_TRY(launch_list_spans(*A, minmax, rows, spanned, spans, c));
+            SG_TRY(launch_scatter_bins(n, bins, C_row_ptr, rows, h->dstate, c));
             SG_TRY(launch_symbolic(*A, *B, pairs, ccnt, rows, h->hstate->bin_count[0], C_row_ptr,
-                                   &h->dstate->err, w + L.gws, gws_bytes, spans, c));
+                                   &h->dstate->err, w + L.gws, gws_bytes, rspan, c));
         }
         SG_TRY(launch_scan_counts(C_row_ptr, n, &h->dstate->nnz, w + L.tmp, c));
-        SG_TRY(launch_numeric_binning(n, C_row_ptr, flops, bins, h->dstate, c, h->narrow ? nlo : nullptr));
+        SG_TRY(launch_numeric_binning(n, C_row_ptr, flops, bins, cls, rspan, h->dstate, c, h->narrow ? nlo : nullptr));
         SG_TRY(fetch_state(h, s));
         SG_TRY(device_errors(h->hstate->err));
         *nnz_C = h->hstate->nnz;
         h->mean_flops = (double)h->hstate->flops_total / (double)n;
         memcpy(h->num_counts, h->hstate->bin_count[1], sizeof(h->num_counts));
+        for (int k = 0; k < NCLS; k++) {
+            h->cls.count[k] = h->hstate->cls_count[k];
+            h->cls.nnz[k] = h->hstate->cls_nnz[k];
+            h->cls.words[k] = h->hstate->cls_words[k];
+        }
         h->max_row_nnz = h->hstate->max_row_nnz;
         h->b_sorted = h->hstate->b_unsorted == 0;
         h->max_alen = h->hstate->max_alen;
-        h->num_gws = h->num_counts[BIN_HUGE]
+        h->num_gws = h->cls.count[CLS_HUGE]
                          ? std::max(numeric_global_ws(h->max_row_nnz, B->ncols, h->nsm, SPGEMM_F64),
                                     window_global_ws(h->max_alen, h->nsm))
                          : 0;
@@ -454,8 +458,8 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
     uint8_t *bins = (uint8_t *)(h->ws + L.bins);
     int32_t *rows = (int32_t *)(h->ws + L.rows);
     const int4 *bdesc = (const int4 *)(h->ws + L.desc);
-    const int2 *bmm = (const int2 *)(h->ws + L.mm);
-    int2 *spans = (int2 *)(h->ws + L.spans);
+    const uint8_t *cls = (const uint8_t *)(h->ws + L.cls);
+    const int2 *rspan = (const int2 *)(h->ws + L.spans);
     const int32_t *nlo = (const int32_t *)(h->ws + L.nlo);
     const uint8_t *nwords = (const uint8_t *)(h->ws + L.nwords);
     const uint2 *ulist = (const uint2 *)(h->ws + L.ulist);
@@ -471,15 +475,11 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
     tune.G = h->g_numeric ? h->g_numeric : lanes_for(h->mean_flops / 80.0);
     tune.small_cap = h->small_cap;
     tune.slot_factor = h->slot_factor;
-    const int first_list = tune.small_cap >= 32 ? 3 : 2;
+    const int first_list = tune.small_cap >= 32 ? CLS_RANK_S : CLS_B2;
     long long listed = 0;
-    for (int b = first_list; b <= BIN_HUGE; b++) listed += h->num_counts[b];
+    for (int k = first_list; k < NCLS; k++) listed += h->cls.count[k];
     if (listed > 0 && h->num_lists != first_list) {
-        SG_TRY(launch_scatter_bins(n, bins, C->row_ptr, rows, h->dstate, 1, c, first_list));
-        // spans of the listed rows up to bin 4 (the kernels that choose by span)
-        long long spanned = 0;
-        for (int b = first_list; b <= 4; b++) spanned += h->num_counts[b];
-        SG_TRY(launch_list_spans(*A, bmm, rows, spanned, spans, c));
+        SG_TRY(launch_scatter_cls(n, cls, rows, h->dstate, first_list, c));
         h->num_lists = first_list;
     }
     if (h->num_counts[BIN_NARROW] > 0) {
@@ -489,8 +489,8 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
         const int gn = h->g_narrow_num ? h->g_narrow_num : (mean_blen <= 8.0 ? 4 : 8);
         SG_TRY(launch_num_narrow(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, bins, &h->dstate->err, gn, c));
     }
-    return launch_numeric(dtype, h->f64_native, *A, *B, *C, bins, bdesc, spans, rows, h->num_counts,
-                          h->dstate, bsplit, gws, h->num_gws, h->max_row_nnz, tune, h->b_sorted,
+    return launch_numeric(dtype, h->f64_native, *A, *B, *C, bins, bdesc, rspan, rows, h->num_counts,
+                          h->cls, h->dstate, bsplit, gws, h->num_gws, h->max_row_nnz, tune, h->b_sorted,
                           h->max_alen, c);
 }
 

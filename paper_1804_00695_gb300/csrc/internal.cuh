@@ -47,6 +47,11 @@ struct DevState {          // lives in device memory, one per handle
     int long_rows;           // the compression met rows for its warp-per-row pass
     long long max_alen;      // longest row of A (analysis)
     unsigned long long triangles;   // spgemm_triangles: the count
+    // numeric rows by class (NumCls): rows, list cursors, largest row of C,
+    // largest column span in 32-column blocks
+    long long cls_count[16];
+    long long cls_cursor[16];
+    int cls_nnz[16], cls_words[16];
 };
 
 // ---------------------------------------------------------------- bins
@@ -88,6 +93,39 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
     int b = 1;
     while (b < BIN_HUGE && (keys > sym_cap(b) || cpairs > 64 * sym_cap(b))) b++;
     return b;
+}
+
+// Class of a row of numeric bins 2..6: the kernel that takes it, given by
+// its outputs, its column span and its products.  The lists of the numeric
+// phase are in class order.
+//   CLS_B2      bin 2 (a list only when the small-row kernel stops at 16)
+//   CLS_RANK_S  at most RANK_S_NNZ outputs over at most RANK_S_WORDS blocks
+//   CLS_RANK_M4, CLS_RANK_M5  wider spans up to RANK_M_WORDS blocks: rows
+//               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
+//   CLS_WIDE3 .. CLS_WIDE4C   other rows of bins 3 and 4 by outputs
+//   CLS_BLOCK, CLS_HUGE       other rows of bins 5 and 6
+// Why the lines lie there: 2048 blocks are the bitmap that 128 threads scan in
+// one step of 16 words, 8192 the one that 512 threads do; a row of 8192 FP64
+// outputs over 8192 blocks takes 167 KB of shared memory, the next power of
+// two would not fit.  Below them the rank accumulators measured 2.6-5x
+// faster than the maps and windows (rank.cu has the figures).
+enum NumCls {
+    CLS_NONE = 0, CLS_B2, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
+    CLS_BLOCK, CLS_HUGE, NCLS
+};
+constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
+constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit 32 bits)
+__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words) {
+    if (bin < 2 || bin > BIN_HUGE) return CLS_NONE;
+    if (bin == 2) return CLS_B2;
+    if (words > 0 && flops <= RANK_FLOPS) {
+        if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_S_WORDS) return CLS_RANK_S;
+        if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_M_WORDS) return CLS_RANK_M4;
+        if (nnz <= RANK_M_NNZ && words <= RANK_M_WORDS) return CLS_RANK_M5;
+    }
+    if (bin == 3) return CLS_WIDE3;
+    if (bin == 4) return nnz <= 256 ? CLS_WIDE4A : nnz <= 512 ? CLS_WIDE4B : CLS_WIDE4C;
+    return bin == 5 ? CLS_BLOCK : CLS_HUGE;
 }
 
 // Narrow rows (narrow.cu): rows of C whose columns all fall within
@@ -202,25 +240,24 @@ size_t scan_tmp_bytes(int64_t n);
 // x[0..n] holds counts in x[1..n]; on return x is the exclusive prefix
 // (x[0] = 0); *total (device) = x[n].
 int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &c);
-// Per row i of A: flops, symbolic bin; empty rows get crp[i+1] = 0.
-int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, int64_t *flops,
-                   uint8_t *bins, int64_t *crp, DevState *st, Ctx &c);
+// Per row i of A: flops, symbolic bin, column-block span rspan[i] = {first
+// block, blocks} of the rows of B it reaches ({INT_MAX, 0} if none; bmm[k] =
+// {first block, last block} of B_k); empty rows get crp[i+1] = 0.
+int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, const int2 *bmm, int64_t *flops,
+                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, Ctx &c);
 // Numeric bin of every row from its output count crp[i+1]-crp[i] and flops;
 // rows the symbolic phase found narrow (nlo[i] >= 0; nlo may be null) that
 // fit the narrow numeric kernel get BIN_NARROW.
-int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins,
-                           DevState *st, Ctx &c, const int32_t *nlo = nullptr);
-// Row lists per bin: rows[offset(b) + t]; offsets from st->bin_count[phase]
-// (phase 0: symbolic second pass, phase 1: numeric bins 3..6).
-int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows,
-                        DevState *st, int phase, Ctx &c, int first_bin = 3);
+// cls[i]: the row's class (num_cls); rows, largest row and span per class in st.
+int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
+                           const int2 *rspan, DevState *st, Ctx &c, const int32_t *nlo = nullptr);
+// Row lists of the symbolic second pass by bin: rows[offset(b) + t], offsets
+// from st->bin_count[0].
+int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows, DevState *st, Ctx &c);
+// Row lists of the numeric phase by class (classes first_cls and up), offsets
+// from st->cls_count.
+int launch_scatter_cls(int64_t n, const uint8_t *cls, int32_t *rows, DevState *st, int first_cls, Ctx &c);
 int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, int *err, Ctx &c);
-// Column-block span of each listed row of C, once for all the kernels that
-// choose by it: spans[t] = {first block, number of blocks} of the blocks the
-// rows of B reached by row rows[t] of A cover (bmm[k] = {first block, last
-// block} of B_k); {INT_MAX, 0} when they cover none.
-int launch_list_spans(const spgemm_csr &A, const int2 *bmm, const int32_t *rows, int64_t count, int2 *spans,
-                      Ctx &c);
 
 // narrow.cu
 // Analysis of every row of A (flops, symbolic bin, as launch_analyze) with
@@ -231,7 +268,7 @@ int launch_list_spans(const spgemm_csr &A, const int2 *bmm, const int32_t *rows,
 // ulist[i*NARROW_NMAX ...] (first NARROW_NMAX of them; {word | rank of its
 // first column << 8, mask}) and their number in nwords[i].
 int launch_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
-                      const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int32_t *nlo,
+                      const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
                       uint8_t *nwords, uint2 *ulist, DevState *st, int G, Ctx &c);
 // Numeric phase of the rows with bins[i] == BIN_NARROW (F32 or native F64),
 // from the word lists of the symbolic phase; G lanes per row (4, 8 or 16).
@@ -245,18 +282,18 @@ int launch_num_narrow(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgem
 int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc,
                           const int2 *pairs, int64_t *crp, DevState *st, int G, Ctx &c);
 // Second pass: kernels of bins 2..6; counts[b] = rows in bin b (host),
-// rows = concatenated bin lists, spans[t] = span of rows[t] (bins 2..5).
+// rows = concatenated bin lists, rspan[i] = column-block span of row i.
 // Writes nnz(C_i) to crp[i+1].
 int launch_symbolic(const spgemm_csr &A, const spgemm_csr &B, const int2 *pairs,
                     const int32_t *ccnt, const int32_t *rows, const long long *counts,
-                    int64_t *crp, int *err, void *gws, size_t gws_bytes, const int2 *spans, Ctx &c);
+                    int64_t *crp, int *err, void *gws, size_t gws_bytes, const int2 *rspan, Ctx &c);
 size_t symbolic_global_ws(int64_t ncols_b, int nsm);
 
 // numeric.cu
-// Runs the numeric kernels: bins 1-2 over all rows in order (bins[i]), bins
-// 3..6 from the row lists (counts[b] rows in bin b, host; spans[t] = span of
-// rows[t] for the lists of bins up to 4).  FP64 uses double-word
-// accumulation unless f64_native; bsplit: room for nnz(B) float2.
+// Runs the numeric kernels: bins 1-2 over all rows in order (bins[i]), the
+// others from the row lists by class (cls rows, largest row and span of each
+// class, host).  FP64 uses double-word accumulation unless f64_native;
+// bsplit: room for nnz(B) float2.
 // Tunables of the numeric phase: lanes per row of the small-row kernel,
 // largest output row it takes (16 or 32; bin 2 rows go to the warp kernel
 // when 16), and map slots per output entry (2 or 4).
@@ -265,14 +302,25 @@ struct NumTune {
     int small_cap = 32;
     int slot_factor = 2;
 };
+struct ClsInfo {
+    long long count[NCLS] = {0};
+    int nnz[NCLS] = {0}, words[NCLS] = {0};
+};
 int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm_csr &B,
-                   spgemm_csr &C, const uint8_t *bins, const int4 *bdesc, const int2 *spans,
+                   spgemm_csr &C, const uint8_t *bins, const int4 *bdesc, const int2 *rspan,
                    const int32_t *rows,
-                   const long long *counts, DevState *st, float2 *bsplit, void *gws,
+                   const long long *counts, const ClsInfo &cls, DevState *st, float2 *bsplit, void *gws,
                    size_t gws_bytes, int64_t max_row_nnz, const NumTune &tune, bool b_sorted,
                    int64_t max_alen, Ctx &c);
 size_t numeric_global_ws(int64_t max_row_nnz, int64_t ncols_b, int nsm, int dtype);
 size_t window_global_ws(int64_t max_alen, int nsm);
+
+// rank.cu: listed rows with a dense rank accumulator (a block each), in FP32
+// or native FP64; rows wider than max_words blocks or with more than max_nnz
+// outputs are skipped.  small: rows of CLS_RANK_S (or CLS_B2).
+int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
+                    const int2 *rspan, const int32_t *rows, int64_t count, bool small, int64_t max_nnz,
+                    int64_t max_words, int *err, Ctx &c);
 
 // batched.cu: one instance of a batch, with its place in the stacked arrays.
 struct BatchInst {

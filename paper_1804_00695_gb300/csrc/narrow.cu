@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
     int64_t n, int64_t nrows_b, int64_t nwords_b, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc, const int2 *__restrict__ bmm,
     const int2 *__restrict__ pairs, int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
-    int64_t *__restrict__ crp, int32_t *__restrict__ nlo, uint8_t *__restrict__ nwords,
+    int64_t *__restrict__ crp, int2 *__restrict__ rspan, int32_t *__restrict__ nlo, uint8_t *__restrict__ nwords,
     uint2 *__restrict__ ulist, DevState *st) {
     constexpr int WPB = NARROW_SYM_WPB;
     constexpr int RPW = 32 / G, NR = WPB * RPW, QPL = NARROW_W / 4 / G;
@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
         const bool lead = live && gl == 0;
         if (lead) {
             flops[i] = f;
+            rspan[i] = make_int2(lo, hi >= lo ? hi - lo + 1 : 0);
             wf += f;
             wl = max(wl, (long long)plen);
             if (nar) {
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
 
 template <int G>
 static int run_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
-                          const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int32_t *nlo,
+                          const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
                           uint8_t *nwords, uint2 *ulist, DevState *st, Ctx &c) {
     constexpr int NT = NARROW_SYM_WPB * 32, NR = NARROW_SYM_WPB * (32 / G);
     int64_t blocks = (A.nrows + NR - 1) / NR;
@@ -301,21 +302,21 @@ static int run_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *
     const int64_t nwb = (B.ncols + 31) / 32;
     c.begin("symbolic.narrow", A.nrows);
     k_sym_narrow<G><<<(unsigned)blocks, NT, 0, c.s>>>(A.nrows, B.nrows, nwb, A.row_ptr, A.col_idx, desc, bmm,
-                                                      pairs, flops, bins, crp, nlo, nwords, ulist, st);
+                                                      pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
 int launch_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
-                      const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int32_t *nlo,
+                      const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
                       uint8_t *nwords, uint2 *ulist, DevState *st, int G, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     switch (G) {
-        case 4: return run_sym_narrow<4>(A, B, desc, bmm, pairs, flops, bins, crp, nlo, nwords, ulist, st, c);
-        case 8: return run_sym_narrow<8>(A, B, desc, bmm, pairs, flops, bins, crp, nlo, nwords, ulist, st, c);
-        case 16: return run_sym_narrow<16>(A, B, desc, bmm, pairs, flops, bins, crp, nlo, nwords, ulist, st, c);
-        default: return run_sym_narrow<32>(A, B, desc, bmm, pairs, flops, bins, crp, nlo, nwords, ulist, st, c);
+        case 4: return run_sym_narrow<4>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
+        case 8: return run_sym_narrow<8>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
+        case 16: return run_sym_narrow<16>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
+        default: return run_sym_narrow<32>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
     }
 }
 

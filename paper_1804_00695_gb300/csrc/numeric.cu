@@ -5,10 +5,11 @@
 // * bins 1-2 (<= 32 outputs): groups of G lanes per row, a shared-memory
 //   hash map from column to value per row (the sparse hash accumulators of
 //   Section 2.1), products dealt evenly over the lanes;
-// * bins 3-4 (<= 1024 outputs): a warp per row with a dense rank
-//   accumulator over the row's column span (bitmap, prefix counts, values
-//   by rank) when the span is at most 2048 blocks of 32 columns (three
-//   bitmap sizes), else a warp-level shared hash map;
+// * larger rows whose columns span a bitmap that fits shared memory: a block
+//   per row with a dense rank accumulator (rank.cu; for double-words, up to
+//   2048 blocks of 32 columns, a warp per row here, three bitmap sizes);
+// * bins 3-4 (<= 1024 outputs) over wider spans: a warp per row, shared hash
+//   map;
 // * bin 5 (<= 4096 outputs): a block per row, shared hash map;
 // * bin 6 (more): a windowed dense accumulator when the rows of B are
 //   sorted, else a two-level hash map (shared, then global memory: Section
@@ -608,22 +609,21 @@ __device__ __forceinline__ int rank_tier(int span, int nn) {
 // Section 3.1, restricted to the span and held in shared memory).  Pass 1
 // marks every reachable column in a bitmap over the span; prefix counts of
 // the bitmap words turn a column into its rank in the output row; pass 2
-// adds every product into vals[rank] (atomically: FP32 and native FP64 in
-// their type, double-words through the three-level dw_atomic_acc).  The row
+// adds every product into vals[rank] (atomically, through the three-level
+// dw_atomic_acc; rows outside the double-word range in native FP64).  The row
 // is then written in column order straight from the bitmap: no hash map,
 // no sort.  Products are dealt out over the warp's 32 lanes as in the other
-// kernels.  Per warp: bitmap, 16-bit prefix counts, NMAX values.
-template <int MODE>
-struct RankVal {
-    static constexpr int bytes = MODE == MODE_F32 ? 4 : (MODE == MODE_DW ? 12 : 8);
-};
+// kernels.  Per warp: bitmap, 16-bit prefix counts, NMAX values.  Double-word
+// accumulation only: FP32 and native FP64 rows go to the block-per-row
+// kernel of rank.cu.
+constexpr int RANK_VAL_BYTES = 12;   // a double-word and its third level
 
 constexpr int RANK_U = 4;   // products per lane per step in the rank kernels
 
-template <int BW, int NMAX, int WPB, int MODE>
+template <int BW, int NMAX, int WPB>
 struct RankLayout {
     static constexpr size_t per_warp =
-        ((size_t)BW * 6 + (size_t)BW / 8 + (size_t)NMAX * RankVal<MODE>::bytes + 32 * 16 + 33 * 4 + 64 + 15) &
+        ((size_t)BW * 6 + (size_t)BW / 8 + (size_t)NMAX * RANK_VAL_BYTES + 32 * 16 + 33 * 4 + 64 + 15) &
         ~(size_t)15;
     static constexpr size_t bytes = per_warp * WPB;
 };
@@ -632,13 +632,12 @@ struct RankLayout {
 // per word), so the prefix counts, the output and the clean-up visit only
 // those words: the work per row follows its outputs, not its span.  A row
 // leaves its bitmap words and summary zero for the next.
-template <int BW, int NMAX, int WPB, int MODE>
+template <int BW, int NMAX, int WPB>
 __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__restrict__ bdesc,
-                                                       const int2 *__restrict__ spans,
+                                                       const int2 *__restrict__ rspan,
                                                        const int32_t *__restrict__ rows, int64_t count,
                                                        int tier, const DevState *st, int *err) {
-    using Lay = RankLayout<BW, NMAX, WPB, MODE>;
-    using V = ValT<MODE>;
+    using Lay = RankLayout<BW, NMAX, WPB>;
     constexpr int E = 32, NS = BW / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -649,12 +648,11 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__
     unsigned *summ = bits + BW;
     unsigned short *pref = (unsigned short *)(summ + NS);
     unsigned char *vbase = (unsigned char *)(((uintptr_t)(pref + BW) + 15) & ~(uintptr_t)15);
-    float *vf = (float *)vbase;                              // FP32
     double *v8 = (double *)vbase;                            // native FP64
     float2 *v2 = (float2 *)vbase;                            // double-word hi, lo
     float *v3 = (float *)(v2 + NMAX);                        // third level
-    int *pre = (int *)(vbase + (size_t)NMAX * RankVal<MODE>::bytes);
-    const bool b_bad = MODE == MODE_DW && st->b_out_of_range;
+    int *pre = (int *)(vbase + (size_t)NMAX * RANK_VAL_BYTES);
+    const bool b_bad = st->b_out_of_range;
     int flag = 0;
     for (int x = lane; x < BW; x += 32) bits[x] = 0;
     for (int x = lane; x < NS; x += 32) summ[x] = 0;
@@ -664,21 +662,20 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__
         const int64_t out = a.crp[i];
         const int nn = (int)(a.crp[i + 1] - out);
         if (nn > NMAX) continue;
-        const int2 sp = spans[t];
+        const int2 sp = rspan[i];
         const int bmin = sp.x, nw = sp.y;
         if (nw > BW || nw == 0 || rank_tier(nw, nn) != tier) continue;
         const int64_t p0 = a.arp[i];
         const int plen = (int)(a.arp[i + 1] - p0);
-        bool nat = MODE == MODE_F64 || b_bad;
-        if (MODE == MODE_DW && !nat) {
+        bool nat = b_bad;
+        if (!nat) {
             bool ok = true;
             for (int pp = lane; pp < plen; pp += 32) dw_split(((const double *)a.aval)[p0 + pp], ok);
             nat = !__all_sync(0xffffffffu, ok);
         }
         for (int x = lane; x < nn; x += 32) {
-            if (MODE == MODE_F32) vf[x] = 0.f;
-            else if (MODE == MODE_DW) { v2[x] = make_float2(0.f, 0.f); v3[x] = 0.f; }
-            else v8[x] = 0.0;
+            v2[x] = make_float2(0.f, 0.f);
+            v3[x] = 0.f;
         }
         const int ns = (nw + 31) / 32;                 // summary words of the span
         const int sper = (ns + 31) / 32;               // per lane, contiguous
@@ -698,14 +695,14 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__
                         const int4 d = bdesc[a.acol[p0 + pb + lane]];
                         len = d.z;
                         eq0[lane] = desc_start(d);
-                        const V av = ((const V *)a.aval)[p0 + pb + lane];
-                        if (MODE == MODE_DW && !nat) {
+                        const double av = ((const double *)a.aval)[p0 + pb + lane];
+                        if (!nat) {
                             bool dummy = true;
-                            const float2 s2 = dw_split((double)av, dummy);
+                            const float2 s2 = dw_split(av, dummy);
                             ea[lane] = __longlong_as_double(((long long)__float_as_uint(s2.y) << 32) |
                                                             (long long)__float_as_uint(s2.x));
                         } else {
-                            ea[lane] = (double)av;
+                            ea[lane] = av;
                         }
                     }
                     int incl = len;
@@ -751,19 +748,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__
                             if (atomicOr(&bits[wd], 1u << (col & 31)) == 0)
                                 atomicOr(&summ[wd >> 5], 1u << (wd & 31));
                         }
-                    } else if (MODE == MODE_F32) {
-                        float bv[RANK_U];
-#pragma unroll
-                        for (int u = 0; u < RANK_U; u++) bv[u] = ee[u] >= 0 ? ((const float *)a.bval)[qq[u]] : 0.f;
-#pragma unroll
-                        for (int u = 0; u < RANK_U; u++) {
-                            if (ee[u] < 0) continue;
-                            const int col = cc[u];
-                            const int wd = (col >> 5) - bmin;
-                            const int r = (int)pref[wd] + __popc(bits[wd] & ((1u << (col & 31)) - 1));
-                            atomicAdd(&vf[r], (float)ea[ee[u]] * bv[u]);
-                        }
-                    } else if (MODE == MODE_DW && !nat) {
+                    } else if (!nat) {
                         float2 bv[RANK_U];
 #pragma unroll
                         for (int u = 0; u < RANK_U; u++) bv[u] = ee[u] >= 0 ? a.bsplit[qq[u]] : make_float2(0.f, 0.f);
@@ -837,8 +822,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_rank(NumP a, const int4 *__
                     word &= word - 1;
                     if (r < nn) {
                         a.ccol[out + r] = (bmin + x) * 32 + b;
-                        if (MODE == MODE_F32) ((float *)a.cval)[out + r] = vf[r];
-                        else if (MODE == MODE_DW && !nat) ((double *)a.cval)[out + r] = dw3_to_double(v2[r].x, v2[r].y, v3[r]);
+                        if (!nat) ((double *)a.cval)[out + r] = dw3_to_double(v2[r].x, v2[r].y, v3[r]);
                         else ((double *)a.cval)[out + r] = v8[r];
                     }
                     r++;
@@ -880,7 +864,7 @@ struct WideLayout {
 
 template <int SMAX, int BW, int WPB, int MODE>
 __global__ void __launch_bounds__(WPB * 32, 1) k_num_wide(NumP a, const int4 *__restrict__ bdesc,
-                                                       const int2 *__restrict__ spans,
+                                                       const int2 *__restrict__ rspan,
                                                        const int32_t *__restrict__ rows, int64_t count,
                                                        int min_nnz, int min_span_words, const DevState *st,
                                                        int *err) {
@@ -910,7 +894,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) k_num_wide(NumP a, const int4 *__
         const int64_t out = a.crp[i];
         const int nn = (int)(a.crp[i + 1] - out);
         if (nn < min_nnz || nn > SMAX / 2) continue;
-        if (min_span_words > 0 && rank_tier(spans[t].y, nn) != 0) continue;
+        if (min_span_words > 0 && rank_tier(rspan[i].y, nn) != 0) continue;
         int S = next_pow2(2 * nn);
         S = S < 32 ? 32 : (S > SMAX ? SMAX : S);
         const int L = __ffs(S) - 1;
@@ -1549,15 +1533,15 @@ static int run_small_g(const NumTune &t, const NumP &a, const int4 *bdesc, int64
     }
 }
 
-template <int BW, int NMAX, int WPB, int MODE>
-static int run_rank(const NumP &a, const int4 *bdesc, const int2 *spans, const int32_t *rows, int64_t count,
+template <int BW, int NMAX, int WPB>
+static int run_rank(const NumP &a, const int4 *bdesc, const int2 *rspan, const int32_t *rows, int64_t count,
                     int tier, DevState *st, int *err, const char *label, Ctx &c) {
-    const size_t smem = RankLayout<BW, NMAX, WPB, MODE>::bytes;
-    SG_TRY(prep(k_num_rank<BW, NMAX, WPB, MODE>, smem));
+    const size_t smem = RankLayout<BW, NMAX, WPB>::bytes;
+    SG_TRY(prep(k_num_rank<BW, NMAX, WPB>, smem));
     int64_t blocks = (count + WPB - 1) / WPB;
     blocks = blocks < (int64_t)c.nsm * 32 ? blocks : (int64_t)c.nsm * 32;
     c.begin(label, count);
-    k_num_rank<BW, NMAX, WPB, MODE><<<(unsigned)blocks, WPB * 32, smem, c.s>>>(a, bdesc, spans, rows, count,
+    k_num_rank<BW, NMAX, WPB><<<(unsigned)blocks, WPB * 32, smem, c.s>>>(a, bdesc, rspan, rows, count,
                                                                                 tier, st, err);
     c.end();
     SG_CUDA(cudaGetLastError());
@@ -1565,14 +1549,14 @@ static int run_rank(const NumP &a, const int4 *bdesc, const int2 *spans, const i
 }
 
 template <int SMAX, int BW, int WPB, int MODE>
-static int run_wide(const NumP &a, const int4 *bdesc, const int2 *spans, const int32_t *rows, int64_t count,
+static int run_wide(const NumP &a, const int4 *bdesc, const int2 *rspan, const int32_t *rows, int64_t count,
                     int min_nnz, int min_span, DevState *st, int *err, const char *label, Ctx &c) {
     const size_t smem = WideLayout<SMAX, BW, WPB, MODE>::bytes;
     SG_TRY(prep(k_num_wide<SMAX, BW, WPB, MODE>, smem));
     int64_t blocks = (count + WPB - 1) / WPB;
     blocks = blocks < (int64_t)c.nsm * 32 ? blocks : (int64_t)c.nsm * 32;
     c.begin(label, count);
-    k_num_wide<SMAX, BW, WPB, MODE><<<(unsigned)blocks, WPB * 32, smem, c.s>>>(a, bdesc, spans, rows, count, min_nnz,
+    k_num_wide<SMAX, BW, WPB, MODE><<<(unsigned)blocks, WPB * 32, smem, c.s>>>(a, bdesc, rspan, rows, count, min_nnz,
                                                                                 min_span, st, err);
     c.end();
     SG_CUDA(cudaGetLastError());
@@ -1649,46 +1633,80 @@ static int run_window(const NumP &a, const int32_t *rows, int64_t cnt, int *err,
     return SPGEMM_OK;
 }
 
-template <int MODE>
-static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, const uint8_t *bins,
-                   const int4 *bdesc, const int2 *spans, const int32_t *rows, const long long *counts, DevState *st,
-                   void *gws, size_t gws_bytes, int64_t max_row_nnz, const NumTune &t, bool b_sorted,
-                   int64_t max_alen, Ctx &c) {
-    using V = typename std::conditional<MODE == MODE_F32, float, double>::type;
+// Double-word rows spanning at most RANK_S_WORDS blocks: dense rank
+// accumulators of a warp each (three span limits).
+static int run_warp_rank(const NumP &a, const int4 *bdesc, const int2 *rspan, const int32_t *r, int64_t cnt,
+                         DevState *st, Ctx &c) {
     int *err = &st->err;
-    const int first_list = t.small_cap >= 32 ? 3 : 2;
-    if (counts[1] + (first_list == 3 ? counts[2] : 0) > 0)
+    SG_TRY((run_rank<RANK_BW1, RANK_NMAX1, 8>(a, bdesc, rspan, r, cnt, 1, st, err, "numeric.rank512", c)));
+    SG_TRY((run_rank<RANK_BW2, RANK_NMAX2, 8>(a, bdesc, rspan, r, cnt, 2, st, err, "numeric.rank1024", c)));
+    return run_rank<RANK_BW3, RANK_NMAX3, 4>(a, bdesc, rspan, r, cnt, 3, st, err, "numeric.rank2048", c);
+}
+
+template <int MODE>
+static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const uint8_t *bins,
+                   const int4 *bdesc, const int2 *rspan, const int32_t *rows, const long long *counts,
+                   const ClsInfo &cls, DevState *st, void *gws, size_t gws_bytes, int64_t max_row_nnz,
+                   const NumTune &t, bool b_sorted, int64_t max_alen, Ctx &c) {
+    using V = typename std::conditional<MODE == MODE_F32, float, double>::type;
+    constexpr int DT = MODE == MODE_F32 ? SPGEMM_F32 : SPGEMM_F64;
+    int *err = &st->err;
+    const int first = t.small_cap >= 32 ? CLS_RANK_S : CLS_B2;
+    if (counts[1] + (first == CLS_RANK_S ? counts[2] : 0) > 0)
         SG_TRY(run_small_g<MODE>(t, a, bdesc, A.nrows, bins, st, err, c));
     int64_t off = 0;
-    for (int b = first_list; b <= BIN_HUGE; b++) {
-        const int64_t cnt = counts[b];
+    for (int k = first; k < NCLS; k++) {
+        int64_t cnt = cls.count[k];
         const int32_t *r = rows + off;
-        const int2 *sp = spans + off;
         off += cnt;
         if (cnt == 0) continue;
-        switch (b) {
-            case 2:
-            case 3:
-            case 4:
-                // dense rank accumulators for the rows rank_takes accepts (two span
-                // limits), hash maps for the others (two map sizes)
-                SG_TRY((run_rank<RANK_BW1, RANK_NMAX1, 8, MODE>(a, bdesc, sp, r, cnt, 1, st, err,
-                                                                 "numeric.rank512", c)));
-                SG_TRY((run_rank<RANK_BW2, RANK_NMAX2, 8, MODE>(a, bdesc, sp, r, cnt, 2, st, err,
-                                                                 "numeric.rank1024", c)));
-                SG_TRY((run_rank<RANK_BW3, RANK_NMAX3, 4, MODE>(a, bdesc, sp, r, cnt, 3, st, err,
-                                                                 "numeric.rank2048", c)));
-                // the rows left to the maps span more than RANK_BW3 words, so the
-                // maps' own bitmap output (spans up to 32 * BW columns) is kept small
-                if (b <= 3) {
-                    SG_TRY((run_wide<256, 64, 8, MODE>(a, bdesc, sp, r, cnt, 0, 1, st, err, "numeric.wide3", c)));
-                } else {
-                    SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, sp, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
-                    SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, sp, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
-                    SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, sp, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
-                }
+        // rows left to the maps span more than RANK_S_WORDS blocks, so the
+        // maps' own bitmap output (spans up to 32 * BW columns) is kept small
+        switch (k) {
+            case CLS_B2:
+            case CLS_RANK_S:
+                if (MODE == MODE_DW)
+                    SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
+                else
+                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, true, cls.nnz[k],
+                                           std::min(cls.words[k], RANK_S_WORDS), err, c));
+                if (k == CLS_B2 && cls.words[k] > RANK_S_WORDS)
+                    SG_TRY((run_wide<256, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide3", c)));
                 break;
-            case 5: SG_TRY((run_block<256, 8192, V>(a, r, cnt, err, b, c))); break;
+            case CLS_RANK_M4:
+                if (MODE == MODE_DW) {
+                    SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
+                    SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
+                    SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
+                    break;
+                }
+                if (cls.count[CLS_RANK_M5]) break;   // one launch with the next list
+                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, false, cls.nnz[k], cls.words[k], err, c));
+                break;
+            case CLS_RANK_M5: {
+                int nmax = cls.nnz[k], words = cls.words[k];
+                if (MODE != MODE_DW) {
+                    r -= cls.count[CLS_RANK_M4];
+                    cnt += cls.count[CLS_RANK_M4];
+                    nmax = std::max(nmax, cls.nnz[CLS_RANK_M4]);
+                    words = std::max(words, cls.words[CLS_RANK_M4]);
+                }
+                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, false, nmax, words, err, c));
+                break;
+            }
+            case CLS_WIDE3:
+                SG_TRY((run_wide<256, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide3", c)));
+                break;
+            case CLS_WIDE4A:
+                SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
+                break;
+            case CLS_WIDE4B:
+                SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
+                break;
+            case CLS_WIDE4C:
+                SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
+                break;
+            case CLS_BLOCK: SG_TRY((run_block<256, 8192, V>(a, r, cnt, err, BIN_HUGE - 1, c))); break;
             default:
                 if (b_sorted) SG_TRY(run_window<V>(a, r, cnt, err, gws, gws_bytes, max_alen, c));
                 else SG_TRY(run_huge<V>(a, B, r, cnt, err, gws, gws_bytes, max_row_nnz, c));
@@ -1698,16 +1716,16 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, cons
 }
 
 int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C,
-                   const uint8_t *bins, const int4 *bdesc, const int2 *spans, const int32_t *rows,
-                   const long long *counts, DevState *st, float2 *bsplit, void *gws,
+                   const uint8_t *bins, const int4 *bdesc, const int2 *rspan, const int32_t *rows,
+                   const long long *counts, const ClsInfo &cls, DevState *st, float2 *bsplit, void *gws,
                    size_t gws_bytes, int64_t max_row_nnz, const NumTune &G, bool b_sorted,
                    int64_t max_alen, Ctx &c) {
     NumP a{A.row_ptr, A.col_idx, A.values, B.row_ptr, B.col_idx, B.values, bsplit,
            C.row_ptr, C.col_idx, C.values};
     if (dtype == SPGEMM_F32)
-        return run_all<MODE_F32>(a, A, B, bins, bdesc, spans, rows, counts, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+        return run_all<MODE_F32>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
     if (f64_native)
-        return run_all<MODE_F64>(a, A, B, bins, bdesc, spans, rows, counts, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+        return run_all<MODE_F64>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
     SG_CUDA(cudaMemsetAsync(&st->b_out_of_range, 0, sizeof(int), c.s));
     if (B.nnz > 0) {
         int64_t blocks = (B.nnz + 255) / 256;
@@ -1717,7 +1735,7 @@ int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm
         c.end();
         SG_CUDA(cudaGetLastError());
     }
-    return run_all<MODE_DW>(a, A, B, bins, bdesc, spans, rows, counts, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+    return run_all<MODE_DW>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
 }
 
 }  // namespace sg
