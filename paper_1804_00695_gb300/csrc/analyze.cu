@@ -351,7 +351,7 @@ int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, i
 __global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
                                   const int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
                                   uint8_t *__restrict__ cls, const int2 *__restrict__ rspan, DevState *st,
-                                  const int32_t *__restrict__ nlo) {
+                                  bool dense_ok, const int32_t *__restrict__ nlo) {
     __shared__ unsigned long long hist[NBINS];
     __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS];
     if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
@@ -369,7 +369,7 @@ __global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
         int k = CLS_NONE;
         if (b >= 2 && b <= BIN_HUGE) {
             const int words = rspan[i].y;
-            k = num_cls(b, c, f, words);
+            k = num_cls(b, c, f, words, dense_ok && st->b_unsorted == 0);
             atomicAdd(&ccnt[k], 1);
             if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
             if (words > cwords[k]) atomicMax(&cwords[k], words);
@@ -390,10 +390,10 @@ __global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
 }
 
 int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                           const int2 *rspan, DevState *st, Ctx &c, const int32_t *nlo) {
+                           const int2 *rspan, DevState *st, bool dense_ok, Ctx &c, const int32_t *nlo) {
     if (n == 0) return SPGEMM_OK;
     c.begin("numeric_binning", n);
-    k_numeric_binning<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, crp, flops, bins, cls, rspan, st, nlo);
+    k_numeric_binning<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, crp, flops, bins, cls, rspan, st, dense_ok, nlo);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;

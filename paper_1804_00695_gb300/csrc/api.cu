@@ -404,7 +404,10 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
                                    &h->dstate->err, w + L.gws, gws_bytes, rspan, c));
         }
         SG_TRY(launch_scan_counts(C_row_ptr, n, &h->dstate->nnz, w + L.tmp, c));
-        SG_TRY(launch_numeric_binning(n, C_row_ptr, flops, bins, cls, rspan, h->dstate, c, h->narrow ? nlo : nullptr));
+        // the split table of the dense rows stays within B's own size (and 64 MB)
+        const size_t dense_bytes = dense_ws(B->nrows, B->ncols);
+        const bool dense_ok = dense_bytes <= (size_t)B->nnz * 12 + ((size_t)64 << 20);
+        SG_TRY(launch_numeric_binning(n, C_row_ptr, flops, bins, cls, rspan, h->dstate, dense_ok, c, h->narrow ? nlo : nullptr));
         SG_TRY(fetch_state(h, s));
         SG_TRY(device_errors(h->hstate->err));
         *nnz_C = h->hstate->nnz;
@@ -422,6 +425,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
                          ? std::max(numeric_global_ws(h->max_row_nnz, B->ncols, h->nsm, SPGEMM_F64),
                                     window_global_ws(h->max_alen, h->nsm))
                          : 0;
+        if (h->cls.count[CLS_DENSE]) h->num_gws = std::max(h->num_gws, dense_bytes);
         h->num_lists = 0;
         // numeric scratch: B split into double-words, then the second-level maps
         SG_TRY(ws_reserve(h, L.persist + align_up((size_t)B->nnz * 8) + h->num_gws, s, L.persist));

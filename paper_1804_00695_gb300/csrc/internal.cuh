@@ -52,6 +52,7 @@ struct DevState {          // lives in device memory, one per handle
     long long cls_count[16];
     long long cls_cursor[16];
     int cls_nnz[16], cls_words[16];
+    unsigned long long next_row;   // rows a kernel has handed out (cleared before it)
 };
 
 // ---------------------------------------------------------------- bins
@@ -104,6 +105,8 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
 //   CLS_WIDE3 .. CLS_WIDE4C   other rows of bins 3 and 4 by outputs
 //   CLS_BLOCK, CLS_HUGE       other rows of bins 5 and 6
+//   CLS_DENSE   rows of B sorted: rows with more outputs than the rank
+//               accumulators hold, or many products over their span
 // Why the lines lie there: 2048 blocks are the bitmap that 128 threads scan in
 // one step of 16 words, 8192 the one that 512 threads do; a row of 8192 FP64
 // outputs over 8192 blocks takes 167 KB of shared memory, the next power of
@@ -111,13 +114,22 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 // faster than the maps and windows (rank.cu has the figures).
 enum NumCls {
     CLS_NONE = 0, CLS_B2, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
-    CLS_BLOCK, CLS_HUGE, NCLS
+    CLS_BLOCK, CLS_DENSE, CLS_HUGE, NCLS
 };
 constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
 constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit 32 bits)
-__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words) {
+// Dense windows from one product per 8 columns of the span on (their cost per
+// row is the span written out plus the products, the rank accumulators' the
+// products twice over) and above the 6144 products that a rank block keeps in
+// registers: A*A of R-MAT graphs, FP64, scale 16 with 12 edges a vertex 11.9
+// ms (one per 4 columns 12.4), scale 15 with 5 2.91 (2.94, one per 2 3.02).
+constexpr long long DENSE_FLOPS = 6144;
+__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words, bool dense_ok) {
     if (bin < 2 || bin > BIN_HUGE) return CLS_NONE;
     if (bin == 2) return CLS_B2;
+    if (dense_ok && bin >= 5 && words > 0 && flops < (1LL << 31) &&
+        (nnz > RANK_M_NNZ || (flops > DENSE_FLOPS && flops * 8 >= (long long)words * 32)))
+        return CLS_DENSE;
     if (words > 0 && flops <= RANK_FLOPS) {
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_S_WORDS) return CLS_RANK_S;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_M_WORDS) return CLS_RANK_M4;
@@ -250,7 +262,7 @@ int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, co
 // fit the narrow numeric kernel get BIN_NARROW.
 // cls[i]: the row's class (num_cls); rows, largest row and span per class in st.
 int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                           const int2 *rspan, DevState *st, Ctx &c, const int32_t *nlo = nullptr);
+                           const int2 *rspan, DevState *st, bool dense_ok, Ctx &c, const int32_t *nlo = nullptr);
 // Row lists of the symbolic second pass by bin: rows[offset(b) + t], offsets
 // from st->bin_count[0].
 int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows, DevState *st, Ctx &c);
@@ -321,6 +333,13 @@ size_t window_global_ws(int64_t max_alen, int nsm);
 int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
                     const int2 *rspan, const int32_t *rows, int64_t count, bool small, int64_t max_nnz,
                     int64_t max_words, int *err, Ctx &c);
+
+// dense.cu: listed rows over windows of a dense accumulator (rows of B
+// sorted); dense_ws: bytes of the split table (either type); next: device counter.
+size_t dense_ws(int64_t nrows_b, int64_t ncols_b);
+int launch_num_dense(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
+                     const int2 *rspan, const int32_t *rows, int64_t count, void *ws, size_t ws_bytes,
+                     unsigned long long *next, int *err, Ctx &c);
 
 // batched.cu: one instance of a batch, with its place in the stacked arrays.
 struct BatchInst {

@@ -11,8 +11,11 @@
 // * bins 3-4 (<= 1024 outputs) over wider spans: a warp per row, shared hash
 //   map;
 // * bin 5 (<= 4096 outputs): a block per row, shared hash map;
-// * bin 6 (more): a windowed dense accumulator when the rows of B are
-//   sorted, else a two-level hash map (shared, then global memory: Section
+// * rows with many products over their span, or more outputs than the rank
+//   accumulators hold, when the rows of B are sorted: windows of a dense
+//   accumulator (dense.cu);
+// * the rest of bin 6: column windows walked by cursors when the rows of B
+//   are sorted (the split table of dense.cu would outgrow B), else a two-level hash map (shared, then global memory: Section
 //   3.3's multilevel memory).
 //
 // Output rows have ascending columns.  FP64 values are accumulated as
@@ -1707,6 +1710,9 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                 SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
                 break;
             case CLS_BLOCK: SG_TRY((run_block<256, 8192, V>(a, r, cnt, err, BIN_HUGE - 1, c))); break;
+            case CLS_DENSE:
+                SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, r, cnt, gws, gws_bytes, &st->next_row, err, c));
+                break;
             default:
                 if (b_sorted) SG_TRY(run_window<V>(a, r, cnt, err, gws, gws_bytes, max_alen, c));
                 else SG_TRY(run_huge<V>(a, B, r, cnt, err, gws, gws_bytes, max_row_nnz, c));
