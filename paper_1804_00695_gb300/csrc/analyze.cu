@@ -21,14 +21,14 @@ namespace sg {
 // addresses 32 rows apart from its neighbours' in one load instruction), and
 // every lane then reads its row from there; otherwise every lane loads its
 // own row.
-constexpr int64_t COMPRESS_LONG = 128;   // rows longer than this take a warp each
+constexpr int64_t COMPRESS_LONG = 128;   // rows longer than this take a block each
 constexpr int COMPRESS_STAGE = 1024;     // staged entries per warp
 constexpr int COMPRESS_WPB = 8;
 
 __global__ void __launch_bounds__(COMPRESS_WPB * 32) k_compress(
     int64_t nrows, int64_t ncols, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
     int2 *__restrict__ pairs, int32_t *__restrict__ ccnt, int2 *__restrict__ minmax, int4 *__restrict__ desc,
-    int2 *__restrict__ ana, int *err, int *unsorted_flag, int *long_flag) {
+    int2 *__restrict__ ana, int *err, int *unsorted_flag, int *long_count, int32_t *__restrict__ long_list) {
     __shared__ int stage_all[COMPRESS_WPB * COMPRESS_STAGE];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int *stage = stage_all + w * COMPRESS_STAGE;
@@ -54,7 +54,13 @@ __global__ void __launch_bounds__(COMPRESS_WPB * 32) k_compress(
     }
     __syncwarp();
     const bool lng = end - beg > COMPRESS_LONG;   // k_compress_long
-    if (lng && long_flag) *long_flag = 1;
+    const unsigned longs = __ballot_sync(0xffffffffu, lng);
+    if (longs) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(long_count, __popc(longs));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (lng) long_list[at + __popc(longs & ((1u << lane) - 1u))] = (int32_t)r;
+    }
     if (!live || lng) return;
     const int *src = staged ? stage + (beg - wbeg) : col + beg;
     const int len = (int)(end - beg);
@@ -98,121 +104,130 @@ __global__ void __launch_bounds__(COMPRESS_WPB * 32) k_compress(
     if (unsorted && unsorted_flag) atomicOr(unsorted_flag, 1);
 }
 
-// The same for the rows longer than COMPRESS_LONG, a warp per row, 32
-// consecutive entries at a time: a pair starts where an entry's block
-// differs from the previous entry's; the masks of a run are ORed by a
-// segmented scan over the lanes; a run that reaches the end of the 32 is
-// carried into the next 32 (its pair written once it ends).
-__global__ void k_compress_long(int64_t nrows, int64_t ncols, const int64_t *__restrict__ rp,
-                                const int32_t *__restrict__ col, int2 *__restrict__ pairs,
-                                int32_t *__restrict__ ccnt, int2 *__restrict__ minmax,
-                                int4 *__restrict__ desc, int2 *__restrict__ ana, int *err,
-                                int *unsorted_flag, const int *long_flag) {
-    // k_compress found no long row (the flag is cleared before it runs)
-    if (long_flag && *(volatile const int *)long_flag == 0) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// The same for the listed rows (longer than COMPRESS_LONG), a block per row,
+// COMPRESS_CHUNK entries at a time staged in shared memory: a pair starts
+// where an entry's block differs from the previous entry's (its place is the
+// number of starts before it, a block scan), and the thread at a start ORs the
+// bits of the run that follows.  A warp per row took 32 entries at a time with
+// a segmented scan of the masks and a carried run: a serial chain of 488
+// steps for the longest row of an R-MAT graph of scale 17, 1.5 ms for its 3.7 M
+// entries (0.074 now; scale 13 0.25 -> 0.015 ms).
+constexpr int COMPRESS_BS = 256, COMPRESS_PT = 4, COMPRESS_CHUNK = COMPRESS_BS * COMPRESS_PT;
+
+__global__ void __launch_bounds__(COMPRESS_BS) k_compress_long(
+    int64_t ncols, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int2 *__restrict__ pairs,
+    int32_t *__restrict__ ccnt, int2 *__restrict__ minmax, int4 *__restrict__ desc, int2 *__restrict__ ana, int *err,
+    int *unsorted_flag, const int *long_count, const int32_t *__restrict__ long_list) {
+    constexpr int NW = COMPRESS_BS / 32;
+    __shared__ __align__(16) int st[COMPRESS_CHUNK];
+    __shared__ int wsum[NW], wmin[NW], wmax[NW];
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int nlong = *(volatile const int *)long_count;
     bool bad = false, unsorted = false;
-    // a warp tests 32 rows at once and compresses the long ones among them;
-    // the rows a warp tests are `warps` apart (row wg + warps * m), so that
-    // long rows stored next to each other (the heavy rows of a power-law
-    // graph cluster at the low indices) go to different warps
-    for (int64_t m0 = 0; wg + warps * m0 < nrows; m0 += 32) {
-      const int64_t rl = wg + warps * (m0 + lane);
-      unsigned longs = __ballot_sync(0xffffffffu, rl < nrows && rp[rl + 1] - rp[rl] > COMPRESS_LONG);
-      while (longs) {
-        const int64_t r = wg + warps * (m0 + __ffs(longs) - 1);
-        longs &= longs - 1u;
+    for (int t = blockIdx.x; t < nlong; t += gridDim.x) {
+        const int64_t r = long_list[t];
         const int64_t beg = rp[r], end = rp[r + 1];
-        int cblk = -1;          // block of the run carried from the previous 32 (-1: none)
-        unsigned cmask = 0;
-        int npairs = 0;         // runs started so far (the carried one included)
-        int prevc = -1;         // last valid column of the previous 32
-        int bmin = INT_MAX, bmax = INT_MIN;
-        for (int64_t base = beg; base < end; base += 32) {
-            const int64_t p = base + lane;
-            int c = p < end ? col[p] : -1;
-            if (c >= 0 && (int64_t)c >= ncols) { bad = true; c = -1; }
-            if (p < end && c < 0) bad = true;
-            const bool valid = c >= 0;
-            // sortedness against the previous valid entry in storage order
-            int pc = __shfl_up_sync(0xffffffffu, c, 1);
-            if (lane == 0) pc = prevc;
-            unsorted |= valid && pc >= 0 && c <= pc;
-            const int b = valid ? c >> 5 : -2;
-            int pb = __shfl_up_sync(0xffffffffu, b, 1);
-            if (lane == 0) pb = cblk;
-            bool start = valid && b != pb;
-            unsigned m = valid ? 1u << (c & 31) : 0u;
-            if (lane == 0 && valid && !start) m |= cmask;   // continues the carried run
-            // invalid lanes (bad columns) break runs: they act as run starts with no bits
-            bool seg = start || !valid;
+        int npairs = 0, bmin = INT_MAX, bmax = INT_MIN;
+        for (int64_t base = beg; base < end; base += COMPRESS_CHUNK) {
+            const int n = (int)min((int64_t)COMPRESS_CHUNK, end - base);
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < COMPRESS_PT; u++) {
+                const int x = tid + u * COMPRESS_BS;
+                int c = x < n ? col[base + x] : -1;
+                if (x < n && (c < 0 || (int64_t)c >= ncols)) { bad = true; c = -1; }   // breaks its run
+                st[x] = c;
+            }
+            int prev = -1;
+            if (tid == 0 && base > beg) {
+                prev = col[base - 1];
+                if (prev < 0 || (int64_t)prev >= ncols) prev = -1;
+            }
+            __syncthreads();
+            const int e0 = tid * COMPRESS_PT;
+            if (tid > 0) prev = st[e0 - 1];
+            unsigned starts = 0;
+#pragma unroll
+            for (int u = 0; u < COMPRESS_PT; u++) {
+                const int c = st[e0 + u];
+                if (c >= 0) {
+                    if (prev < 0 || (c >> 5) != (prev >> 5)) starts |= 1u << u;
+                    unsorted |= c <= prev;
+                    bmin = min(bmin, c >> 5);
+                    bmax = max(bmax, c >> 5);
+                }
+                prev = c;
+            }
+            const int mine = __popc(starts);
+            int incl = mine;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
-                const unsigned ym = __shfl_up_sync(0xffffffffu, m, d);
-                const bool ys = __shfl_up_sync(0xffffffffu, seg, d);
-                if (lane >= d && !seg) m |= ym;
-                if (lane >= d) seg = seg || ys;
+                const int y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += y;
             }
-            const unsigned starts = __ballot_sync(0xffffffffu, start);
-            const int idx = npairs + __popc(starts & ((2u << lane) - 1u)) - 1;
-            // the carried run, if it ends before this 32 continues it
-            if (lane == 0 && cblk >= 0 && !(valid && !start)) {
-                if (pairs) pairs[beg + npairs - 1] = make_int2(cblk, (int)cmask);
+            if (lane == 31) wsum[w] = incl;
+            __syncthreads();
+            int idx = npairs + incl - mine;
+#pragma unroll
+            for (int j = 0; j < NW; j++) {
+                if (j < w) idx += wsum[j];
+                npairs += wsum[j];
             }
-            const bool nxt_start = __shfl_down_sync(0xffffffffu, start || !valid, 1);
-            const bool last_valid = valid && (lane == 31 || nxt_start);
-            const unsigned lastm = __ballot_sync(0xffffffffu, valid);
-            const int top = lastm ? 31 - __clz(lastm) : -1;   // last valid lane
-            // runs that end inside this 32 are written; the one at the last
-            // valid lane is carried unless the row ends here
-            const bool row_ends = base + 32 >= end;
-            if (last_valid && (lane != top || row_ends) && pairs && idx >= 0) pairs[beg + idx] = make_int2(b, (int)m);
-            npairs += __popc(starts);
-            if (top >= 0) {
-                const int tb = __shfl_sync(0xffffffffu, b, top);
-                const unsigned tm = __shfl_sync(0xffffffffu, m, top);
-                cblk = row_ends ? -1 : tb;
-                cmask = row_ends ? 0u : tm;
-                prevc = __shfl_sync(0xffffffffu, c, top);
+            while (starts) {
+                const int e = e0 + __ffs(starts) - 1;
+                starts &= starts - 1u;
+                const int b = st[e] >> 5;
+                unsigned m = 0;
+                int p = e;
+                for (; p < n && st[p] >> 5 == b; p++) m |= 1u << (st[p] & 31);   // -1 >> 5 is no block
+                for (int64_t q = base + n; p == n && q < end; q++) {             // a run past the chunk
+                    const int c = col[q];
+                    if (c >> 5 != b) break;
+                    m |= 1u << (c & 31);
+                }
+                if (pairs) pairs[beg + idx] = make_int2(b, (int)m);
+                idx++;
             }
-            if (valid) { bmin = min(bmin, b); bmax = max(bmax, b); }
         }
-        if (cblk >= 0 && lane == 0 && pairs) pairs[beg + npairs - 1] = make_int2(cblk, (int)cmask);
-        for (int d = 16; d > 0; d >>= 1) {
-            bmin = min(bmin, __shfl_xor_sync(0xffffffffu, bmin, d));
-            bmax = max(bmax, __shfl_xor_sync(0xffffffffu, bmax, d));
-        }
+        bmin = __reduce_min_sync(0xffffffffu, bmin);
+        bmax = __reduce_max_sync(0xffffffffu, bmax);
         if (lane == 0) {
+            wmin[w] = bmin;
+            wmax[w] = bmax;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            for (int j = 1; j < NW; j++) {
+                bmin = min(bmin, wmin[j]);
+                bmax = max(bmax, wmax[j]);
+            }
             const int len = (int)(end - beg);
             if (ccnt) ccnt[r] = npairs;
             if (minmax) minmax[r] = make_int2(bmin, bmax);
             if (desc) desc[r] = make_int4((int)(unsigned)(uint64_t)beg, (int)((uint64_t)beg >> 32), len, npairs);
             if (ana) ana[r] = make_int2(len, npairs);
         }
-      }
     }
-    unsorted = __any_sync(0xffffffffu, unsorted);
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane == 0 && bad) atomicOr(err, DERR_COL_RANGE);
-    if (lane == 0 && unsorted && unsorted_flag) atomicOr(unsorted_flag, 1);
+    if (bad) atomicOr(err, DERR_COL_RANGE);
+    if (unsorted && unsorted_flag) *unsorted_flag = 1;
 }
 
 int launch_compress(const spgemm_csr &M, int2 *pairs, int32_t *ccnt, int2 *minmax, int4 *desc,
-                    int2 *ana, int *err, Ctx &c, int *unsorted, int *long_flag) {
+                    int2 *ana, int *err, int *long_count, int32_t *long_list, Ctx &c, int *unsorted) {
     if (M.nrows == 0) return SPGEMM_OK;
     int64_t blocks = (M.nrows + COMPRESS_WPB * 32 - 1) / (COMPRESS_WPB * 32);
     c.begin("compress", M.nrows);
     k_compress<<<(unsigned)blocks, COMPRESS_WPB * 32, 0, c.s>>>(M.nrows, M.ncols, M.row_ptr, M.col_idx, pairs,
-                                                    ccnt, minmax, desc, ana, err, unsorted, long_flag);
+                                                    ccnt, minmax, desc, ana, err, unsorted, long_count, long_list);
     c.end();
-    // one resident wave (it returns at once when no row is long)
-    const int64_t wblocks = std::min<int64_t>((M.nrows + 255) / 256, resident_blocks(k_compress_long, 256, c.nsm));
-    c.begin("compress_long", M.nrows);
-    k_compress_long<<<(unsigned)wblocks, 256, 0, c.s>>>(M.nrows, M.ncols, M.row_ptr, M.col_idx, pairs, ccnt,
-                                                        minmax, desc, ana, err, unsorted, long_flag);
-    c.end();
+    if (M.nnz > COMPRESS_LONG) {
+        // one resident wave (it returns at once when no row is long)
+        const int64_t wblocks = std::min<int64_t>(M.nnz / (COMPRESS_LONG + 1), resident_blocks(k_compress_long, COMPRESS_BS, c.nsm));
+        c.begin("compress_long", M.nrows);
+        k_compress_long<<<(unsigned)wblocks, COMPRESS_BS, 0, c.s>>>(M.ncols, M.row_ptr, M.col_idx, pairs, ccnt, minmax,
+                                                                    desc, ana, err, unsorted, long_count, long_list);
+        c.end();
+    }
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
@@ -229,10 +244,12 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
                           const int64_t *__restrict__ arp, const int32_t *__restrict__ acol,
                           const int2 *__restrict__ ana, const int2 *__restrict__ bmm, int64_t *__restrict__ flops,
                           uint8_t *__restrict__ bins, int64_t *__restrict__ crp, int2 *__restrict__ rspan,
-                          DevState *st) {
+                          DevState *st, bool bitmaps) {
     __shared__ unsigned long long hist[NBINS];
     __shared__ unsigned long long fsum;
     __shared__ unsigned long long alen_max;
+    __shared__ int marks[2];   // rows without a mark, with one
+    if (threadIdx.x < 2) marks[threadIdx.x] = 0;
     if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) { fsum = 0; alen_max = 0; }
     __syncthreads();
@@ -248,10 +265,11 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
         const bool live = i < nrows;
         long long f = 0, cp = 0;
         int lo = INT_MAX, hi = -1;
+        bool rowbad = false;
         if (live) {
             for (int64_t p = arp[i] + lane; p < arp[i + 1]; p += AN_G) {
                 int k = acol[p];
-                if (k < 0 || (int64_t)k >= nrows_b) { bad = true; continue; }
+                if (k < 0 || (int64_t)k >= nrows_b) { bad = rowbad = true; continue; }
                 const int2 d = ana[k], m = bmm[k];
                 f += d.x;
                 cp += d.y;
@@ -265,6 +283,7 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
             lo = min(lo, __shfl_xor_sync(gmask, lo, d, AN_G));
             hi = max(hi, __shfl_xor_sync(gmask, hi, d, AN_G));
         }
+        rowbad = (__ballot_sync(0xffffffffu, rowbad) & gmask) != 0;
         int b = BIN_EMPTY;
         const bool lead = live && lane == 0;
         if (lead) {
@@ -273,8 +292,16 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
             flops[i] = f;
             bins[i] = (uint8_t)b;
             rspan[i] = make_int2(lo, hi >= lo ? hi - lo + 1 : 0);
-            if (b == BIN_EMPTY) crp[i + 1] = 0;
-            if (b == BIN_HUGE) crp[i + 1] = -1;
+            if (bitmaps) {
+                if (rowbad) b = BIN_EMPTY;
+                bins[i] = (uint8_t)b;
+                const int mark = b == BIN_EMPTY ? 0 : sym_mark(cp, hi - lo + 1);
+                crp[i + 1] = mark;
+                if (b != BIN_EMPTY) marks[mark != 0] = 1;
+            } else {
+                if (b == BIN_EMPTY) crp[i + 1] = 0;
+                if (b == BIN_HUGE) crp[i + 1] = -1;
+            }
             wf += f;
             wl = max(wl, (long long)(arp[i + 1] - arp[i]));
         }
@@ -290,6 +317,8 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
     if ((threadIdx.x & 31) == 0 && wl) atomicMax(&alen_max, (unsigned long long)wl);
     __syncthreads();
     if (threadIdx.x == 0 && fsum) atomicAdd((unsigned long long *)&st->flops_total, fsum);
+    if (threadIdx.x == 0 && marks[0]) *(volatile int *)&st->sym_first = 1;
+    if (threadIdx.x == 0 && marks[1]) *(volatile int *)&st->sym_marked = 1;
     if (threadIdx.x == 0 && alen_max && alen_max > (unsigned long long)*(volatile long long *)&st->max_alen)
         atomicMax((unsigned long long *)&st->max_alen, alen_max);
     if (threadIdx.x < NBINS && hist[threadIdx.x]) {
@@ -300,7 +329,7 @@ __global__ void k_analyze(int64_t nrows, int64_t nrows_b, int64_t nwords,
 }
 
 int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, const int2 *bmm, int64_t *flops,
-                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, Ctx &c) {
+                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, bool bitmaps, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     int64_t threads = A.nrows * AN_G;
     int64_t blocks = (threads + 255) / 256;
@@ -308,7 +337,7 @@ int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, co
     int64_t nwords = (B.ncols + 31) / 32;
     c.begin("analyze", A.nrows);
     k_analyze<<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, B.nrows, nwords, A.row_ptr, A.col_idx,
-                                                   ana, bmm, flops, bins, crp, rspan, st);
+                                                   ana, bmm, flops, bins, crp, rspan, st, bitmaps);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
@@ -347,58 +376,7 @@ int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, i
     return SPGEMM_OK;
 }
 
-// ---------------------------------------------------------------- numeric bins
-__global__ void k_numeric_binning(int64_t n, const int64_t *__restrict__ crp,
-                                  const int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
-                                  uint8_t *__restrict__ cls, const int2 *__restrict__ rspan, DevState *st,
-                                  bool dense_ok, const int32_t *__restrict__ nlo) {
-    __shared__ unsigned long long hist[NBINS];
-    __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS];
-    if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
-    if (threadIdx.x < NCLS) ccnt[threadIdx.x] = cnnz[threadIdx.x] = cwords[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int b = BIN_EMPTY;
-    if (i < n) {
-        long long c = crp[i + 1] - crp[i];
-        const long long f = flops[i];
-        b = c > 0 ? num_bin(c, f) : BIN_EMPTY;
-        if (b != BIN_EMPTY && nlo && nlo[i] >= 0 && c <= NARROW_NMAX && f <= NARROW_FLOPS) b = BIN_NARROW;
-        bins[i] = (uint8_t)b;
-        if (b == BIN_HUGE) atomicMax((unsigned long long *)&st->max_row_nnz, (unsigned long long)c);
-        int k = CLS_NONE;
-        if (b >= 2 && b <= BIN_HUGE) {
-            const int words = rspan[i].y;
-            k = num_cls(b, c, f, words, dense_ok && st->b_unsorted == 0);
-            atomicAdd(&ccnt[k], 1);
-            if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
-            if (words > cwords[k]) atomicMax(&cwords[k], words);
-        }
-        cls[i] = (uint8_t)k;
-    }
-    warp_hist(hist, i < n, b);
-    __syncthreads();
-    if (threadIdx.x < NBINS && hist[threadIdx.x])
-        atomicAdd((unsigned long long *)&st->bin_count[1][threadIdx.x], hist[threadIdx.x]);
-    if (threadIdx.x < NCLS && ccnt[threadIdx.x]) {
-        atomicAdd((unsigned long long *)&st->cls_count[threadIdx.x], (unsigned long long)ccnt[threadIdx.x]);
-        if (cnnz[threadIdx.x] > *(volatile int *)&st->cls_nnz[threadIdx.x])
-            atomicMax(&st->cls_nnz[threadIdx.x], cnnz[threadIdx.x]);
-        if (cwords[threadIdx.x] > *(volatile int *)&st->cls_words[threadIdx.x])
-            atomicMax(&st->cls_words[threadIdx.x], cwords[threadIdx.x]);
-    }
-}
-
-int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                           const int2 *rspan, DevState *st, bool dense_ok, Ctx &c, const int32_t *nlo) {
-    if (n == 0) return SPGEMM_OK;
-    c.begin("numeric_binning", n);
-    k_numeric_binning<<<(unsigned)((n + 255) / 256), 256, 0, c.s>>>(n, crp, flops, bins, cls, rspan, st, dense_ok, nlo);
-    c.end();
-    SG_CUDA(cudaGetLastError());
-    return SPGEMM_OK;
-}
-
+// ---------------------------------------------------------------- row lists
 // Row lists for the list-driven kernels.  CLS false (symbolic second pass):
 // rows marked -1 in crp[i+1] (overflowed the first pass, or bin 6), listed by
 // max(key[i], 2), key the bins.  CLS true (numeric): rows of the classes
@@ -458,9 +436,9 @@ int launch_scatter_cls(int64_t n, const uint8_t *cls, int32_t *rows, DevState *s
 }
 
 // ---------------------------------------------------------------- scan
-// Reduce-then-scan over tiles of SCAN_TILE counts: tile sums, one block scans
-// the sums (looping with a carry), then every tile is rescanned with its
-// offset.  x[0] is set to 0 and x[1..n] becomes the inclusive prefix.
+// Reduce-then-scan over tiles of SCAN_TILE counts: tile sums, then every tile
+// is rescanned with the sum of the tiles before it (with more than SCAN_DIRECT
+// tiles, one block scans the sums first, looping with a carry).  x[0] is set to 0 and x[1..n] becomes the inclusive prefix.
 constexpr int SCAN_BS = 256, SCAN_PT = 8, SCAN_TILE = SCAN_BS * SCAN_PT;
 
 size_t scan_tmp_bytes(int64_t n) {
@@ -521,11 +499,47 @@ __global__ void k_scan_sums(long long *tile_sums, int64_t tiles, long long *tota
     if (threadIdx.x == 0) *total = carry;
 }
 
-__global__ void k_scan_apply(int64_t *__restrict__ x, int64_t n, const long long *tile_sums) {
+// Numeric bin and class of the rows whose counts the scan walks over, in the
+// same pass (k_scan_apply<true>): the counts are in registers there, and a
+// pass of its own read the offsets again and cost a launch.
+struct ScanBins {
+    const int64_t *flops;
+    uint8_t *bins, *cls;
+    const int2 *rspan;
+    const int32_t *nlo;   // may be null
+    DevState *st;
+    bool dense_ok;
+};
+
+// SUMMED: tile_sums holds the tiles' exclusive prefix (k_scan_sums); else
+// every block adds up the sums of the tiles before its own, which costs less
+// than the launch of k_scan_sums while there are at most SCAN_DIRECT tiles,
+// and the last block writes the total.
+constexpr int64_t SCAN_DIRECT = 4096;
+
+template <bool BINS, bool SUMMED>
+__global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x, int64_t n,
+                                                        const long long *__restrict__ tile_sums, long long *total,
+                                                        ScanBins b) {
     __shared__ long long sh[SCAN_BS / 32];
     __shared__ long long tot;
+    __shared__ unsigned long long hist[NBINS];
+    __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS];
+    if (BINS) {
+        if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
+        if (threadIdx.x < NCLS) ccnt[threadIdx.x] = cnnz[threadIdx.x] = cwords[threadIdx.x] = 0;
+    }
+    long long before = 0;
+    if (SUMMED) {
+        before = tile_sums[blockIdx.x];
+    } else if (blockIdx.x > 0) {
+        long long s = 0;
+        for (unsigned t = threadIdx.x; t < blockIdx.x; t += SCAN_BS) s += tile_sums[t];
+        block_excl_scan(s, sh, &tot);
+        before = tot;
+    }
     int64_t *x1 = x + 1;
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_PT;
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_PT;
     long long v[SCAN_PT];
     long long s = 0;
 #pragma unroll
@@ -533,13 +547,69 @@ __global__ void k_scan_apply(int64_t *__restrict__ x, int64_t n, const long long
         v[j] = base + j < n ? x1[base + j] : 0;
         s += v[j];
     }
-    long long e = block_excl_scan(s, sh, &tot) + tile_sums[blockIdx.x];
+    long long e = before + block_excl_scan(s, sh, &tot);
+    if (!SUMMED && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = before + tot;
 #pragma unroll
     for (int j = 0; j < SCAN_PT; j++) {
         e += v[j];
         if (base + j < n) x1[base + j] = e;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) x[0] = 0;
+    if (!BINS) return;
+#pragma unroll
+    for (int j = 0; j < SCAN_PT; j++) {
+        const int64_t i = base + j;
+        int bin = BIN_EMPTY;
+        if (i < n) {
+            const long long c = v[j], f = b.flops[i];
+            bin = c > 0 ? num_bin(c, f) : BIN_EMPTY;
+            if (bin != BIN_EMPTY && b.nlo && b.nlo[i] >= 0 && c <= NARROW_NMAX && f <= NARROW_FLOPS) bin = BIN_NARROW;
+            b.bins[i] = (uint8_t)bin;
+            if (bin == BIN_HUGE) atomicMax((unsigned long long *)&b.st->max_row_nnz, (unsigned long long)c);
+            int k = CLS_NONE;
+            if (bin >= 2 && bin <= BIN_HUGE) {
+                const int words = b.rspan[i].y;
+                k = num_cls(bin, c, f, words, b.dense_ok && b.st->b_unsorted == 0);
+                atomicAdd(&ccnt[k], 1);
+                if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
+                if (words > cwords[k]) atomicMax(&cwords[k], words);
+            }
+            b.cls[i] = (uint8_t)k;
+        }
+        warp_hist(hist, i < n, bin);
+    }
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < NBINS && hist[t]) atomicAdd((unsigned long long *)&b.st->bin_count[1][t], hist[t]);
+    if (t < NCLS && ccnt[t]) {
+        atomicAdd((unsigned long long *)&b.st->cls_count[t], (unsigned long long)ccnt[t]);
+        if (cnnz[t] > *(volatile int *)&b.st->cls_nnz[t]) atomicMax(&b.st->cls_nnz[t], cnnz[t]);
+        if (cwords[t] > *(volatile int *)&b.st->cls_words[t]) atomicMax(&b.st->cls_words[t], cwords[t]);
+    }
+}
+
+template <bool BINS>
+static int run_scan(int64_t *x, int64_t n, long long *total, void *tmp, const ScanBins &b, Ctx &c) {
+    const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    long long *sums = (long long *)tmp;
+    if (tiles > 1) {
+        c.begin("scan_tiles", n);
+        k_scan_tiles<<<(unsigned)tiles, SCAN_BS, 0, c.s>>>(x + 1, n, sums);
+        c.end();
+    }
+    if (tiles > SCAN_DIRECT) {
+        c.begin("scan_sums", tiles);
+        k_scan_sums<<<1, SCAN_BS, 0, c.s>>>(sums, tiles, total);
+        c.end();
+    }
+    c.begin("scan_apply", n);
+    if (tiles > SCAN_DIRECT)
+        k_scan_apply<BINS, true><<<(unsigned)tiles, SCAN_BS, 0, c.s>>>(x, n, sums, total, b);
+    else
+        k_scan_apply<BINS, false><<<(unsigned)tiles, SCAN_BS, 0, c.s>>>(x, n, sums, total, b);
+    c.end();
+    SG_CUDA(cudaGetLastError());
+    return SPGEMM_OK;
 }
 
 int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &c) {
@@ -548,19 +618,13 @@ int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &
         SG_CUDA(cudaMemsetAsync(total, 0, sizeof(long long), c.s));
         return SPGEMM_OK;
     }
-    int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    long long *sums = (long long *)tmp;
-    c.begin("scan_tiles", n);
-    k_scan_tiles<<<(unsigned)tiles, SCAN_BS, 0, c.s>>>(x + 1, n, sums);
-    c.end();
-    c.begin("scan_sums", tiles);
-    k_scan_sums<<<1, SCAN_BS, 0, c.s>>>(sums, tiles, total);
-    c.end();
-    c.begin("scan_apply", n);
-    k_scan_apply<<<(unsigned)tiles, SCAN_BS, 0, c.s>>>(x, n, sums);
-    c.end();
-    SG_CUDA(cudaGetLastError());
-    return SPGEMM_OK;
+    return run_scan<false>(x, n, total, tmp, ScanBins{}, c);
+}
+
+int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
+                        const int2 *rspan, const int32_t *nlo, DevState *st, bool dense_ok, Ctx &c) {
+    if (n == 0) return launch_scan_counts(crp, n, &st->nnz, tmp, c);
+    return run_scan<true>(crp, n, &st->nnz, tmp, ScanBins{flops, bins, cls, rspan, nlo, st, dense_ok}, c);
 }
 
 }  // namespace sg

@@ -308,7 +308,7 @@ static int lanes_for(double x, int lo = 8) {
 // overlap it.
 struct WsLayout {
     size_t bins, cls, rows, desc, mm, spans, nlo, nwords, ulist, persist;   // persistent
-    size_t ana, flops, pairs, ccnt, tmp, gws;                          // symbolic scratch
+    size_t ana, flops, pairs, ccnt, longs, tmp, gws;                   // symbolic scratch
 };
 static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     WsLayout L;
@@ -326,7 +326,8 @@ static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     L.pairs = L.ana + align_up((size_t)nb * 8);
     L.flops = L.pairs + align_up((size_t)nnzb * 8);
     L.ccnt = L.flops + align_up((size_t)n * 8);
-    L.tmp = L.ccnt + align_up((size_t)nb * 4);
+    L.longs = L.ccnt + align_up((size_t)nb * 4);
+    L.tmp = L.longs + align_up((size_t)nb * 4);
     L.gws = L.tmp + align_up(scan_tmp_bytes(n));
     return L;
 }
@@ -374,8 +375,11 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         const double mean_alen = (double)A->nnz / (double)n;
         const double mean_pairs = mean_alen * ((double)B->nnz / (double)(B->nrows > 0 ? B->nrows : 1)) * 0.6;
         const int gs = h->g_symbolic ? h->g_symbolic : lanes_for(mean_pairs / 64.0);
-        SG_TRY(launch_compress(*B, pairs, ccnt, minmax, desc, ana, &h->dstate->err, c,
-                               &h->dstate->b_unsorted, &h->dstate->long_rows));
+        SG_TRY(launch_compress(*B, pairs, ccnt, minmax, desc, ana, &h->dstate->err, &h->dstate->long_rows,
+                               (int32_t *)(w + L.longs), c, &h->dstate->b_unsorted));
+        // B's column blocks fit a bitmap in shared memory: every row is counted
+        // without a list length on the host, so the host waits once a call
+        const bool bitmaps = (B->ncols + 31) / 32 <= SYM_BITMAP_WORDS;
         h->sym_narrow_used = h->narrow;
         if (h->narrow) {
             // analysis and the narrow rows' counts in one pass; the first
@@ -383,34 +387,39 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
             // lanes per row: rows of A longer than 32 entries take 8
             const int gn = h->g_narrow_sym ? h->g_narrow_sym : (mean_alen <= 32.0 ? 4 : 8);
             SG_TRY(launch_sym_narrow(*A, *B, desc, minmax, pairs, flops, bins, C_row_ptr, rspan, nlo, nwords,
-                                     ulist, h->dstate, gn, c));
+                                     ulist, h->dstate, bitmaps, gn, c));
         } else {
-            SG_TRY(launch_analyze(*A, *B, ana, minmax, flops, bins, C_row_ptr, rspan, h->dstate, c));
+            SG_TRY(launch_analyze(*A, *B, ana, minmax, flops, bins, C_row_ptr, rspan, h->dstate, bitmaps, c));
         }
-        SG_TRY(launch_symbolic_first(*A, bins, desc, pairs, C_row_ptr, h->dstate, gs, c));
-        SG_TRY(fetch_state(h, s));
-        SG_TRY(device_errors(h->hstate->err));
-        long long second = 0;
-        for (int b = 2; b <= BIN_HUGE; b++) second += h->hstate->bin_count[0][b];
-        long long first = 0;
-        for (int b = 1; b < BIN_HUGE; b++) first += h->hstate->sym_hist[b];
-        h->sym_counts[0] = h->hstate->sym_hist[0];
-        h->sym_counts[1] = first - (second - h->hstate->bin_count[0][BIN_HUGE]);
-        for (int b = 2; b < NBINS; b++) h->sym_counts[b] = h->hstate->bin_count[0][b];
-        h->sym_counts[BIN_NARROW] = h->hstate->sym_hist[BIN_NARROW];
-        if (second > 0) {
-            SG_TRY(launch_scatter_bins(n, bins, C_row_ptr, rows, h->dstate, c));
-            SG_TRY(launch_symbolic(*A, *B, pairs, ccnt, rows, h->hstate->bin_count[0], C_row_ptr,
-                                   &h->dstate->err, w + L.gws, gws_bytes, rspan, c));
+        SG_TRY(launch_symbolic_first(*A, bins, desc, pairs, C_row_ptr, rows, h->dstate, bitmaps, gs, c));
+        if (bitmaps) {
+            SG_TRY(launch_symbolic_bitmaps(*A, *B, desc, pairs, rspan, rows, C_row_ptr, h->dstate, c));
+        } else {
+            SG_TRY(fetch_state(h, s));
+            SG_TRY(device_errors(h->hstate->err));
+            long long second = 0, first = 0;
+            for (int b = 2; b <= BIN_HUGE; b++) second += h->hstate->bin_count[0][b];
+            for (int b = 1; b < BIN_HUGE; b++) first += h->hstate->sym_hist[b];
+            h->sym_counts[0] = h->hstate->sym_hist[0];
+            h->sym_counts[1] = first - (second - h->hstate->bin_count[0][BIN_HUGE]);
+            for (int b = 2; b < NBINS; b++) h->sym_counts[b] = h->hstate->bin_count[0][b];
+            h->sym_counts[BIN_NARROW] = h->hstate->sym_hist[BIN_NARROW];
+            if (second > 0) {
+                SG_TRY(launch_scatter_bins(n, bins, C_row_ptr, rows, h->dstate, c));
+                SG_TRY(launch_symbolic(*A, *B, pairs, ccnt, rows, h->hstate->bin_count[0], C_row_ptr,
+                                       &h->dstate->err, w + L.gws, gws_bytes, rspan, c));
+            }
         }
-        SG_TRY(launch_scan_counts(C_row_ptr, n, &h->dstate->nnz, w + L.tmp, c));
         // the split table of the dense rows stays within B's own size (and 64 MB)
         const size_t dense_bytes = dense_ws(B->nrows, B->ncols);
         const bool dense_ok = dense_bytes <= (size_t)B->nnz * 12 + ((size_t)64 << 20);
-        SG_TRY(launch_numeric_binning(n, C_row_ptr, flops, bins, cls, rspan, h->dstate, dense_ok, c, h->narrow ? nlo : nullptr));
+        SG_TRY(launch_scan_binning(C_row_ptr, n, w + L.tmp, flops, bins, cls, rspan, h->narrow ? nlo : nullptr,
+                                   h->dstate, dense_ok, c));
         SG_TRY(fetch_state(h, s));
         SG_TRY(device_errors(h->hstate->err));
         *nnz_C = h->hstate->nnz;
+        if (bitmaps)
+            for (int b = 0; b < NBINS; b++) h->sym_counts[b] = h->hstate->sym_hist[b];
         h->mean_flops = (double)h->hstate->flops_total / (double)n;
         memcpy(h->num_counts, h->hstate->bin_count[1], sizeof(h->num_counts));
         for (int k = 0; k < NCLS; k++) {
@@ -1081,12 +1090,13 @@ int spgemm_compress(spgemm_handle h, const spgemm_csr *M, int32_t *count, uint32
     SG_TRY(check_csr(M, "M", false));
     cudaStream_t s = (cudaStream_t)stream;
     SG_CUDA(cudaSetDevice(h->device));
-    size_t need = align_up((size_t)M->nrows * 8);
-    SG_TRY(ws_reserve(h, need, s));
+    const size_t need = align_up((size_t)M->nrows * 8);
+    SG_TRY(ws_reserve(h, need + align_up((size_t)M->nrows * 4), s));
     h->sym_valid = false;
     Ctx c = h->ctx(s);
-    SG_TRY(launch_compress(*M, (int2 *)pairs, count, (int2 *)h->ws, nullptr, nullptr,
-                           &h->dstate->err, c));
+    SG_CUDA(cudaMemsetAsync(&h->dstate->long_rows, 0, sizeof(int), s));
+    SG_TRY(launch_compress(*M, (int2 *)pairs, count, (int2 *)h->ws, nullptr, nullptr, &h->dstate->err,
+                           &h->dstate->long_rows, (int32_t *)(h->ws + need), c));
     return SPGEMM_OK;
 }
 

@@ -44,7 +44,7 @@ struct DevState {          // lives in device memory, one per handle
     long long max_row_nnz;   // largest row of C (numeric binning)
     long long flops_total;   // products of the whole product (analysis)
     int b_unsorted;          // some row of B has columns out of ascending order
-    int long_rows;           // the compression met rows for its warp-per-row pass
+    int long_rows;           // rows the compression left to its block-per-row pass
     long long max_alen;      // longest row of A (analysis)
     unsigned long long triangles;   // spgemm_triangles: the count
     // numeric rows by class (NumCls): rows, list cursors, largest row of C,
@@ -53,6 +53,10 @@ struct DevState {          // lives in device memory, one per handle
     long long cls_cursor[16];
     int cls_nnz[16], cls_words[16];
     unsigned long long next_row;   // rows a kernel has handed out (cleared before it)
+    // symbolic phase: whether the 32-slot maps have rows, whether rows are
+    // marked for bitmaps; rows of a warp's bitmap, rows of a block's bitmap
+    int sym_first, sym_marked;
+    unsigned long long sym_warp, sym_block;
 };
 
 // ---------------------------------------------------------------- bins
@@ -62,6 +66,23 @@ struct DevState {          // lives in device memory, one per handle
 constexpr int BIN_EMPTY = 0;
 constexpr int BIN_HUGE = 6;     // widest bin: unbounded accumulator
 constexpr int NBINS = SPGEMM_NBINS;
+
+// Symbolic phase of a B of at most SYM_BITMAP_WORDS blocks of 32 columns (its
+// bitmap fits a block's shared memory), rows that are not narrow: at most
+// SYM_FIRST_PAIRS compressed pairs: a 32-slot map, which holds them whatever
+// their blocks; more pairs over at most SYM_WARP_WORDS blocks and at most
+// SYM_WARP_PAIRS of them: a warp and a bitmap of the row's span (marked
+// SYM_MARK_WARP in crp[i+1] until counted); the others: a block and a bitmap
+// (SYM_MARK_BLOCK).  A wider B goes through the optimistic first pass and the
+// lists by bin.
+constexpr int64_t SYM_BITMAP_WORDS = 53248;   // 208 KB
+constexpr int SYM_WARP_WORDS = 2048;
+constexpr long long SYM_FIRST_PAIRS = 32, SYM_WARP_PAIRS = 4096;
+constexpr int SYM_MARK_WARP = -1, SYM_MARK_BLOCK = -2;
+__host__ __device__ inline int sym_mark(long long cpairs, int words) {
+    if (cpairs <= SYM_FIRST_PAIRS) return 0;
+    return cpairs <= SYM_WARP_PAIRS && words <= SYM_WARP_WORDS ? SYM_MARK_WARP : SYM_MARK_BLOCK;
+}
 
 // Numeric bins by exact output count (and product count):
 //   1: <= 16 entries, 2: <= 32 (both: lanes of a warp, map in shared memory,
@@ -240,11 +261,10 @@ struct Ctx {
 // desc[k] = {row_ptr[k] low, high 32 bits, entries, pairs};
 // ana[k] = {entries, pairs}.  Any output may be NULL.
 // `unsorted` (may be null) is set to 1 if a row of M is not strictly ascending.
-// `long_flag` (may be null; device, cleared by the caller before the call)
-// is set to 1 if a row is long enough for the warp-per-row pass, which
-// otherwise returns at once; with null that pass tests every row.
+// `long_count` (device, cleared by the caller before the call) and
+// `long_list` (room for M.nrows): the rows left to the block-per-row pass.
 int launch_compress(const spgemm_csr &M, int2 *pairs, int32_t *ccnt, int2 *minmax, int4 *desc,
-                    int2 *ana, int *err, Ctx &c, int *unsorted = nullptr, int *long_flag = nullptr);
+                    int2 *ana, int *err, int *long_count, int32_t *long_list, Ctx &c, int *unsorted = nullptr);
 __device__ __forceinline__ int64_t desc_start(int4 d) {
     return (int64_t)(((uint64_t)(unsigned)d.y << 32) | (uint64_t)(unsigned)d.x);
 }
@@ -254,15 +274,18 @@ size_t scan_tmp_bytes(int64_t n);
 int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &c);
 // Per row i of A: flops, symbolic bin, column-block span rspan[i] = {first
 // block, blocks} of the rows of B it reaches ({INT_MAX, 0} if none; bmm[k] =
-// {first block, last block} of B_k); empty rows get crp[i+1] = 0.
+// {first block, last block} of B_k); empty rows get crp[i+1] = 0.  bitmaps: B fits
+// SYM_BITMAP_WORDS, and rows get their mark (sym_mark) in crp[i+1]; a row with
+// a column of A out of range gets 0 then (no kernel may read it).
 int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, const int2 *bmm, int64_t *flops,
-                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, Ctx &c);
-// Numeric bin of every row from its output count crp[i+1]-crp[i] and flops;
-// rows the symbolic phase found narrow (nlo[i] >= 0; nlo may be null) that
-// fit the narrow numeric kernel get BIN_NARROW.
-// cls[i]: the row's class (num_cls); rows, largest row and span per class in st.
-int launch_numeric_binning(int64_t n, const int64_t *crp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                           const int2 *rspan, DevState *st, bool dense_ok, Ctx &c, const int32_t *nlo = nullptr);
+                   uint8_t *bins, int64_t *crp, int2 *rspan, DevState *st, bool bitmaps, Ctx &c);
+// launch_scan_counts of the counts of C's rows into st->nnz, and in the same
+// pass the numeric bin of every row from its outputs and flops; rows the
+// symbolic phase found narrow (nlo[i] >= 0; nlo may be null) that fit the
+// narrow numeric kernel get BIN_NARROW.  cls[i]: the row's class (num_cls);
+// rows, largest row and span per class in st.
+int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
+                        const int2 *rspan, const int32_t *nlo, DevState *st, bool dense_ok, Ctx &c);
 // Row lists of the symbolic second pass by bin: rows[offset(b) + t], offsets
 // from st->bin_count[0].
 int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows, DevState *st, Ctx &c);
@@ -281,7 +304,7 @@ int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, i
 // first column << 8, mask}) and their number in nwords[i].
 int launch_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
                       const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
-                      uint8_t *nwords, uint2 *ulist, DevState *st, int G, Ctx &c);
+                      uint8_t *nwords, uint2 *ulist, DevState *st, bool bitmaps, int G, Ctx &c);
 // Numeric phase of the rows with bins[i] == BIN_NARROW (F32 or native F64),
 // from the word lists of the symbolic phase; G lanes per row (4, 8 or 16).
 int launch_num_narrow(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
@@ -290,9 +313,15 @@ int launch_num_narrow(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgem
 
 // symbolic.cu
 // First pass over all rows with a 32-slot map and G lanes per row (rows of
-// bins EMPTY, HUGE and NARROW are skipped).
-int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc,
-                          const int2 *pairs, int64_t *crp, DevState *st, int G, Ctx &c);
+// bins EMPTY, HUGE and NARROW are skipped).  With bitmaps, marked rows are
+// skipped too and listed instead (room for all rows): those for a warp from
+// rows[0] on, those for a block from rows[nrows(A) - 1] downwards.
+int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
+                          int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, int G, Ctx &c);
+// The listed rows, counted over bitmaps of their span; no list length is
+// needed on the host.
+int launch_symbolic_bitmaps(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *pairs,
+                            const int2 *rspan, const int32_t *rows, int64_t *crp, DevState *st, Ctx &c);
 // Second pass: kernels of bins 2..6; counts[b] = rows in bin b (host),
 // rows = concatenated bin lists, rspan[i] = column-block span of row i.
 // Writes nnz(C_i) to crp[i+1].

@@ -100,13 +100,15 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc, const int2 *__restrict__ bmm,
     const int2 *__restrict__ pairs, int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
     int64_t *__restrict__ crp, int2 *__restrict__ rspan, int32_t *__restrict__ nlo, uint8_t *__restrict__ nwords,
-    uint2 *__restrict__ ulist, DevState *st) {
+    uint2 *__restrict__ ulist, DevState *st, bool bitmaps) {
     constexpr int WPB = NARROW_SYM_WPB;
     constexpr int RPW = 32 / G, NR = WPB * RPW, QPL = NARROW_W / 4 / G;
     constexpr int P = G >= 8 ? 1 : 8 / G;
     __shared__ __align__(16) unsigned tab_all[NR * NARROW_TAB_STRIDE];
     __shared__ unsigned long long hist[NBINS];
     __shared__ unsigned long long fsum, alen_max;
+    __shared__ int marks[2];   // rows without a mark (sym_mark), with one
+    if (threadIdx.x < 2) marks[threadIdx.x] = 0;
     if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) { fsum = 0; alen_max = 0; }
     __syncthreads();
@@ -264,9 +266,16 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
             } else {
                 const long long keys = cp < (long long)nwords_b ? cp : (long long)nwords_b;
                 b = sym_bin(keys, cp);
+                if (bitmaps) {
+                    if (rowbad) b = BIN_EMPTY;
+                    const int mark = b == BIN_EMPTY ? 0 : sym_mark(cp, hi - lo + 1);
+                    crp[i + 1] = mark;
+                    if (b != BIN_EMPTY) marks[mark != 0] = 1;
+                } else {
+                    if (b == BIN_EMPTY) crp[i + 1] = 0;
+                    if (b == BIN_HUGE) crp[i + 1] = -1;
+                }
                 bins[i] = (uint8_t)b;
-                if (b == BIN_EMPTY) crp[i + 1] = 0;
-                if (b == BIN_HUGE) crp[i + 1] = -1;
                 nlo[i] = -1;
             }
         }
@@ -282,6 +291,8 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
     if (lane == 0 && wl) atomicMax(&alen_max, (unsigned long long)wl);
     __syncthreads();
     if (threadIdx.x == 0 && fsum) atomicAdd((unsigned long long *)&st->flops_total, fsum);
+    if (threadIdx.x == 0 && marks[0]) *(volatile int *)&st->sym_first = 1;
+    if (threadIdx.x == 0 && marks[1]) *(volatile int *)&st->sym_marked = 1;
     if (threadIdx.x == 0 && alen_max && alen_max > (unsigned long long)*(volatile long long *)&st->max_alen)
         atomicMax((unsigned long long *)&st->max_alen, alen_max);
     if (threadIdx.x < NBINS && hist[threadIdx.x]) {
@@ -294,7 +305,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
 template <int G>
 static int run_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
                           const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
-                          uint8_t *nwords, uint2 *ulist, DevState *st, Ctx &c) {
+                          uint8_t *nwords, uint2 *ulist, DevState *st, bool bitmaps, Ctx &c) {
     constexpr int NT = NARROW_SYM_WPB * 32, NR = NARROW_SYM_WPB * (32 / G);
     int64_t blocks = (A.nrows + NR - 1) / NR;
     const int64_t cap = resident_blocks(k_sym_narrow<G>, NT, c.nsm);
@@ -302,7 +313,7 @@ static int run_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *
     const int64_t nwb = (B.ncols + 31) / 32;
     c.begin("symbolic.narrow", A.nrows);
     k_sym_narrow<G><<<(unsigned)blocks, NT, 0, c.s>>>(A.nrows, B.nrows, nwb, A.row_ptr, A.col_idx, desc, bmm,
-                                                      pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st);
+                                                      pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, bitmaps);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
@@ -310,13 +321,13 @@ static int run_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *
 
 int launch_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
                       const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
-                      uint8_t *nwords, uint2 *ulist, DevState *st, int G, Ctx &c) {
+                      uint8_t *nwords, uint2 *ulist, DevState *st, bool bitmaps, int G, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     switch (G) {
-        case 4: return run_sym_narrow<4>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
-        case 8: return run_sym_narrow<8>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
-        case 16: return run_sym_narrow<16>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
-        default: return run_sym_narrow<32>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, c);
+        case 4: return run_sym_narrow<4>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, bitmaps, c);
+        case 8: return run_sym_narrow<8>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, bitmaps, c);
+        case 16: return run_sym_narrow<16>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, bitmaps, c);
+        default: return run_sym_narrow<32>(A, B, desc, bmm, pairs, flops, bins, crp, rspan, nlo, nwords, ulist, st, bitmaps, c);
     }
 }
 

@@ -4,11 +4,15 @@
 // block to the OR of its masks, and the count is the sum of popcounts
 // (Section 2.1: compression turns union into bitwise operations).
 //
-// Rows are sized by an upper bound on their distinct blocks.  A first pass
-// takes every row with bound <= 4096 in row order with a 32-slot map per
-// row, G lanes sharing the row's stored a_ik; rows that do not fit are
-// marked and, with the rows whose bound exceeds 4096, handled by a second
-// pass from row lists.  In bins 2-5 a row whose column blocks span at most
+// When a bitmap of all column blocks of B fits shared memory (up to 1.7 M
+// columns), rows with at most 32 pairs take a 32-slot map, G lanes sharing the
+// row's stored a_ik, and the others a bitmap of their span, by a warp or a
+// block (k_sym_rows).
+//
+// With a wider B, rows are sized by an upper bound on their distinct blocks.
+// A first pass takes every row with bound <= 4096 in row order with the
+// 32-slot map; rows that do not fit are marked and, with the rows whose bound
+// exceeds 4096, handled by a second pass from row lists.  In bins 2-5 a row whose column blocks span at most
 // 2048 blocks takes a warp with a bitmap over its span (k_sym_span); wider
 // rows take a warp with a 128- or 512-slot map (bins 2, 3) or a block with
 // a 2048- or 8192-slot map (bins 4, 5).  Bin 6 takes a block with a dense
@@ -44,18 +48,41 @@ struct SymFirstLayout {
 // of the widest bin or narrow: the histogram of the analysis, complete
 // before this kernel starts on the same stream); the kernel then returns
 // at once instead of reading every row's bin.
-__device__ __forceinline__ bool first_pass_empty(const DevState *st) {
+// With bitmaps: the rows it left unmarked.
+__device__ __forceinline__ bool first_pass_empty(const DevState *st, bool bitmaps) {
+    if (bitmaps) return *(volatile const int *)&st->sym_first == 0;
     long long m = 0;
 #pragma unroll
     for (int b = 1; b < BIN_HUGE; b++) m += *(volatile const long long *)&st->sym_hist[b];
     return m == 0;
 }
 
+// The marked rows' lists: a warp takes 32 rows at a time and reserves their
+// places with one atomic per list.
+__device__ __forceinline__ void list_marked(int64_t n, const int64_t *__restrict__ crp, int32_t *__restrict__ rows,
+                                            DevState *st) {
+    if (*(volatile int *)&st->sym_marked == 0) return;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n;
+         i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + lane;
+        const int64_t m = i < n ? crp[i + 1] : 0;
+        const unsigned mw = __ballot_sync(0xffffffffu, m == SYM_MARK_WARP), mb = __ballot_sync(0xffffffffu, m == SYM_MARK_BLOCK);
+        long long at = 0;
+        if (lane == 0 && mw) at = (long long)atomicAdd(&st->sym_warp, (unsigned long long)__popc(mw));
+        if (lane == 1 && mb) at = (long long)atomicAdd(&st->sym_block, (unsigned long long)__popc(mb));
+        const long long aw = __shfl_sync(0xffffffffu, at, 0), ab = __shfl_sync(0xffffffffu, at, 1);
+        if (m == SYM_MARK_WARP) rows[aw + __popc(mw & below)] = (int32_t)i;
+        if (m == SYM_MARK_BLOCK) rows[n - 1 - (ab + __popc(mb & below))] = (int32_t)i;
+    }
+}
+
 template <int G>
 __global__ void __launch_bounds__(256) k_sym_first(
     int64_t n, const uint8_t *__restrict__ bins, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc,
-    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, DevState *st) {
+    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, DevState *st, bool bitmaps) {
     using Lay = SymFirstLayout<G>;
     constexpr int S = Lay::S, L = 5, RPW = 32 / G, WPB = 8, PER = S / G;
     constexpr int E = Lay::E, EL = E / G, NR = WPB * RPW;
@@ -70,11 +97,12 @@ __global__ void __launch_bounds__(256) k_sym_first(
     int *pre = reg + Lay::o_pre;
     const unsigned lmask = (G == 32) ? 0xffffffffu : ((1u << G) - 1);
     const int64_t stride = (int64_t)gridDim.x * WPB * RPW;
-    if (first_pass_empty(st)) return;
+    if (bitmaps) list_marked(n, crp, rows, st);
+    if (first_pass_empty(st, bitmaps)) return;
     for (int64_t base = ((int64_t)blockIdx.x * WPB + w) * RPW; base < n; base += stride) {
         const int64_t i = base + g;
         const int b = i < n ? bins[i] : 0;
-        const bool active = b != BIN_EMPTY && b != BIN_HUGE && b != BIN_NARROW;
+        const bool active = b != BIN_EMPTY && b != BIN_NARROW && (bitmaps ? crp[i + 1] >= 0 : b != BIN_HUGE);
         if (!__any_sync(0xffffffffu, active)) continue;   // rows done elsewhere
         const int64_t p0 = active ? arp[i] : 0;
         const int plen = active ? (int)(arp[i + 1] - p0) : 0;
@@ -170,7 +198,7 @@ template <int G>
 __global__ void __launch_bounds__(256) k_sym_first_strided(
     int64_t n, const uint8_t *__restrict__ bins, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc,
-    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, DevState *st) {
+    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, DevState *st, bool bitmaps) {
     using Lay = SymFirstLayout<G>;
     constexpr int S = Lay::S, L = 5, RPW = 32 / G, WPB = 8, PER = S / G;
     constexpr int E = Lay::E, EL = E / G, NR = WPB * RPW;
@@ -185,11 +213,12 @@ __global__ void __launch_bounds__(256) k_sym_first_strided(
     int *pre = reg + Lay::o_pre;
     const unsigned lmask = (G == 32) ? 0xffffffffu : ((1u << G) - 1);
     const int64_t stride = (int64_t)gridDim.x * WPB * RPW;
-    if (first_pass_empty(st)) return;
+    if (bitmaps) list_marked(n, crp, rows, st);
+    if (first_pass_empty(st, bitmaps)) return;
     for (int64_t base = ((int64_t)blockIdx.x * WPB + w) * RPW; base < n; base += stride) {
         const int64_t i = base + g;
         const int b = i < n ? bins[i] : 0;
-        const bool active = b != BIN_EMPTY && b != BIN_HUGE && b != BIN_NARROW;
+        const bool active = b != BIN_EMPTY && b != BIN_NARROW && (bitmaps ? crp[i + 1] >= 0 : b != BIN_HUGE);
         if (!__any_sync(0xffffffffu, active)) continue;   // rows done elsewhere
         const int64_t p0 = active ? arp[i] : 0;
         const int plen = active ? (int)(arp[i + 1] - p0) : 0;
@@ -491,7 +520,7 @@ __global__ void __launch_bounds__(BS) k_sym_bitmap(
 }
 
 constexpr int BITMAP_BS = 512;
-constexpr int64_t SMEM_BITMAP_WORDS = 53248;  // 208 KiB of shared memory
+constexpr int64_t SMEM_BITMAP_WORDS = SYM_BITMAP_WORDS;
 
 size_t symbolic_global_ws(int64_t ncols_b, int nsm) {
     int64_t nwords = (ncols_b + 31) / 32;
@@ -510,7 +539,7 @@ static int prep(K kern, size_t smem) {
 
 template <int G>
 static int run_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
-                     int64_t *crp, DevState *st, Ctx &c) {
+                     int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, Ctx &c) {
     constexpr int GPB = 256 / G;   // rows per block: 8 warps x 32/G rows
     int64_t blocks = (A.nrows + GPB - 1) / GPB;
     // one resident wave striding over the rows: when the analysis left this
@@ -522,24 +551,215 @@ static int run_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc,
     c.begin("symbolic.first", A.nrows);
     if (G <= 8)
         k_sym_first_strided<G><<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, bins, A.row_ptr, A.col_idx, desc,
-                                                                  pairs, crp, st);
+                                                                  pairs, crp, rows, st, bitmaps);
     else
         k_sym_first<G><<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, bins, A.row_ptr, A.col_idx, desc,
-                                                       pairs, crp, st);
+                                                       pairs, crp, rows, st, bitmaps);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
-int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc,
-                          const int2 *pairs, int64_t *crp, DevState *st, int G, Ctx &c) {
+int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
+                          int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, int G, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     switch (G) {
-        case 4: return run_first<4>(A, bins, desc, pairs, crp, st, c);
-        case 8: return run_first<8>(A, bins, desc, pairs, crp, st, c);
-        case 16: return run_first<16>(A, bins, desc, pairs, crp, st, c);
-        default: return run_first<32>(A, bins, desc, pairs, crp, st, c);
+        case 4: return run_first<4>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
+        case 8: return run_first<8>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
+        case 16: return run_first<16>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
+        default: return run_first<32>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
     }
+}
+
+// ---------------------------------------------------------------- marked rows
+// Column-set union of a row as a bitwise OR of compressed pairs into a bitmap
+// of its span (Section 2.1), by a warp (NT = 32) or a block of NT threads per
+// row.  The row's pairs are dealt out flat, 32 consecutive ones a step, as the
+// products are in rank.cu: the entries of A are staged with the prefix sums of
+// pairs(B_k), the entries that start within a step set a bit each, and a
+// pair's entry is the number of bits up to its lane; BM_U steps' loads are in
+// flight together.  Then the bitmap is counted and cleared 16 bytes at a time.
+// What bounds it: instruction issue and, in rows of a few hundred pairs, the
+// chain of loads A -> descriptors -> pairs.  Measured (one GB300, symbolic
+// second pass and the first pass whose rows mostly failed it, before -> now):
+// batch of 64 products of uniform rows (921,066 rows, 294 M products) 2.9 ->
+// 1.0 ms; A*A of an R-MAT graph, scale 17 8.8 -> 3.0 ms (block hash maps of
+// 8192 slots before), scale 13 1.2 -> 0.12 ms (a warp walked rows of up to
+// half a million pairs); 41,472 rows of 5,000 pairs 0.78 -> 0.35 ms.  The rows
+// are listed and counted without a list length on the host, so the call waits
+// for the device once instead of twice.
+constexpr int BM_U = 4, BM_WPB = 8;
+
+struct BitmapP {
+    const int64_t *arp; const int32_t *acol;
+    const int4 *desc; const int2 *pairs; const int2 *rspan;
+    const int32_t *rows;
+    int64_t n;
+    int64_t *crp;
+    int bw;   // bitmap words (a multiple of 4)
+};
+
+template <int NT>
+struct BitmapSmem {   // words per row in flight: bitmap, starts of the entries (8 bytes each), their first pairs
+    static constexpr int E = NT, extra = 2 * E + E + 40;
+    static size_t bytes(int bw, int rows) { return (size_t)rows * (size_t)(bw + extra) * 4; }
+};
+
+template <int NT>
+__global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(BitmapP a, DevState *st) {
+    constexpr bool WARP = NT == 32;
+    constexpr int NW = NT / 32;
+    extern __shared__ __align__(16) unsigned bm_smem[];
+    __shared__ int wsum[NW], wcnt[NW];
+    __shared__ long long row_s;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tid = WARP ? lane : (int)threadIdx.x, w = WARP ? 0 : wid;
+    const unsigned below = (1u << lane) - 1u;
+    unsigned *bits = bm_smem + (WARP ? (size_t)wid * (size_t)(a.bw + BitmapSmem<NT>::extra) : 0);
+    long long *eq = (long long *)(bits + a.bw);   // start of B_k's pairs minus the entry's first pair
+    int *pre = (int *)(eq + NT);                   // first pair of every entry
+    auto sync = [] {
+        if (WARP) __syncwarp();
+        else __syncthreads();
+    };
+    const int64_t count = (int64_t) * (volatile unsigned long long *)(WARP ? &st->sym_warp : &st->sym_block);
+    if (count == 0) return;
+    for (int x = tid; x < a.bw / 4; x += NT) ((uint4 *)bits)[x] = make_uint4(0u, 0u, 0u, 0u);
+    int64_t t = WARP ? (int64_t)blockIdx.x * BM_WPB + wid : 0;
+    while (true) {
+        if (!WARP) {   // rows of very different work: handed out one at a time
+            if (tid == 0) row_s = (long long)atomicAdd(&st->next_row, 1ull);
+            __syncthreads();
+            t = row_s;
+        }
+        if (t >= count) break;
+        const int i = WARP ? a.rows[t] : a.rows[a.n - 1 - t];
+        const int2 sp = a.rspan[i];
+        const int lo = sp.x, nw = sp.y;
+        const int64_t p0 = a.arp[i];
+        const int64_t plen = a.arp[i + 1] - p0;
+        sync();
+        for (int64_t pb = 0; pb < plen; pb += NT) {
+            int len = 0;
+            long long q0 = 0;
+            if (pb + tid < plen) {
+                const int4 d = a.desc[a.acol[p0 + pb + tid]];
+                len = d.w;
+                q0 = desc_start(d);
+            }
+            int incl = len;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += y;
+            }
+            const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+            int base = 0, cb = 0, total, ne;
+            if (WARP) {
+                total = __shfl_sync(0xffffffffu, incl, 31);
+                ne = __popc(some);
+            } else {
+                if (lane == 31) wsum[w] = incl;
+                if (lane == 0) wcnt[w] = __popc(some);
+                __syncthreads();
+                const int nwu = (int)min((int64_t)NW, (plen - pb + 31) >> 5);
+                const int s = lane < nwu ? wsum[lane] : 0, c = lane < nwu ? wcnt[lane] : 0;
+                total = __reduce_add_sync(0xffffffffu, s);
+                ne = __reduce_add_sync(0xffffffffu, c);
+                base = __reduce_add_sync(0xffffffffu, lane < w ? s : 0);
+                cb = __reduce_add_sync(0xffffffffu, lane < w ? c : 0);
+            }
+            if (len > 0) {
+                const int pos = cb + __popc(some & below), first = base + incl - len;
+                pre[pos] = first;
+                eq[pos] = q0 - first;
+            }
+            for (int x = tid; x < 33; x += NT) pre[ne + x] = INT_MAX;   // a step looks 32 entries ahead
+            sync();
+            const int nch = (total + 31) >> 5, pw = (nch + NW - 1) / NW;
+            int tc = w * pw * 32;
+            const int tend = min(total, tc + pw * 32);
+            int e0 = -1;
+            if (tc < tend)
+                for (int x = 0; x < ne; x += 32) {
+                    const unsigned m = __ballot_sync(0xffffffffu, x + lane < ne && pre[x + lane] <= tc);
+                    e0 += __popc(m);
+                    if (m != 0xffffffffu) break;
+                }
+            for (; tc < tend; tc += 32 * BM_U) {
+                int2 pr[BM_U];
+#pragma unroll
+                for (int u = 0; u < BM_U; u++) {
+                    const int tu = tc + 32 * u;
+                    pr[u] = make_int2(lo, 0);
+                    if (tu >= tend) continue;   // uniform in the warp
+                    const int b = pre[e0 + 1 + lane] - tu;
+                    const unsigned m = __reduce_or_sync(0xffffffffu, b < 32 ? 1u << b : 0u);
+                    const int e = e0 + __popc(m & (2u * below + 1u));
+                    e0 += __popc(__ballot_sync(0xffffffffu, b <= 32));
+                    if (tu + lane < total) pr[u] = a.pairs[eq[e] + (tu + lane)];
+                }
+#pragma unroll
+                for (int u = 0; u < BM_U; u++) {
+                    const unsigned wd = (unsigned)(pr[u].x - lo);
+                    if (pr[u].y != 0 && wd < (unsigned)nw) atomicOr(&bits[wd], (unsigned)pr[u].y);
+                }
+            }
+            sync();
+        }
+        int c = 0;
+        for (int x = tid * 4; x < nw; x += NT * 4) {
+            const uint4 v = *(const uint4 *)&bits[x];
+            c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+            *(uint4 *)&bits[x] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (WARP) {
+            if (lane == 0) a.crp[i + 1] = c;
+            t += (int64_t)gridDim.x * BM_WPB;
+        } else {
+            if (lane == 0) wsum[w] = c;
+            __syncthreads();
+            if (tid == 0) {
+                long long s = 0;
+                for (int j = 0; j < NW; j++) s += wsum[j];
+                a.crp[i + 1] = s;
+            }
+        }
+        sync();
+    }
+}
+
+template <int NT>
+static int run_bitmap(const BitmapP &p, DevState *st, const char *label, Ctx &c) {
+    const int threads = NT == 32 ? BM_WPB * 32 : NT;
+    const size_t smem = BitmapSmem<NT>::bytes(p.bw, NT == 32 ? BM_WPB : 1);
+    SG_CUDA(cudaFuncSetAttribute(k_sym_rows<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sym_rows<NT>, threads, smem));
+    if (per_sm < 1) {
+        set_error("symbolic: %zu bytes of shared memory for a bitmap", smem);
+        return SPGEMM_ERR_INTERNAL;
+    }
+    const int64_t blocks = std::min<int64_t>((p.n * NT + threads - 1) / threads, (int64_t)per_sm * c.nsm);
+    c.begin(label, p.n);
+    k_sym_rows<NT><<<(unsigned)blocks, threads, smem, c.s>>>(p, st);
+    c.end();
+    SG_CUDA(cudaGetLastError());
+    return SPGEMM_OK;
+}
+
+int launch_symbolic_bitmaps(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *pairs,
+                            const int2 *rspan, const int32_t *rows, int64_t *crp, DevState *st, Ctx &c) {
+    if (A.nrows == 0) return SPGEMM_OK;
+    const int nwords = (int)((B.ncols + 31) / 32);
+    BitmapP p{A.row_ptr, A.col_idx, desc, pairs, rspan, rows, A.nrows, crp, (std::min(nwords, SYM_WARP_WORDS) + 3) & ~3};
+    SG_TRY(run_bitmap<32>(p, st, "symbolic.warp_rows", c));
+    p.bw = (nwords + 3) & ~3;
+    // a block's threads by the blocks that fit an SM beside its bitmap
+    if (nwords <= 8192) return run_bitmap<256>(p, st, "symbolic.block_rows", c);
+    if (nwords <= 24576) return run_bitmap<512>(p, st, "symbolic.block_rows", c);
+    return run_bitmap<1024>(p, st, "symbolic.block_rows", c);
 }
 
 static const char *SYM_LABEL[NBINS] = {"", "", "symbolic.bin2", "symbolic.bin3",

@@ -230,6 +230,7 @@ size_t triangles_ws(int64_t n, int64_t nnz, int nsm) {
     add((size_t)nnz * 8);            // pairs
     add((size_t)n * 4);              // ccnt
     add((size_t)n * 16);             // desc
+    add((size_t)n * 4);              // long rows of L
     add((size_t)n * 4 * 2);          // light and heavy lists
     add(64);                         // counters
     add(scan_tmp_bytes(n));
@@ -252,6 +253,7 @@ int launch_triangles(const spgemm_csr &A, void *ws, int64_t *perm_out, int64_t *
     int2 *pairs = (int2 *)take((size_t)nnz * 8);
     int32_t *ccnt = (int32_t *)take((size_t)n * 4);
     int4 *desc = (int4 *)take((size_t)n * 16);
+    int32_t *longs = (int32_t *)take((size_t)n * 4);
     int32_t *light = (int32_t *)take((size_t)n * 4);
     int32_t *heavy = (int32_t *)take((size_t)n * 4);
     unsigned long long *cnt = (unsigned long long *)take(64);
@@ -281,7 +283,7 @@ int launch_triangles(const spgemm_csr &A, void *ws, int64_t *perm_out, int64_t *
     spgemm_csr L{n, n, nnz, lrp, lcol, nullptr};
     // nnz(L) is on the device; the compression reads the offsets, so the
     // descriptor's entry count only bounds the arrays
-    SG_TRY(launch_compress(L, pairs, ccnt, nullptr, desc, nullptr, err, c));
+    SG_TRY(launch_compress(L, pairs, ccnt, nullptr, desc, nullptr, err, (int *)(cnt + 4), longs, c));
     c.begin("triangles.bins", n);
     k_tri_bins<<<gw, 256, 0, c.s>>>(n, lrp, lcol, desc, light, heavy, cnt);
     c.end();
