@@ -133,11 +133,14 @@ SPGEMM_API int spgemm_numeric(spgemm_handle handle, int dtype, const spgemm_csr 
  *    most 32 outputs and 8192 products) multiplied over a dense window of
  *    the compressed column sets (Section 2.1) instead of hash maps; the
  *    window gives every column its rank, so those rows need no probe and no
- *    sort.  They accumulate in native precision whatever
+ *    sort.  Rows of up to 256 outputs in at most 32 blocks take the same
+ *    window in FP32 and native FP64 (counted in their bin by outputs).  Rows
+ *    of at most 32 outputs accumulate in native precision whatever
  *    SPGEMM_OPT_F64_NATIVE says.  Takes effect at the next spgemm_symbolic.
  *  SPGEMM_OPT_LANES_NARROW_SYMBOLIC (0, 4, 8, 16, 32) and
  *    SPGEMM_OPT_LANES_NARROW_NUMERIC (0, 4, 8, 16): lanes per row of the
- *    narrow-row kernels (0 = from the mean length of the rows of A).
+ *    narrow-row kernels (0 = from the mean length of the rows of A or B, and
+ *    more when the rows are too few to fill the device).
  *  SPGEMM_OPT_CHUNK_BUFFERS (2 or 3, default 2): buffers per streamed
  *    operand in spgemm_chunked_numeric / spgemm_chunked: 2 = double
  *    buffering (one part is copied while the other is multiplied), 3 =

@@ -507,6 +507,7 @@ struct ScanBins {
     uint8_t *bins, *cls;
     const int2 *rspan;
     const int32_t *nlo;   // may be null
+    const uint8_t *nwords;
     DevState *st;
     bool dense_ok;
 };
@@ -566,10 +567,11 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
             if (bin != BIN_EMPTY && b.nlo && b.nlo[i] >= 0 && c <= NARROW_NMAX && f <= NARROW_FLOPS) bin = BIN_NARROW;
             b.bins[i] = (uint8_t)bin;
             if (bin == BIN_HUGE) atomicMax((unsigned long long *)&b.st->max_row_nnz, (unsigned long long)c);
-            int k = CLS_NONE;
+            int k = bin == BIN_NARROW ? CLS_NARROW : CLS_NONE;
             if (bin >= 2 && bin <= BIN_HUGE) {
                 const int words = b.rspan[i].y;
-                k = num_cls(bin, c, f, words, b.dense_ok && b.st->b_unsorted == 0);
+                const bool listed = b.nlo && b.nlo[i] >= 0 && b.nwords[i] <= NARROW_NMAX;
+                k = num_cls(bin, c, f, words, listed, b.dense_ok && b.st->b_unsorted == 0);
                 atomicAdd(&ccnt[k], 1);
                 if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
                 if (words > cwords[k]) atomicMax(&cwords[k], words);
@@ -581,6 +583,7 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
     __syncthreads();
     const int t = threadIdx.x;
     if (t < NBINS && hist[t]) atomicAdd((unsigned long long *)&b.st->bin_count[1][t], hist[t]);
+    if (t == BIN_NARROW && hist[t]) atomicAdd((unsigned long long *)&b.st->cls_count[CLS_NARROW], hist[t]);
     if (t < NCLS && ccnt[t]) {
         atomicAdd((unsigned long long *)&b.st->cls_count[t], (unsigned long long)ccnt[t]);
         if (cnnz[t] > *(volatile int *)&b.st->cls_nnz[t]) atomicMax(&b.st->cls_nnz[t], cnnz[t]);
@@ -622,9 +625,10 @@ int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &
 }
 
 int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                        const int2 *rspan, const int32_t *nlo, DevState *st, bool dense_ok, Ctx &c) {
+                        const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
+                        Ctx &c) {
     if (n == 0) return launch_scan_counts(crp, n, &st->nnz, tmp, c);
-    return run_scan<true>(crp, n, &st->nnz, tmp, ScanBins{flops, bins, cls, rspan, nlo, st, dense_ok}, c);
+    return run_scan<true>(crp, n, &st->nnz, tmp, ScanBins{flops, bins, cls, rspan, nlo, nwords, st, dense_ok}, c);
 }
 
 }  // namespace sg

@@ -301,6 +301,14 @@ static int lanes_for(double x, int lo = 8) {
     return g;
 }
 
+// Lanes per row, doubled while all rows fit less than one wave of warps (32
+// an SM) and a row has work for them: a row's chain of steps is then the
+// whole kernel.
+static int widen(int lanes, int64_t rows, double work, int nsm) {
+    while (lanes < 32 && rows * lanes < (int64_t)nsm * 32 * 32 && work > 2.0 * lanes) lanes *= 2;
+    return lanes;
+}
+
 // Workspace offsets.  [bins | classes | rows | B descriptors | B block ranges |
 // column-block span of every row | first window block of every row | window
 // words of the narrow rows (count, list)] persist from symbolic to numeric; after
@@ -385,7 +393,8 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
             // analysis and the narrow rows' counts in one pass; the first
             // pass below takes the other rows
             // lanes per row: rows of A longer than 32 entries take 8
-            const int gn = h->g_narrow_sym ? h->g_narrow_sym : (mean_alen <= 32.0 ? 4 : 8);
+            int gn = h->g_narrow_sym ? h->g_narrow_sym : (mean_alen <= 32.0 ? 4 : 8);
+            if (!h->g_narrow_sym) gn = widen(gn, n, mean_alen, h->nsm);
             SG_TRY(launch_sym_narrow(*A, *B, desc, minmax, pairs, flops, bins, C_row_ptr, rspan, nlo, nwords,
                                      ulist, h->dstate, bitmaps, gn, c));
         } else {
@@ -414,7 +423,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         const size_t dense_bytes = dense_ws(B->nrows, B->ncols);
         const bool dense_ok = dense_bytes <= (size_t)B->nnz * 12 + ((size_t)64 << 20);
         SG_TRY(launch_scan_binning(C_row_ptr, n, w + L.tmp, flops, bins, cls, rspan, h->narrow ? nlo : nullptr,
-                                   h->dstate, dense_ok, c));
+                                   nwords, h->dstate, dense_ok, c));
         SG_TRY(fetch_state(h, s));
         SG_TRY(device_errors(h->hstate->err));
         *nnz_C = h->hstate->nnz;
@@ -488,9 +497,12 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
     tune.G = h->g_numeric ? h->g_numeric : lanes_for(h->mean_flops / 80.0);
     tune.small_cap = h->small_cap;
     tune.slot_factor = h->slot_factor;
-    const int first_list = tune.small_cap >= 32 ? CLS_RANK_S : CLS_B2;
+    const int first_list = tune.small_cap >= 32 ? CLS_B2 + 1 : CLS_B2;
+    // narrow rows are listed when other rows lie between them: a warp takes
+    // several consecutive ones, and the others would leave its lanes idle
     long long listed = 0;
-    for (int k = first_list; k < NCLS; k++) listed += h->cls.count[k];
+    for (int k = first_list; k < NCLS; k++)
+        if (k != CLS_NARROW || h->cls.count[k] < n) listed += h->cls.count[k];
     if (listed > 0 && h->num_lists != first_list) {
         SG_TRY(launch_scatter_cls(n, cls, rows, h->dstate, first_list, c));
         h->num_lists = first_list;
@@ -499,11 +511,19 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
         // lanes per row: a chunk of G consecutive entries of a row of B per
         // step, so G follows the mean length of the rows of B
         const double mean_blen = (double)B->nnz / (double)(B->nrows > 0 ? B->nrows : 1);
-        const int gn = h->g_narrow_num ? h->g_narrow_num : (mean_blen <= 8.0 ? 4 : 8);
-        SG_TRY(launch_num_narrow(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, bins, &h->dstate->err, gn, c));
+        int gn = h->g_narrow_num ? h->g_narrow_num : (mean_blen <= 8.0 ? 4 : 8);
+        const int64_t count = h->cls.count[CLS_NARROW];
+        const int32_t *list = count < n ? rows + (listed - count) : nullptr;
+        if (!h->g_narrow_num) gn = widen(gn, count, h->mean_flops, h->nsm);
+        if (gn == 32) {
+            const bool block = count < (int64_t)h->nsm * 8 && h->mean_flops >= 512.0;
+            SG_TRY(launch_num_window(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, list, count, block, NARROW_NMAX,
+                                     "numeric.narrow", &h->dstate->err, c));
+        } else
+        SG_TRY(launch_num_narrow(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, list, count, &h->dstate->err, gn, c));
     }
     return launch_numeric(dtype, h->f64_native, *A, *B, *C, bins, bdesc, rspan, rows, h->num_counts,
-                          h->cls, h->dstate, bsplit, gws, h->num_gws, h->max_row_nnz, tune, h->b_sorted,
+                          h->cls, NarrowInfo{nlo, nwords, ulist}, h->dstate, bsplit, gws, h->num_gws, h->max_row_nnz, tune, h->b_sorted,
                           h->max_alen, c);
 }
 

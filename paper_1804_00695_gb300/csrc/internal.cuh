@@ -121,6 +121,10 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 // its outputs, its column span and its products.  The lists of the numeric
 // phase are in class order.
 //   CLS_B2      bin 2 (a list only when the small-row kernel stops at 16)
+//   CLS_WINDOW_W, CLS_WINDOW_B  narrow rows of 33 to WINDOW_NNZ outputs whose
+//               word list the symbolic phase left whole: a warp, or from
+//               WINDOW_FLOPS products on a block
+//   CLS_NARROW  BIN_NARROW (a list only when other rows lie between them)
 //   CLS_RANK_S  at most RANK_S_NNZ outputs over at most RANK_S_WORDS blocks
 //   CLS_RANK_M4, CLS_RANK_M5  wider spans up to RANK_M_WORDS blocks: rows
 //               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
@@ -134,8 +138,8 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 // two would not fit.  Below them the rank accumulators measured 2.6-5x
 // faster than the maps and windows (rank.cu has the figures).
 enum NumCls {
-    CLS_NONE = 0, CLS_B2, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
-    CLS_BLOCK, CLS_DENSE, CLS_HUGE, NCLS
+    CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
+    CLS_BLOCK, CLS_DENSE, CLS_HUGE, CLS_NARROW, NCLS
 };
 constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
 constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit 32 bits)
@@ -145,9 +149,14 @@ constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit
 // registers: A*A of R-MAT graphs, FP64, scale 16 with 12 edges a vertex 11.9
 // ms (one per 4 columns 12.4), scale 15 with 5 2.91 (2.94, one per 2 3.02).
 constexpr long long DENSE_FLOPS = 6144;
-__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words, bool dense_ok) {
-    if (bin < 2 || bin > BIN_HUGE) return CLS_NONE;
+constexpr int WINDOW_NNZ = 256;
+constexpr long long WINDOW_FLOPS = 4096;
+// listed: the row is narrow and its words are all in its list.
+__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words, bool listed, bool dense_ok) {
+    if (bin < 2) return CLS_NONE;
+    if (bin == 7) return CLS_NARROW;
     if (bin == 2) return CLS_B2;
+    if (listed && nnz <= WINDOW_NNZ) return flops < WINDOW_FLOPS ? CLS_WINDOW_W : CLS_WINDOW_B;
     if (dense_ok && bin >= 5 && words > 0 && flops < (1LL << 31) &&
         (nnz > RANK_M_NNZ || (flops > DENSE_FLOPS && flops * 8 >= (long long)words * 32)))
         return CLS_DENSE;
@@ -285,7 +294,8 @@ int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, co
 // narrow numeric kernel get BIN_NARROW.  cls[i]: the row's class (num_cls);
 // rows, largest row and span per class in st.
 int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                        const int2 *rspan, const int32_t *nlo, DevState *st, bool dense_ok, Ctx &c);
+                        const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
+                        Ctx &c);
 // Row lists of the symbolic second pass by bin: rows[offset(b) + t], offsets
 // from st->bin_count[0].
 int launch_scatter_bins(int64_t n, const uint8_t *bins, const int64_t *crp, int32_t *rows, DevState *st, Ctx &c);
@@ -305,11 +315,19 @@ int launch_row_flops(const spgemm_csr &A, const spgemm_csr &B, int64_t *flops, i
 int launch_sym_narrow(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *bmm,
                       const int2 *pairs, int64_t *flops, uint8_t *bins, int64_t *crp, int2 *rspan, int32_t *nlo,
                       uint8_t *nwords, uint2 *ulist, DevState *st, bool bitmaps, int G, Ctx &c);
-// Numeric phase of the rows with bins[i] == BIN_NARROW (F32 or native F64),
+// Numeric phase of the rows of BIN_NARROW (F32 or native F64),
 // from the word lists of the symbolic phase; G lanes per row (4, 8 or 16).
+// rows: their list (count), or null: every row of A is one.
 int launch_num_narrow(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const uint8_t *bins, int *err,
-                      int G, Ctx &c);
+                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const int32_t *rows,
+                      int64_t count, int *err, int G, Ctx &c);
+
+// Numeric phase of the listed rows of CLS_WINDOW_W (block false) or
+// CLS_WINDOW_B, FP32 or native FP64; max_nnz: the largest row.  Also the rows
+// of BIN_NARROW when they are few (rows null: every row of A).
+int launch_num_window(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
+                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const int32_t *rows, int64_t count,
+                      bool block, int max_nnz, const char *label, int *err, Ctx &c);
 
 // symbolic.cu
 // First pass over all rows with a 32-slot map and G lanes per row (rows of
@@ -347,10 +365,16 @@ struct ClsInfo {
     long long count[NCLS] = {0};
     int nnz[NCLS] = {0}, words[NCLS] = {0};
 };
+// What the symbolic phase left of the narrow rows (all rows; device).
+struct NarrowInfo {
+    const int32_t *nlo;
+    const uint8_t *nwords;
+    const uint2 *ulist;
+};
 int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm_csr &B,
                    spgemm_csr &C, const uint8_t *bins, const int4 *bdesc, const int2 *rspan,
                    const int32_t *rows,
-                   const long long *counts, const ClsInfo &cls, DevState *st, float2 *bsplit, void *gws,
+                   const long long *counts, const ClsInfo &cls, const NarrowInfo &nar, DevState *st, float2 *bsplit, void *gws,
                    size_t gws_bytes, int64_t max_row_nnz, const NumTune &tune, bool b_sorted,
                    int64_t max_alen, Ctx &c);
 size_t numeric_global_ws(int64_t max_row_nnz, int64_t ncols_b, int nsm, int dtype);

@@ -336,8 +336,8 @@ struct NarrowP {
     const int64_t *arp; const int32_t *acol; const void *aval;
     const int32_t *bcol; const void *bval;
     const int64_t *crp; int32_t *ccol; void *cval;
-    const int4 *bdesc; const int32_t *nlo; const uint8_t *nwords; const uint2 *ulist; const uint8_t *bins;
-    int64_t n, nrows_b;
+    const int4 *bdesc; const int32_t *nlo; const uint8_t *nwords; const uint2 *ulist; const int32_t *rows;
+    int64_t n, nrows_b;   // n: rows of the list, or of A
 };
 
 // A staged entry of the product pass: the start of B_k in B (as 32-bit
@@ -397,7 +397,9 @@ constexpr int NARROW_U = 3;
 constexpr int NARROW_MINB4 = 6;
 
 // G lanes per row, 32/G rows per warp, WPB warps per block, batches of E
-// stored entries; rows with bins[i] == BIN_NARROW, in row order.  The row's
+// stored entries; LIST: the rows of a list, else all rows.  (In elasticity's
+// A*P 41% of the rows have more than 32 outputs; taken in row order they left
+// two of five row slots idle.)  The row's
 // word list (left by the symbolic phase) is scattered into the window table
 // and kept in registers for the output (and to clear the table again after
 // the row: the table is cleared once at the start and holds only the
@@ -407,7 +409,7 @@ constexpr int NARROW_MINB4 = 6;
 // first entry of B and skips its update (predicated), and so does a column
 // missing from the row's window (flagged).  IDX32: B has fewer than 2^31
 // entries (32-bit offsets).
-template <int G, int WPB, int E, typename V, bool IDX32>
+template <int G, int WPB, int E, typename V, bool IDX32, bool LIST>
 __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_narrow(NarrowP a, int *err) {
     using S = NarrowSmem<G, WPB, E, V, IDX32>;
     constexpr int RPW = 32 / G, NR = WPB * RPW, U = NARROW_U, EL = E / G;
@@ -434,9 +436,8 @@ __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_nar
     int flag = 0;
     const int64_t stride = (int64_t)gridDim.x * NR;
     for (int64_t rb = (int64_t)blockIdx.x * NR + w * RPW; rb < a.n; rb += stride) {
-        const int64_t i = rb + g;
-        bool act = i < a.n && a.bins[i] == BIN_NARROW;
-        if (!__any_sync(0xffffffffu, act)) continue;
+        bool act = rb + g < a.n;
+        const int64_t i = LIST ? (act ? a.rows[rb + g] : 0) : rb + g;
         const int lo = act ? a.nlo[i] : 0;
         const int64_t p0 = act ? a.arp[i] : 0;
         int plen = act ? (int)(a.arp[i + 1] - p0) : 0;
@@ -574,38 +575,258 @@ __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_nar
     if (flag) atomicOr(err, flag);
 }
 
-template <int G, int E, typename V, bool IDX32>
+template <int G, int E, typename V, bool IDX32, bool LIST>
 static int run_num_narrow(const NarrowP &p, int *err, Ctx &c) {
     constexpr int WPB = 4, NR = WPB * (32 / G);
     int64_t blocks = (p.n + NR - 1) / NR;
-    const int64_t cap = resident_blocks(k_num_narrow<G, WPB, E, V, IDX32>, WPB * 32, c.nsm);
+    const int64_t cap = resident_blocks(k_num_narrow<G, WPB, E, V, IDX32, LIST>, WPB * 32, c.nsm);
     blocks = blocks < cap ? blocks : cap;
     c.begin("numeric.narrow", p.n);
-    k_num_narrow<G, WPB, E, V, IDX32><<<(unsigned)blocks, WPB * 32, 0, c.s>>>(p, err);
+    k_num_narrow<G, WPB, E, V, IDX32, LIST><<<(unsigned)blocks, WPB * 32, 0, c.s>>>(p, err);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
-template <typename V, bool IDX32>
+template <typename V, bool IDX32, bool LIST>
 static int run_num_narrow_g(const NarrowP &p, int *err, int G, Ctx &c) {
     switch (G) {
-        case 4: return run_num_narrow<4, 16, V, IDX32>(p, err, c);
-        case 8: return run_num_narrow<8, 32, V, IDX32>(p, err, c);
-        default: return run_num_narrow<16, 32, V, IDX32>(p, err, c);
+        case 4: return run_num_narrow<4, 16, V, IDX32, LIST>(p, err, c);
+        case 8: return run_num_narrow<8, 32, V, IDX32, LIST>(p, err, c);
+        default: return run_num_narrow<16, 32, V, IDX32, LIST>(p, err, c);
     }
 }
 
+template <typename V>
+static int run_num_narrow_v(const NarrowP &p, bool i32, int *err, int G, Ctx &c) {
+    if (p.rows) return i32 ? run_num_narrow_g<V, true, true>(p, err, G, c) : run_num_narrow_g<V, false, true>(p, err, G, c);
+    return i32 ? run_num_narrow_g<V, true, false>(p, err, G, c) : run_num_narrow_g<V, false, false>(p, err, G, c);
+}
+
 int launch_num_narrow(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const uint8_t *bins, int *err,
-                      int G, Ctx &c) {
-    if (A.nrows == 0) return SPGEMM_OK;
+                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const int32_t *rows,
+                      int64_t count, int *err, int G, Ctx &c) {
+    if (count == 0) return SPGEMM_OK;
     NarrowP p{A.row_ptr, A.col_idx, A.values, B.col_idx, B.values, C.row_ptr, C.col_idx, C.values,
-              bdesc, nlo, nwords, ulist, bins, A.nrows, B.nrows};
+              bdesc, nlo, nwords, ulist, rows, count, B.nrows};
     const bool i32 = B.nnz < ((int64_t)1 << 31);
-    if (dtype == SPGEMM_F32)
-        return i32 ? run_num_narrow_g<float, true>(p, err, G, c) : run_num_narrow_g<float, false>(p, err, G, c);
-    return i32 ? run_num_narrow_g<double, true>(p, err, G, c) : run_num_narrow_g<double, false>(p, err, G, c);
+    return dtype == SPGEMM_F32 ? run_num_narrow_v<float>(p, i32, err, G, c) : run_num_narrow_v<double>(p, i32, err, G, c);
+}
+
+// ---------------------------------------------------------------- wider narrow rows
+// Narrow rows of 33 to WINDOW_NNZ outputs (block operators: elasticity's
+// triple products): the same window table and ranks, WR warps per row.  A
+// row's entries are dealt out over subgroups of 16 lanes, each with an
+// accumulator of its own: within a subgroup the lanes hold entries of one row
+// of B, whose columns are distinct, so an update is a plain read-fma-write (one
+// FP64 operation, no atomic, no retry where thousands of products meet in a
+// few dozen slots).  The subgroups' sums are added when the row is written.
+//
+// What bounds it: the chain of loads and the shared-memory lookups of a step
+// (20-odd instructions for 32 products); the FP64 floor of the products is a
+// third of it.  Measured (one GB300, elasticity on 32^3, FP64): A*P and
+// R*(AP), 61,398 such rows, 1.61 -> 0.45 ms against the rank accumulators,
+// whose atomics retried on the few slots of a row and of which a row of
+// R*(AP) (12,000 products) had one block's share of a chip that 3,969 rows do
+// not fill.  The block variant from 4096 products on.  Rows of at most 32
+// outputs come here too when they fill less than a wave of warps at eight
+// lanes a row: R*(AP) of 45^3 (3375 rows) 0.09 -> 0.03 ms, and the 24 such
+// rows of elasticity's R*(AP) 0.15 -> 0.02 ms.
+constexpr int WIN_G = 16, WIN_U = 4;
+
+template <typename V, typename Q>
+struct WinEnt {
+    Q q;
+    int len;
+    V a;
+};
+
+struct WindowP {
+    const int64_t *arp; const int32_t *acol; const void *aval;
+    const int32_t *bcol; const void *bval;
+    const int64_t *crp; int32_t *ccol; void *cval;
+    const int4 *bdesc; const int32_t *nlo; const uint8_t *nwords; const uint2 *ulist;
+    const int32_t *rows;
+    int64_t count, nrows_b;
+    int stride;   // slots of an accumulator (odd: the subgroups' start on different banks)
+};
+
+template <typename V, typename Q, int WR>
+struct WindowSmem {   // per row in flight
+    static constexpr int E = WR == 1 ? 64 : WR * 32, NSG = WR * (32 / WIN_G);
+    static size_t bytes(int stride) {
+        return ((size_t)NSG * stride * sizeof(V) + 15) / 16 * 16 + (sizeof(WinEnt<V, Q>) * E + 15) / 16 * 16 + NARROW_W * 5;
+    }
+};
+
+template <typename V, typename Q, int WR>
+__global__ void __launch_bounds__(256) k_num_window_rows(WindowP a, size_t per_row, int *err) {
+    using S = WindowSmem<V, Q, WR>;
+    constexpr int NT = WR * 32, RPB = 8 / WR, NSG = S::NSG, E = S::E, U = WIN_U;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int ok_s;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int slot = WR == 1 ? wid : 0, tid = WR == 1 ? lane : (int)threadIdx.x;
+    const int sg = tid / WIN_G, gl = tid % WIN_G;
+    unsigned char *mine = smem_raw + (size_t)slot * per_row;
+    V *acc_all = (V *)mine;
+    V *acc = acc_all + sg * a.stride;
+    WinEnt<V, Q> *ent = (WinEnt<V, Q> *)(mine + ((size_t)NSG * a.stride * sizeof(V) + 15) / 16 * 16);
+    unsigned *tab = (unsigned *)((unsigned char *)ent + (sizeof(WinEnt<V, Q>) * E + 15) / 16 * 16);
+    unsigned char *base = (unsigned char *)(tab + NARROW_W);
+    const V *__restrict__ aval = (const V *)a.aval;
+    const V *__restrict__ bval = (const V *)a.bval;
+    const int32_t *__restrict__ bcol = a.bcol;
+    auto sync = [] {
+        if (WR == 1) __syncwarp();
+        else __syncthreads();
+    };
+    for (int x = tid; x < NARROW_W; x += NT) tab[x] = 0u;
+    sync();
+    int flag = 0;
+    for (int64_t t = (int64_t)blockIdx.x * RPB + slot; t < a.count; t += (int64_t)gridDim.x * RPB) {
+        const int i = a.rows ? a.rows[t] : (int)t;
+        const int lo = a.nlo[i], nw = a.nwords[i];
+        const int64_t p0 = a.arp[i], out = a.crp[i];
+        const int plen = (int)(a.arp[i + 1] - p0);
+        const int64_t nn64 = a.crp[i + 1] - out;
+        const int nn = (int)nn64;
+        uint2 lw = make_uint2(0u, 0u);
+        bool ok = lo >= 0 && nn64 <= a.stride && nw <= NARROW_NMAX;
+        if (WR == 1 || wid == 0) {
+            if (ok && lane < nw) lw = a.ulist[(int64_t)i * NARROW_NMAX + lane];
+            const int total = __reduce_add_sync(0xffffffffu, __popc(lw.y));
+            ok = ok && total == nn;
+            if (!ok) lw = make_uint2(0u, 0u);
+            if (lw.y) {
+                tab[lw.x & (NARROW_W - 1)] = lw.y;
+                base[lw.x & (NARROW_W - 1)] = (unsigned char)(lw.x >> 8);
+            }
+            if (WR > 1 && lane == 0) ok_s = ok;
+        }
+        for (int x = tid; x < NSG * a.stride; x += NT) acc_all[x] = V(0);
+        sync();
+        if (WR > 1) ok = ok_s;
+        if (!ok) flag |= DERR_COUNT;   // not the pattern of the symbolic phase
+        for (int pb = 0; ok && pb < plen; pb += E) {
+            const int nb = min(E, plen - pb);
+            for (int x = tid; x < nb; x += NT) {
+                const int k = a.acol[p0 + pb + x];
+                WinEnt<V, Q> en;
+                en.q = 0;
+                en.len = 0;
+                en.a = aval[p0 + pb + x];
+                if ((unsigned)k < (unsigned)a.nrows_b) {
+                    const int4 d = a.bdesc[k];
+                    en.q = (Q)desc_start(d);
+                    en.len = d.z;
+                } else {
+                    flag |= DERR_COL_RANGE;
+                }
+                ent[x] = en;
+            }
+            sync();
+            int e = sg, j = gl, clen = 0;
+            Q cq = 0;
+            V ca = V(0);
+            if (e < nb) {
+                cq = ent[e].q;
+                clen = ent[e].len;
+                ca = ent[e].a;
+            }
+            while (__any_sync(0xffffffffu, e < nb)) {
+                int c[U], rk[U];
+                V v[U], av[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const bool live = j < clen;
+                    rk[u] = live ? 0 : -1;
+                    c[u] = 0;
+                    v[u] = V(0);
+                    if (live) {
+                        c[u] = bcol[cq + j];
+                        v[u] = bval[cq + j];
+                    }
+                    av[u] = ca;
+                    j += WIN_G;
+                    if (j - gl >= clen && e < nb) {
+                        e += NSG;
+                        j = gl;
+                        clen = 0;
+                        if (e < nb) {
+                            cq = ent[e].q;
+                            clen = ent[e].len;
+                            ca = ent[e].a;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const unsigned wd = (unsigned)((c[u] >> 5) - lo) & (NARROW_W - 1);
+                    const unsigned m = tab[wd], sh = (unsigned)c[u] & 31u;
+                    const bool hit = (m >> sh) & 1u;
+                    if (rk[u] == 0 && !hit) flag |= DERR_COUNT;
+                    rk[u] = rk[u] == 0 && hit ? min((int)base[wd] + popc_below(m, sh), a.stride - 1) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (rk[u] >= 0) acc[rk[u]] = fma(av[u], v[u], acc[rk[u]]);
+                    __syncwarp();
+                }
+            }
+            sync();
+        }
+        if (ok)
+            for (int x = tid; x < nn; x += NT) {
+                V s = acc_all[x];
+#pragma unroll
+                for (int y = 1; y < NSG; y++) s += acc_all[y * a.stride + x];
+                ((V *)a.cval)[out + x] = s;
+            }
+        if (lw.y) {
+            unsigned m = lw.y;
+            int64_t at = out + (int)(lw.x >> 8);
+            const int wd = (int)(lw.x & (NARROW_W - 1));
+            for (; m; m &= m - 1u) a.ccol[at++] = (lo + wd) * 32 + __ffs(m) - 1;
+            tab[wd] = 0u;
+        }
+        sync();
+    }
+    if (flag) atomicOr(err, flag);
+}
+
+template <typename V, typename Q, int WR>
+static int run_window_rows(WindowP &p, int *err, const char *label, Ctx &c) {
+    const size_t per_row = (WindowSmem<V, Q, WR>::bytes(p.stride) + 15) / 16 * 16, smem = per_row * (8 / WR);
+    SG_CUDA(cudaFuncSetAttribute(k_num_window_rows<V, Q, WR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_num_window_rows<V, Q, WR>, 256, smem));
+    if (per_sm < 1) {
+        set_error("numeric: %zu bytes of shared memory for the window rows", smem);
+        return SPGEMM_ERR_INTERNAL;
+    }
+    const int64_t blocks = std::min<int64_t>((p.count * WR + 7) / 8, (int64_t)per_sm * c.nsm);
+    c.begin(label, p.count);
+    k_num_window_rows<V, Q, WR><<<(unsigned)blocks, 256, smem, c.s>>>(p, per_row, err);
+    c.end();
+    SG_CUDA(cudaGetLastError());
+    return SPGEMM_OK;
+}
+
+int launch_num_window(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
+                      const int32_t *nlo, const uint8_t *nwords, const uint2 *ulist, const int32_t *rows, int64_t count,
+                      bool block, int max_nnz, const char *label, int *err, Ctx &c) {
+    if (count <= 0) return SPGEMM_OK;
+    WindowP p{A.row_ptr, A.col_idx, A.values, B.col_idx, B.values, C.row_ptr, C.col_idx, C.values,
+              bdesc, nlo, nwords, ulist, rows, count, B.nrows, max_nnz | 1};
+    auto go = [&](auto v, auto q) -> int {
+        using V = decltype(v);
+        using Q = decltype(q);
+        return block ? run_window_rows<V, Q, 8>(p, err, label, c) : run_window_rows<V, Q, 1>(p, err, label, c);
+    };
+    const bool i32 = B.nnz < ((int64_t)1 << 31);
+    if (dtype == SPGEMM_F32) return i32 ? go(0.f, 0) : go(0.f, 0LL);
+    return i32 ? go(0.0, 0) : go(0.0, 0LL);
 }
 
 }  // namespace sg

@@ -1649,13 +1649,13 @@ static int run_warp_rank(const NumP &a, const int4 *bdesc, const int2 *rspan, co
 template <int MODE>
 static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const uint8_t *bins,
                    const int4 *bdesc, const int2 *rspan, const int32_t *rows, const long long *counts,
-                   const ClsInfo &cls, DevState *st, void *gws, size_t gws_bytes, int64_t max_row_nnz,
+                   const ClsInfo &cls, const NarrowInfo &nar, DevState *st, void *gws, size_t gws_bytes, int64_t max_row_nnz,
                    const NumTune &t, bool b_sorted, int64_t max_alen, Ctx &c) {
     using V = typename std::conditional<MODE == MODE_F32, float, double>::type;
     constexpr int DT = MODE == MODE_F32 ? SPGEMM_F32 : SPGEMM_F64;
     int *err = &st->err;
-    const int first = t.small_cap >= 32 ? CLS_RANK_S : CLS_B2;
-    if (counts[1] + (first == CLS_RANK_S ? counts[2] : 0) > 0)
+    const int first = t.small_cap >= 32 ? CLS_B2 + 1 : (int)CLS_B2;
+    if (counts[1] + (first > CLS_B2 ? counts[2] : 0) > 0)
         SG_TRY(run_small_g<MODE>(t, a, bdesc, A.nrows, bins, st, err, c));
     int64_t off = 0;
     for (int k = first; k < NCLS; k++) {
@@ -1666,6 +1666,15 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
         // rows left to the maps span more than RANK_S_WORDS blocks, so the
         // maps' own bitmap output (spans up to 32 * BW columns) is kept small
         switch (k) {
+            case CLS_WINDOW_W:
+            case CLS_WINDOW_B:
+                if (MODE == MODE_DW)
+                    SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
+                else
+                    SG_TRY(launch_num_window(DT, A, B, C, bdesc, nar.nlo, nar.nwords, nar.ulist, r, cnt,
+                                             k == CLS_WINDOW_B, cls.nnz[k],
+                                             k == CLS_WINDOW_B ? "numeric.window_block" : "numeric.window_warp", err, c));
+                break;
             case CLS_B2:
             case CLS_RANK_S:
                 if (MODE == MODE_DW)
@@ -1713,6 +1722,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
             case CLS_DENSE:
                 SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, r, cnt, gws, gws_bytes, &st->next_row, err, c));
                 break;
+            case CLS_NARROW: break;   // launch_num_narrow
             default:
                 if (b_sorted) SG_TRY(run_window<V>(a, r, cnt, err, gws, gws_bytes, max_alen, c));
                 else SG_TRY(run_huge<V>(a, B, r, cnt, err, gws, gws_bytes, max_row_nnz, c));
@@ -1723,15 +1733,15 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
 
 int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C,
                    const uint8_t *bins, const int4 *bdesc, const int2 *rspan, const int32_t *rows,
-                   const long long *counts, const ClsInfo &cls, DevState *st, float2 *bsplit, void *gws,
+                   const long long *counts, const ClsInfo &cls, const NarrowInfo &nar, DevState *st, float2 *bsplit, void *gws,
                    size_t gws_bytes, int64_t max_row_nnz, const NumTune &G, bool b_sorted,
                    int64_t max_alen, Ctx &c) {
     NumP a{A.row_ptr, A.col_idx, A.values, B.row_ptr, B.col_idx, B.values, bsplit,
            C.row_ptr, C.col_idx, C.values};
     if (dtype == SPGEMM_F32)
-        return run_all<MODE_F32>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+        return run_all<MODE_F32>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, nar, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
     if (f64_native)
-        return run_all<MODE_F64>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+        return run_all<MODE_F64>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, nar, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
     SG_CUDA(cudaMemsetAsync(&st->b_out_of_range, 0, sizeof(int), c.s));
     if (B.nnz > 0) {
         int64_t blocks = (B.nnz + 255) / 256;
@@ -1741,7 +1751,7 @@ int launch_numeric(int dtype, bool f64_native, const spgemm_csr &A, const spgemm
         c.end();
         SG_CUDA(cudaGetLastError());
     }
-    return run_all<MODE_DW>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
+    return run_all<MODE_DW>(a, A, B, C, bins, bdesc, rspan, rows, counts, cls, nar, st, gws, gws_bytes, max_row_nnz, G, b_sorted, max_alen, c);
 }
 
 }  // namespace sg
