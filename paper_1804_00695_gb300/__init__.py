@@ -232,7 +232,7 @@ def placed_empty(n: int, dtype, placement: str, device="cuda"):
     if placement == "device":
         return torch.empty(n, dtype=dtype, device=device)
     if placement == "pinned":
-        return torch.empty(n, dtype=dtype).pin_memory()
+        return torch.empty(n, dtype=dtype, pin_memory=True)
     if placement == "managed":
         z = np.empty(n, dtype={torch.int64: np.int64, torch.int32: np.int32, torch.float64: np.float64,
                                torch.float32: np.float32}[dtype])
@@ -243,7 +243,7 @@ def placed_empty(n: int, dtype, placement: str, device="cuda"):
 def _empty_like_placed(t):
     """An uninitialised tensor like t in t's placement (pinned stays pinned)."""
     torch = _torch()
-    return torch.empty_like(t).pin_memory() if t.device.type == "cpu" else torch.empty_like(t)
+    return torch.empty_like(t, pin_memory=t.device.type == "cpu")
 
 
 @dataclass
@@ -379,7 +379,7 @@ class Handle:
     def chunked_symbolic(self, A: "HostCsr", B: "HostCsr", budget: int, stream=None, out=None):
         """Row offsets of C (host int64 tensor, pinned; `out` if given) and nnz(C)."""
         torch = _torch()
-        rp = out if out is not None else torch.empty(A.nrows + 1, dtype=torch.int64).pin_memory()
+        rp = out if out is not None else torch.empty(A.nrows + 1, dtype=torch.int64, pin_memory=True)
         if rp.dtype != torch.int64 or rp.numel() != A.nrows + 1 or rp.device.type != "cpu":
             raise ValueError("out must be a host int64 tensor of nrows(A) + 1 entries")
         nnz = C.c_int64()
@@ -392,8 +392,8 @@ class Handle:
                         stream=None) -> "HostCsr":
         """Columns and values of C into pinned host tensors (synchronised)."""
         torch = _torch()
-        col = torch.empty(nnz, dtype=torch.int32).pin_memory()
-        val = torch.empty(nnz, dtype=A.val.dtype).pin_memory()
+        col = torch.empty(nnz, dtype=torch.int32, pin_memory=True)
+        val = torch.empty(nnz, dtype=A.val.dtype, pin_memory=True)
         Cm = HostCsr(A.nrows, B.ncols, row_ptr, col, val)
         da, db, dc = A.desc(), B.desc(), Cm.desc()
         _check(_lib.spgemm_chunked_numeric(self._h, A.dtype_code(), C.byref(da), C.byref(db), C.byref(dc),
@@ -415,13 +415,13 @@ class Handle:
         """Both chunked phases in one call (spgemm_chunked): the entries of C
         are allocated (pinned) by a callback once nnz(C) is known."""
         torch = _torch()
-        rp = torch.empty(A.nrows + 1, dtype=torch.int64).pin_memory()
+        rp = torch.empty(A.nrows + 1, dtype=torch.int64, pin_memory=True)
         held = {}
 
         def alloc(user, nnz, col_p, val_p):
             try:
-                held["col"] = torch.empty(nnz, dtype=torch.int32).pin_memory()
-                held["val"] = torch.empty(nnz, dtype=A.val.dtype).pin_memory()
+                held["col"] = torch.empty(nnz, dtype=torch.int32, pin_memory=True)
+                held["val"] = torch.empty(nnz, dtype=A.val.dtype, pin_memory=True)
             except Exception:
                 return 1
             col_p[0] = held["col"].data_ptr()
@@ -446,7 +446,7 @@ class Handle:
         if keep_on_device:
             rp = torch.empty(A.nrows + 1, dtype=torch.int64, device=dev)
         else:
-            rp = torch.empty(A.nrows + 1, dtype=torch.int64).pin_memory()
+            rp = torch.empty(A.nrows + 1, dtype=torch.int64, pin_memory=True)
         held = {}
 
         def alloc(user, nnz, col_p, val_p):
@@ -455,8 +455,8 @@ class Handle:
                     held["col"] = torch.empty(nnz, dtype=torch.int32, device=dev)
                     held["val"] = torch.empty(nnz, dtype=A.val.dtype, device=dev)
                 else:
-                    held["col"] = torch.empty(nnz, dtype=torch.int32).pin_memory()
-                    held["val"] = torch.empty(nnz, dtype=A.val.dtype).pin_memory()
+                    held["col"] = torch.empty(nnz, dtype=torch.int32, pin_memory=True)
+                    held["val"] = torch.empty(nnz, dtype=A.val.dtype, pin_memory=True)
             except Exception:
                 return 1
             col_p[0] = held["col"].data_ptr() if nnz else None

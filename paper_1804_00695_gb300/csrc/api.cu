@@ -3,6 +3,8 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -44,6 +46,45 @@ void Ctx::end() {
     open = false;
     cudaEventRecord(recs[*nrec].e1, s);
     (*nrec)++;
+}
+
+int kernel_blocks_per_sm(const void *kern, int threads, size_t smem, int *per_sm) {
+    struct Shape {
+        int threads;
+        size_t smem;
+        int per_sm;
+    };
+    struct Known {   // the last shapes of a kernel, and the dynamic shared memory it is opted in to
+        Shape shape[8] = {};
+        int used = 0, next = 0;
+        size_t opted = 0;
+    };
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, Known> known;
+    int dev = 0;
+    SG_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    Known &k = known[{kern, dev}];
+    for (int x = 0; x < k.used; x++)
+        if (k.shape[x].threads == threads && k.shape[x].smem == smem) {
+            *per_sm = k.shape[x].per_sm;
+            return SPGEMM_OK;
+        }
+    if (smem > k.opted) {   // only ever raised: another thread may be about to launch with less
+        SG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k.opted = smem;
+    }
+    int n = 0;
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem));
+    if (n < 1) {
+        set_error("a kernel of %d threads and %zu bytes of shared memory does not fit an SM", threads, smem);
+        return SPGEMM_ERR_INTERNAL;
+    }
+    k.shape[k.next] = Shape{threads, smem, n};
+    k.next = (k.next + 1) % 8;
+    k.used = std::min(k.used + 1, 8);
+    *per_sm = n;
+    return SPGEMM_OK;
 }
 
 }  // namespace sg

@@ -390,13 +390,8 @@ static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, co
                 (V *)C.values, bdesc, rspan, rows, split, count, W, nwin, next};
     SG_CUDA(cudaMemsetAsync(next, 0, sizeof(*next), c.s));
     auto go = [&](auto kern, int T, size_t smem) -> int {
-        SG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 0;
-        SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem));
-        if (per_sm < 1) {
-            set_error("numeric: %zu bytes of shared memory for a dense accumulator", smem);
-            return SPGEMM_ERR_INTERNAL;
-        }
+        SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
         c.begin("numeric.dense", count);
         kern<<<(unsigned)std::min<int64_t>(count, (int64_t)per_sm * c.nsm), T, smem, c.s>>>(p, err);
         c.end();

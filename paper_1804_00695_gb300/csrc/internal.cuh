@@ -187,15 +187,18 @@ constexpr int NARROW_TAB_STRIDE = NARROW_W + 4;
 constexpr int NARROW_BASE_STRIDE = NARROW_W + 4;
 constexpr int NARROW_ACC_STRIDE = NARROW_NMAX + 1;
 
+// Blocks of a kernel that fit an SM with `threads` threads and `smem` bytes of
+// dynamic shared memory (which the kernel is opted in to).  The driver is asked
+// once for each of a kernel's last few shapes on a device; the answers are
+// shared by all handles and threads.
+int kernel_blocks_per_sm(const void *kern, int threads, size_t smem, int *per_sm);
+
 // Blocks of `kern` that fit on all SMs at once (at least one per SM): the
 // kernels that stride over their rows run one resident wave.
 template <typename K>
 static inline int64_t resident_blocks(K kern, int threads, int nsm) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0) != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
+    if (kernel_blocks_per_sm((const void *)kern, threads, 0, &per_sm) != SPGEMM_OK) per_sm = 1;
     return (int64_t)per_sm * nsm;
 }
 

@@ -798,13 +798,8 @@ __global__ void __launch_bounds__(256) k_num_window_rows(WindowP a, size_t per_r
 template <typename V, typename Q, int WR>
 static int run_window_rows(WindowP &p, int *err, const char *label, Ctx &c) {
     const size_t per_row = (WindowSmem<V, Q, WR>::bytes(p.stride) + 15) / 16 * 16, smem = per_row * (8 / WR);
-    SG_CUDA(cudaFuncSetAttribute(k_num_window_rows<V, Q, WR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_num_window_rows<V, Q, WR>, 256, smem));
-    if (per_sm < 1) {
-        set_error("numeric: %zu bytes of shared memory for the window rows", smem);
-        return SPGEMM_ERR_INTERNAL;
-    }
+    SG_TRY(kernel_blocks_per_sm((const void *)k_num_window_rows<V, Q, WR>, 256, smem, &per_sm));
     const int64_t blocks = std::min<int64_t>((p.count * WR + 7) / 8, (int64_t)per_sm * c.nsm);
     c.begin(label, p.count);
     k_num_window_rows<V, Q, WR><<<(unsigned)blocks, 256, smem, c.s>>>(p, per_row, err);

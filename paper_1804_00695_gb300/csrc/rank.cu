@@ -331,13 +331,8 @@ template <typename V, typename Q, int T, int U, int MINB>
 static int run_rank_block(const RankP<V> &p, int *err, const char *label, Ctx &c) {
     auto kern = k_num_rank_block<V, Q, T, U, MINB>;
     const size_t smem = RankSmem<V, T>(p.bw, p.nmax).bytes;
-    SG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem));
-    if (per_sm < 1) {
-        set_error("numeric: %zu bytes of shared memory for a rank accumulator", smem);
-        return SPGEMM_ERR_INTERNAL;
-    }
+    SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
     const int64_t blocks = std::min<int64_t>(p.count, (int64_t)per_sm * c.nsm);
     c.begin(label, p.count);
     kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);

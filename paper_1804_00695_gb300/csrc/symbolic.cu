@@ -734,13 +734,8 @@ template <int NT>
 static int run_bitmap(const BitmapP &p, DevState *st, const char *label, Ctx &c) {
     const int threads = NT == 32 ? BM_WPB * 32 : NT;
     const size_t smem = BitmapSmem<NT>::bytes(p.bw, NT == 32 ? BM_WPB : 1);
-    SG_CUDA(cudaFuncSetAttribute(k_sym_rows<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sym_rows<NT>, threads, smem));
-    if (per_sm < 1) {
-        set_error("symbolic: %zu bytes of shared memory for a bitmap", smem);
-        return SPGEMM_ERR_INTERNAL;
-    }
+    SG_TRY(kernel_blocks_per_sm((const void *)k_sym_rows<NT>, threads, smem, &per_sm));
     const int64_t blocks = std::min<int64_t>((p.n * NT + threads - 1) / threads, (int64_t)per_sm * c.nsm);
     c.begin(label, p.n);
     k_sym_rows<NT><<<(unsigned)blocks, threads, smem, c.s>>>(p, st);
