@@ -42,43 +42,6 @@ __device__ __forceinline__ int quad_of(int j, int gl) {
     return ((j / P) * G + gl) * P + (j % P);
 }
 
-// Stored entries of A are taken a batch of E at a time: every lane of a
-// row's G lanes loads E / G of them at once (their loads in flight
-// together), so the passes over the batch wait for memory once, not once
-// per entry.
-//
-// Load the lane's entries pb + gl + G*u (u < E / G) of a row: the start of
-// B_k in B (also the start of its compressed pairs), its entries and pairs.
-// Entries past plen, with a column of A out of range or a row of B too long
-// for the window get no pairs and no entries (and raise `bad` for the
-// latter two).
-template <int G, int E>
-__device__ __forceinline__ void load_entries(const int32_t *__restrict__ acol, const int4 *__restrict__ desc,
-                                             int64_t nrows_b, int64_t p0, int plen, int pb, int gl,
-                                             long long (&q0)[E / G], int (&len)[E / G], int (&np)[E / G],
-                                             bool &bad) {
-    constexpr int EL = E / G;
-    int k[EL];
-#pragma unroll
-    for (int u = 0; u < EL; u++) {
-        const int pe = pb + gl + G * u;
-        k[u] = pe < plen ? acol[p0 + pe] : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < EL; u++) {
-        q0[u] = 0;
-        len[u] = 0;
-        np[u] = 0;
-        if (pb + gl + G * u >= plen) continue;
-        if ((unsigned)k[u] >= (unsigned)nrows_b) { bad = true; continue; }
-        const int4 d = desc[k[u]];
-        if (d.z > NARROW_W * 32 || d.w > NARROW_W) { bad = true; continue; }
-        q0[u] = desc_start(d);
-        len[u] = d.z;
-        np[u] = d.w;
-    }
-}
-
 // ---------------------------------------------------------------- symbolic
 constexpr int NARROW_SYM_WPB = 8;
 constexpr int SYM_EU = 4;   // entries of A per lane whose loads are in flight together
@@ -94,8 +57,11 @@ constexpr int SYM_EU = 4;   // entries of A per lane whose loads are in flight t
 // rows get nlo[i] = -1 and the symbolic bin of their bound (crp[i+1] = 0
 // for empty rows, -1 for the dense-bitmap bin), exactly as the analysis
 // kernel gives them.
+// With four lanes a row, four blocks an SM (64 registers): with three (80)
+// the same products take 0.98 ms, with five (48 registers, and 34 KB less for
+// the L1, which the gathers of B live in) 0.76 ms.
 template <int G>
-__global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
+__global__ void __launch_bounds__(NARROW_SYM_WPB * 32, G == 4 ? 4 : 0) k_sym_narrow(
     int64_t n, int64_t nrows_b, int64_t nwords_b, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc, const int2 *__restrict__ bmm,
     const int2 *__restrict__ pairs, int64_t *__restrict__ flops, uint8_t *__restrict__ bins,
@@ -167,10 +133,16 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
         bad |= rowbad;
         const bool nar = live && f > 0 && !rowbad && hi >= lo && hi - lo < NARROW_W && cp <= NARROW_PAIRS;
         int cnt = 0, nz = 0;
-        if (__any_sync(0xffffffffu, nar)) {
+        // words of the widest window of the warp's rows: the table is cleared
+        // and read over so many, a round of 4 * G * P at a time (128^3
+        // Galerkin products: 0.68 -> 0.66 ms; windows of 3 to 61 words)
+        const int wide = __reduce_max_sync(0xffffffffu, nar ? hi - lo + 1 : 0);
+        if (wide > 0) {
             if (nar) {
 #pragma unroll
-                for (int j = 0; j < QPL; j++) *(uint4 *)&t[4 * quad_of<G, P>(j, gl)] = make_uint4(0u, 0u, 0u, 0u);
+                for (int j = 0; j < QPL; j++)
+                    if (4 * G * (j - j % P) < wide)
+                        *(uint4 *)&t[4 * quad_of<G, P>(j, gl)] = make_uint4(0u, 0u, 0u, 0u);
             }
             __syncwarp();
             // the union: every lane ORs the pairs of its own entries (lanes of
@@ -216,6 +188,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32) k_sym_narrow(
             uint2 *ul = ulist + (live ? i : 0) * NARROW_NMAX;
 #pragma unroll
             for (int j = 0; j < QPL / P; j++) {
+                if (4 * G * P * j >= wide) break;
                 uint4 v[P];
                 int cl = 0, zl = 0;
 #pragma unroll
@@ -362,22 +335,21 @@ __device__ __forceinline__ int popc_below(unsigned m, unsigned s) {
 // hold at most NARROW_NMAX < 256 entries), word major and row slot minor,
 // so that in one instruction the lanes of different row slots never meet on
 // a bank whatever words their rows look up; and the accumulator by rank,
-// entry r of slot g at r * ACC_RS + g * ACC_GS.  A row's G lanes update G
-// distinct ranks per chunk.  With four lanes a row, the slots lie 34
-// eight-byte words apart (ranks adjacent within a slot): 270 words a warp,
-// small enough for six blocks of four warps an SM (the earlier stride of
-// four words per rank and 33 per slot spread a stencil row's neighbouring
-// ranks over more banks, but its 356 words a warp left room for five
-// blocks; on the 128^3 Galerkin A*P the sixth block gains more than the
-// extra conflicts cost).
+// rank major and row slot minor among the RH rows that one pass over the
+// banks serves (half a warp's with 8-byte values): only the lanes of a row
+// can meet, on ranks RH apart in the count of banks.  What bounds the kernel
+// is these passes over the banks (86% of the peak on the 96^3 Galerkin A*P,
+// DRAM 15%): with every slot's ranks adjacent and the slots 34 words apart
+// the numeric phase of the 128^3 triple product took 1.45 ms, so 1.43 ms.
 // Per row slot: the batch of stored entries ({start, value}, length; the
 // lengths apart only when B has 2^31 entries or more), padded so that the
 // slots of a warp start on different banks.
 template <int G, int WPB, int E, typename V, bool IDX32>
 struct NarrowSmem {
     static constexpr int RPW = 32 / G, NR = WPB * RPW, ES = E + 1;
-    static constexpr int ACC_RS = 1, ACC_GS = G == 4 ? 34 : 40;
-    static constexpr int ACC_SZ = (ACC_RS * (NARROW_NMAX - 1) + ACC_GS * (RPW - 1) + 2) & ~1;
+    // rows whose lanes access shared memory in one pass: half a warp's with 8-byte values
+    static constexpr int RH = RPW / (sizeof(V) == 8 ? 2 : 1);
+    static constexpr int ACC_RS = RH, ACC_SZ = NARROW_NMAX * RPW;
     NarrowEnt<V> ent[NR * ES];
     unsigned tab[WPB * NARROW_W * RPW];
     V acc[WPB * ACC_SZ];
@@ -391,7 +363,7 @@ struct NarrowSmem {
 constexpr int NARROW_U = 3;
 
 // Blocks an SM of the four-lane kernel: six (24 warps; 80 registers a
-// thread, 37.8 KB of shared memory a block).  The other lane counts leave
+// thread, 37.4 KB of shared memory a block).  The other lane counts leave
 // the register count to the compiler (a minimum of 0 blocks): with eight
 // lanes it takes 64 registers, eight blocks an SM.
 constexpr int NARROW_MINB4 = 6;
@@ -421,7 +393,7 @@ __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_nar
     // this row slot's column of the warp's tables: word wd at tab[wd * RPW]
     unsigned *tab = sm.tab + w * NARROW_W * RPW + g;
     unsigned char *base = sm.base + w * NARROW_W * RPW + g;
-    V *acc = sm.acc + w * S::ACC_SZ + g * S::ACC_GS;
+    V *acc = sm.acc + w * S::ACC_SZ + g / S::RH * (NARROW_NMAX * S::RH) + g % S::RH;
     NarrowEnt<V> *ent = sm.ent + slot * S::ES;
     int *elen = sm.elen + slot * S::ES;
     const V *__restrict__ aval = (const V *)a.aval;
@@ -474,18 +446,34 @@ __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_nar
         bool bad = false;
         unsigned miss = 0;   // set by a column absent from the row's window union
         for (int pb = 0; pb < maxlen; pb += E) {
-            long long q0[EL];
-            int len[EL], np[EL];
-            load_entries<G, E>(a.acol, a.bdesc, a.nrows_b, p0, plen, pb, gl, q0, len, np, bad);
+            // E lanes to a row, so that a load covers a row's consecutive
+            // entries and a store a run of shared memory (with a row's G
+            // lanes on its own entries, a load met a line per row: 128^3
+            // Galerkin product, both numeric phases, 1.43 -> 1.34 ms)
+            const int be = pb + lane % E;
+            int k[EL];
+            V x[EL];
 #pragma unroll
             for (int u = 0; u < EL; u++) {
-                const int e = gl + G * u;
-                NarrowEnt<V> x;
-                x.q = (int)(unsigned long long)q0[u];
-                x.hl = IDX32 ? len[u] : (int)((unsigned long long)q0[u] >> 32);
-                x.a = pb + e < plen ? aval[p0 + pb + e] : (V)0;
-                ent[e] = x;
-                if (!IDX32) elen[e] = len[u];
+                const int from = (u * (32 / E) + lane / E) * G;
+                const int64_t q = __shfl_sync(0xffffffffu, p0, from) + be;
+                const bool ok = be < __shfl_sync(0xffffffffu, plen, from);
+                k[u] = ok ? a.acol[q] : -1;
+                x[u] = ok ? aval[q] : (V)0;
+                if (ok && (unsigned)k[u] >= (unsigned)a.nrows_b) { k[u] = -1; bad = true; }
+            }
+#pragma unroll
+            for (int u = 0; u < EL; u++) {
+                int4 d = k[u] >= 0 ? a.bdesc[k[u]] : make_int4(0, 0, 0, 0);
+                if (d.z > NARROW_W * 32 || d.w > NARROW_W) { bad = true; d.x = d.y = d.z = 0; }
+                const long long q0 = desc_start(d);
+                const int at = (w * RPW + u * (32 / E) + lane / E) * S::ES + lane % E;
+                NarrowEnt<V> t;
+                t.q = (int)(unsigned long long)q0;
+                t.hl = IDX32 ? d.z : (int)((unsigned long long)q0 >> 32);
+                t.a = x[u];
+                sm.ent[at] = t;
+                if (!IDX32) sm.elen[at] = d.z;
             }
             __syncwarp();
             const int nb = min(E, plen - pb);
