@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(NARROW_SYM_WPB * 32, G == 4 ? 4 : 0) k_sym_nar
                     for (int u = 0; u < SYM_EU; u++) {
                         const int4 d = k[u] >= 0 ? desc[k[u]] : make_int4(0, 0, 0, 0);
                         pp[u] = pairs + desc_start(d);
-                        np[u] = d.w <= NARROW_W ? d.w : 0;
+                        np[u] = d.w;   // at most NARROW_PAIRS in a narrow row
                         npmax = max(npmax, np[u]);
                     }
                     for (int tt = 0; tt < npmax; tt++) {
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(WPB * 32, G == 4 ? NARROW_MINB4 : 0) k_num_nar
 #pragma unroll
             for (int u = 0; u < EL; u++) {
                 int4 d = k[u] >= 0 ? a.bdesc[k[u]] : make_int4(0, 0, 0, 0);
-                if (d.z > NARROW_W * 32 || d.w > NARROW_W) { bad = true; d.x = d.y = d.z = 0; }
+                if (d.z > NARROW_W * 32) { bad = true; d.x = d.y = d.z = 0; }
                 const long long q0 = desc_start(d);
                 const int at = (w * RPW + u * (32 / E) + lane / E) * S::ES + lane % E;
                 NarrowEnt<V> t;
