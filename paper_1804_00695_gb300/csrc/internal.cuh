@@ -125,6 +125,7 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //               word list the symbolic phase left whole: a warp, or from
 //               WINDOW_FLOPS products on a block
 //   CLS_NARROW  BIN_NARROW (a list only when other rows lie between them)
+//   CLS_RANK_W  at most RANK_W_FLOPS products over at most RANK_M_WORDS blocks
 //   CLS_RANK_S  at most RANK_S_NNZ outputs over at most RANK_S_WORDS blocks
 //   CLS_RANK_M4, CLS_RANK_M5  wider spans up to RANK_M_WORDS blocks: rows
 //               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
@@ -132,16 +133,19 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //   CLS_BLOCK, CLS_HUGE       other rows of bins 5 and 6
 //   CLS_DENSE   rows of B sorted: rows with more outputs than the rank
 //               accumulators hold, or many products over their span
-// Why the lines lie there: 2048 blocks are the bitmap that 128 threads scan in
+// Why the lines lie there: 512 products are eight a lane for the two warps of
+// a short row (rank.cu has both sides; 8192 blocks keep its first bitmap
+// within 1.5 KB); 2048 blocks are the bitmap that 128 threads scan in
 // one step of 16 words, 8192 the one that 512 threads do; a row of 8192 FP64
 // outputs over 8192 blocks takes 167 KB of shared memory, the next power of
 // two would not fit.  Below them the rank accumulators measured 2.6-5x
 // faster than the maps and windows (rank.cu has the figures).
 enum NumCls {
-    CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
+    CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_W, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
     CLS_BLOCK, CLS_DENSE, CLS_HUGE, CLS_NARROW, NCLS
 };
 constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
+constexpr int RANK_W_FLOPS = 512;
 constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit 32 bits)
 // Dense windows from one product per 8 columns of the span on (their cost per
 // row is the span written out plus the products, the rank accumulators' the
@@ -161,6 +165,7 @@ __host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, 
         (nnz > RANK_M_NNZ || (flops > DENSE_FLOPS && flops * 8 >= (long long)words * 32)))
         return CLS_DENSE;
     if (words > 0 && flops <= RANK_FLOPS) {
+        if (flops <= RANK_W_FLOPS && words <= RANK_M_WORDS) return CLS_RANK_W;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_S_WORDS) return CLS_RANK_S;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_M_WORDS) return CLS_RANK_M4;
         if (nnz <= RANK_M_NNZ && words <= RANK_M_WORDS) return CLS_RANK_M5;
@@ -385,9 +390,11 @@ size_t window_global_ws(int64_t max_alen, int nsm);
 
 // rank.cu: listed rows with a dense rank accumulator (a block each), in FP32
 // or native FP64; rows wider than max_words blocks or with more than max_nnz
-// outputs are skipped.  small: rows of CLS_RANK_S (or CLS_B2).
+// outputs are skipped.  RANK_SHORT: rows of CLS_RANK_W; RANK_ROW: of
+// CLS_RANK_S (or CLS_B2).
+enum RankSize { RANK_SHORT, RANK_ROW, RANK_LONG };
 int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                    const int2 *rspan, const int32_t *rows, int64_t count, bool small, int64_t max_nnz,
+                    const int2 *rspan, const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz,
                     int64_t max_words, int *err, Ctx &c);
 
 // dense.cu: listed rows over windows of a dense accumulator (rows of B

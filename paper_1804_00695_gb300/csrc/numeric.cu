@@ -1657,6 +1657,12 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
     const int first = t.small_cap >= 32 ? CLS_B2 + 1 : (int)CLS_B2;
     if (counts[1] + (first > CLS_B2 ? counts[2] : 0) > 0)
         SG_TRY(run_small_g<MODE>(t, a, bdesc, A.nrows, bins, st, err, c));
+    // Few short rows go along with the longer ones in one launch (their spans
+    // allowing): 538 rows of 1000 columns (FP64) take 10 us so, 22 us apart;
+    // 19,995 rows over 20,001 columns (FP32) 78 and 79 us; 920,127 rows over
+    // up to 65,536 columns 3.47 and 3.00 ms.
+    const bool short_with_rows = MODE != MODE_DW && cls.count[CLS_RANK_S] > 0 && cls.words[CLS_RANK_W] <= RANK_S_WORDS &&
+                                 cls.count[CLS_RANK_W] < (int64_t)c.nsm * 96;
     int64_t off = 0;
     for (int k = first; k < NCLS; k++) {
         int64_t cnt = cls.count[k];
@@ -1675,13 +1681,30 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                                              k == CLS_WINDOW_B, cls.nnz[k],
                                              k == CLS_WINDOW_B ? "numeric.window_block" : "numeric.window_warp", err, c));
                 break;
+            case CLS_RANK_W:
+                if (short_with_rows) break;   // one launch with the next list
+                if (MODE != MODE_DW) {
+                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, RANK_SHORT, cls.nnz[k], cls.words[k], err, c));
+                    break;
+                }
+                SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
+                if (cls.words[k] > RANK_S_WORDS) {
+                    SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
+                    SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
+                }
+                break;
             case CLS_B2:
             case CLS_RANK_S:
                 if (MODE == MODE_DW)
                     SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
-                else
-                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, true, cls.nnz[k],
-                                           std::min(cls.words[k], RANK_S_WORDS), err, c));
+                else {
+                    const bool both = k == CLS_RANK_S && short_with_rows;
+                    const int64_t more = both ? cls.count[CLS_RANK_W] : 0;
+                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r - more, cnt + more, RANK_ROW,
+                                           both ? std::max(cls.nnz[k], cls.nnz[CLS_RANK_W]) : cls.nnz[k],
+                                           std::min(both ? std::max(cls.words[k], cls.words[CLS_RANK_W]) : cls.words[k],
+                                                    RANK_S_WORDS), err, c));
+                }
                 if (k == CLS_B2 && cls.words[k] > RANK_S_WORDS)
                     SG_TRY((run_wide<256, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide3", c)));
                 break;
@@ -1693,7 +1716,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                     break;
                 }
                 if (cls.count[CLS_RANK_M5]) break;   // one launch with the next list
-                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, false, cls.nnz[k], cls.words[k], err, c));
+                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, RANK_LONG, cls.nnz[k], cls.words[k], err, c));
                 break;
             case CLS_RANK_M5: {
                 int nmax = cls.nnz[k], words = cls.words[k];
@@ -1703,7 +1726,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                     nmax = std::max(nmax, cls.nnz[CLS_RANK_M4]);
                     words = std::max(words, cls.words[CLS_RANK_M4]);
                 }
-                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, false, nmax, words, err, c));
+                SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, RANK_LONG, nmax, words, err, c));
                 break;
             }
             case CLS_WIDE3:

@@ -341,22 +341,294 @@ static int run_rank_block(const RankP<V> &p, int *err, const char *label, Ctx &c
     return SPGEMM_OK;
 }
 
+// ---------------------------------------------------------------- short rows
+// Rows of at most RANK_W_FLOPS products: T threads per row, the products in
+// their registers, and the bitmap of the span in two levels.  A first bitmap
+// holds a bit per 32-column block of the span; its prefix counts number the
+// row's non-empty blocks, and only these get a word of the second bitmap.  So
+// what is cleared and scanned is a word per 1024 columns and a word per
+// non-empty block (at most one per output) instead of a word per 32 columns,
+// and shared memory follows the outputs, not the span.
+//
+//   1. The stored a_ik are staged 32 at a time, one a lane; the row's
+//      products 32s .. 32s+31 are slot s / NW of warp s % NW.  Every
+//      product's block is marked in the first bitmap.
+//   2. Its prefix counts give a product's word of the second bitmap; the lane
+//      that sets a bit there first keeps the product as the entry's value.
+//   3. The prefix counts of the second bitmap turn a bit into its rank; first
+//      products are stored, the others added; values and columns leave as
+//      contiguous copies.
+// What bounds it: instruction issue (2.3 of 4 slots a cycle; about 2,100 warp
+// instructions a row of 290 products, of which loading the products takes
+// 360, the two bitmaps 480, the ranks 260, the output 290) and the chain of
+// loads and barriers behind it.  Measured (one GB300, FP32): 795,129 rows of
+// 64 products of up to 65,536 columns, with the block kernel's 124,998 longer
+// ones, 3.47 -> 3.00 ms; 86,197 such rows over 100,000 columns (spans that the
+// 128-thread block's bitmap does not hold) 1.36 -> 0.50 ms; FP64, 299,537
+// rows with 48,168 longer ones, 1.45 -> 1.22 ms.  Two warps a row: a warp
+// with 16 products a lane takes 3.04 ms for the first (its code no longer
+// fits the instruction cache), 128 threads with four a lane 2.83; 96 threads
+// for up to 768 products take all its rows at 3.20.
+//
+// The lanes past a row's last product carry a column of their own beyond the
+// span, whose place in every table is one that nothing reads: no branch keeps
+// them apart.
+template <typename V>
+struct RankWSmem {
+    int np;   // outputs in whole 16-byte words: the place of what nothing reads
+    size_t eq, ea, pre, coarse, cpre, masks, info, cols, acc, bytes;
+    __host__ __device__ RankWSmem(int cw, int nmax) {
+        size_t o = 0;
+        auto take = [&](size_t b) { const size_t p = o; o += (b + 15) & ~(size_t)15; return p; };
+        np = (nmax + 3) & ~3;
+        eq = take(32 * 8);
+        ea = take(32 * sizeof(V));
+        pre = take(32 * 4);
+        coarse = take((size_t)(cw + 1) * 4);
+        cpre = take((size_t)(cw + 1) * 2);
+        masks = take((size_t)(np + 1) * 4);
+        info = take((size_t)(np + 1) * 4);     // per word: block << 16, then + rank of its first column
+        cols = take((size_t)(np + 1) * 4);
+        acc = take((size_t)(np + 1) * sizeof(V));
+        bytes = o;
+    }
+};
+
+// bw, nmax of the parameters: words of the first bitmap, outputs.
+template <typename V, typename Q, int T, int MINB>
+__global__ void __launch_bounds__(T, MINB) k_num_rank_short(RankP<V> a, int *err) {
+    constexpr int NW = T / 32, U = RANK_W_FLOPS / T, UB = U < 8 ? U : 8;
+    static_assert(U * T == RANK_W_FLOPS && U % UB == 0, "whole slots");
+    extern __shared__ __align__(16) unsigned char mem[];
+    __shared__ int s_nz, s_done;
+    const RankWSmem<V> L(a.bw, a.nmax);
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    Q *eq = (Q *)(mem + L.eq);
+    V *ea = (V *)(mem + L.ea), *acc = (V *)(mem + L.acc);
+    int *pre = (int *)(mem + L.pre), *cols = (int *)(mem + L.cols);
+    unsigned *coarse = (unsigned *)(mem + L.coarse), *masks = (unsigned *)(mem + L.masks), *info = (unsigned *)(mem + L.info);
+    unsigned short *cpre = (unsigned short *)(mem + L.cpre);
+    const unsigned below = (1u << lane) - 1u, upto = 2u * below + 1u;
+    const int none = a.bw * 1024;   // column (less the span's first) of no product
+    const int32_t *__restrict__ bcol = a.bcol;
+    const V *__restrict__ bval = a.bval;
+    int flag = 0;
+    for (int x = tid; x < a.bw; x += T) coarse[x] = 0u;
+    for (int x = tid; x < L.np; x += T) masks[x] = 0u;
+    if (tid == 0) {
+        coarse[a.bw] = 0u;
+        cpre[a.bw] = (unsigned short)L.np;
+        masks[L.np] = 0xffffffffu;   // never the first
+    }
+    auto scan = [&](int v) {   // inclusive sum over the lanes
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, v, d);
+            if (lane >= d) v += y;
+        }
+        return v;
+    };
+
+    for (int64_t t = blockIdx.x; t < a.count; t += gridDim.x) {
+        const int i = a.rows[t];
+        const int2 sp = a.rspan[i];
+        const int64_t out = a.crp[i];
+        const int nn = (int)(a.crp[i + 1] - out);
+        const int col0 = sp.x * 32, ncol = sp.y * 32, cwn = (sp.y + 31) >> 5;
+        const int64_t p0 = a.arp[i];
+        const int plen = (int)(a.arp[i + 1] - p0);
+        if (sp.y <= 0 || cwn > a.bw || nn > a.nmax) { flag |= DERR_COUNT; continue; }
+        int c[U];
+        V p[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) c[u] = none;
+        int total = 0;
+        bool fits = true;
+        for (int pb = 0; pb < plen; pb += 32) {   // every warp the same, warp 0 writes
+            int len = 0;
+            Q q0 = 0;
+            if (pb + lane < plen) {
+                const int4 d = a.bdesc[a.acol[p0 + pb + lane]];
+                len = d.z;
+                q0 = (Q)desc_start(d);
+            }
+            const int incl = scan(len), tot = __shfl_sync(0xffffffffu, incl, 31);
+            const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+            fits = tot <= RANK_W_FLOPS - total && __all_sync(0xffffffffu, len <= RANK_W_FLOPS);
+            if (!fits) break;   // A or B changed since the symbolic phase
+            if (pb > 0) __syncthreads();
+            if (w == 0 && len > 0) {
+                const int pos = __popc(some & below), at = total + incl - len;
+                pre[pos] = at;
+                eq[pos] = q0 - at;
+                ea[pos] = a.aval[p0 + pb + lane];
+            }
+            __syncthreads();
+            const int at = lane < __popc(some) ? pre[lane] : INT_MAX;   // first product of entry `lane`
+            const int tend = total + tot;
+#pragma unroll
+            for (int u0 = 0; u0 < U; u0 += UB) {
+                if (32 * (NW * u0 + w) >= tend) break;
+                V av[UB];
+#pragma unroll
+                for (int u = 0; u < UB; u++) {
+                    const int tc = 32 * (NW * (u0 + u) + w), g = tc + lane;
+                    av[u] = V(1);
+                    if (tc < tend && tc + 32 > total) {
+                        // entries that start before the step, and those up to the lane's product
+                        const int b = at - tc;
+                        const unsigned m = __reduce_or_sync(0xffffffffu, (unsigned)b < 32u ? 1u << b : 0u);
+                        const int e = __popc(__ballot_sync(0xffffffffu, b < 0)) + __popc(m & upto) - 1;
+                        if (g >= total && g < tend) {
+                            const Q q = eq[e] + (Q)g;
+                            c[u0 + u] = bcol[q];
+                            p[u0 + u] = bval[q];
+                            av[u] = ea[e];
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UB; u++) {
+                    const int tc = 32 * (NW * (u0 + u) + w), g = tc + lane;
+                    if (tc >= tend) break;
+                    p[u0 + u] *= av[u];
+                    int &cc = c[u0 + u];
+                    if (g >= total && g < tend) {
+                        cc -= col0;
+                        if ((unsigned)cc >= (unsigned)ncol) {
+                            flag |= DERR_COUNT;
+                            cc = none;
+                        }
+                    }
+                    atomicOr(&coarse[cc >> 10], 1u << (cc >> 5 & 31));
+                }
+            }
+            total = tend;
+        }
+        __syncthreads();
+        if (w == 0) {
+            // prefix counts of the first bitmap's words
+            int n = 0;
+            for (int x0 = 0; x0 < cwn; x0 += 32) {
+                const int x = x0 + lane, s = x < cwn ? __popc(coarse[x]) : 0, incl = scan(s);
+                if (x < cwn) cpre[x] = (unsigned short)(n + incl - s);
+                n += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) s_nz = n;
+        }
+        __syncthreads();
+        const int nz = s_nz;
+        const bool listed = fits && nz <= nn;
+        unsigned first = 0, more = 0;
+        if (listed) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (32 * (NW * u + w) >= total) break;
+                const int x = c[u] >> 10;
+                const int k = (int)cpre[x] + __popc(coarse[x] & ((1u << (c[u] >> 5 & 31)) - 1u));
+                const unsigned bit = 1u << (c[u] & 31);
+                const bool is = !(atomicOr(&masks[k], bit) & bit);
+                info[k] = (unsigned)(c[u] >> 5) << 16;
+                first |= is ? 1u << u : 0u;
+                more |= !is && c[u] != none ? 1u << u : 0u;
+                c[u] = (k << 5) | (c[u] & 31);
+            }
+            __syncthreads();
+            if (w == 0) {
+                // prefix counts of the second bitmap's words, four a lane
+                int n = 0;
+                for (int x0 = 0; x0 < nz; x0 += 128) {
+                    const int x = x0 + 4 * lane;
+                    uint4 v = x < nz ? *(const uint4 *)&masks[x] : make_uint4(0u, 0u, 0u, 0u);
+                    v.x = __popc(v.x);
+                    v.y = v.x + __popc(v.y);
+                    v.z = v.y + __popc(v.z);
+                    v.w = v.z + __popc(v.w);
+                    const int incl = scan((int)v.w);
+                    if (x < nz) {
+                        const unsigned r = (unsigned)(n + incl) - v.w;
+                        uint4 f = *(const uint4 *)&info[x];
+                        f.x += r;
+                        f.y += r + v.x;
+                        f.z += r + v.y;
+                        f.w += r + v.z;
+                        *(uint4 *)&info[x] = f;
+                    }
+                    n += __shfl_sync(0xffffffffu, incl, 31);
+                }
+                if (lane == 0) s_done = n;
+            }
+        }
+        __syncthreads();
+        if (listed && s_done == nn) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (32 * (NW * u + w) >= total) break;
+                const int k = c[u] >> 5, b = c[u] & 31;
+                const unsigned in = info[k];
+                const int r = (int)(in & 0xffffu) + __popc(masks[k] & ((1u << b) - 1u));
+                if ((first >> u) & 1u) {
+                    acc[r] = p[u];
+                    cols[r] = col0 + (int)(in >> 16) * 32 + b;
+                }
+            }
+            if (__syncthreads_or(more != 0)) {
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (32 * (NW * u + w) >= total) break;
+                    if (!((more >> u) & 1u)) continue;
+                    const int k = c[u] >> 5;
+                    atomicAdd(&acc[(int)(info[k] & 0xffffu) + __popc(masks[k] & ((1u << (c[u] & 31)) - 1u))], p[u]);
+                }
+                __syncthreads();
+            }
+            for (int x = tid; x < nn; x += T) {
+                a.ccol[out + x] = cols[x];
+                a.cval[out + x] = acc[x];
+            }
+        } else {
+            flag |= DERR_COUNT;   // not the pattern of the symbolic phase: nothing is written
+        }
+        if (listed)
+            for (int x = 4 * tid; x < nz; x += 4 * T) *(uint4 *)&masks[x] = make_uint4(0u, 0u, 0u, 0u);
+        for (int x = tid; x < cwn; x += T) coarse[x] = 0u;
+        __syncthreads();
+    }
+    if (flag) atomicOr(err, flag);
+}
+
 template <typename V, typename Q>
 static int num_rank(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc, const int2 *rspan,
-                    const int32_t *rows, int64_t count, bool small, int64_t max_nnz, int64_t max_words, int *err,
+                    const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz, int64_t max_words, int *err,
                     Ctx &c) {
+    if (size == RANK_SHORT) {
+        constexpr int T = 64;
+        RankP<V> p{A.row_ptr, A.col_idx, (const V *)A.values, B.col_idx, (const V *)B.values,
+                   C.row_ptr, C.col_idx, (V *)C.values, bdesc, rspan, rows, count,
+                   (int)((max_words + 31) / 32), (int)max_nnz};
+        auto kern = k_num_rank_short<V, Q, T, 16>;
+        const size_t smem = RankWSmem<V>(p.bw, p.nmax).bytes;
+        int per_sm = 0;
+        SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
+        const int64_t blocks = std::min<int64_t>(count, (int64_t)per_sm * c.nsm);
+        c.begin("numeric.rank_short", count);
+        kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);
+        c.end();
+        SG_CUDA(cudaGetLastError());
+        return SPGEMM_OK;
+    }
     const int bw = (int)((max_words + 15) & ~(int64_t)15);
     RankP<V> p{A.row_ptr, A.col_idx, (const V *)A.values, B.col_idx, (const V *)B.values,
                C.row_ptr, C.col_idx, (V *)C.values, bdesc, rspan, rows, count, bw, (int)max_nnz};
-    if (small) return run_rank_block<V, Q, 128, 8, 8>(p, err, "numeric.rank_row", c);
+    if (size == RANK_ROW) return run_rank_block<V, Q, 128, 8, 8>(p, err, "numeric.rank_row", c);
     return run_rank_block<V, Q, 512, 12, 2>(p, err, "numeric.rank_long", c);
 }
 
 int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                    const int2 *rspan, const int32_t *rows, int64_t count, bool small, int64_t max_nnz,
+                    const int2 *rspan, const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz,
                     int64_t max_words, int *err, Ctx &c) {
     if (count <= 0) return SPGEMM_OK;
-    auto go = [&](auto run) { return run(A, B, C, bdesc, rspan, rows, count, small, max_nnz, max_words, err, c); };
+    auto go = [&](auto run) { return run(A, B, C, bdesc, rspan, rows, count, size, max_nnz, max_words, err, c); };
     if (B.nnz < ((int64_t)1 << 31) - RANK_FLOPS)   // offsets less a row's first products stay in an int
         return dtype == SPGEMM_F32 ? go(num_rank<float, int>) : go(num_rank<double, int>);
     return dtype == SPGEMM_F32 ? go(num_rank<float, long long>) : go(num_rank<double, long long>);
