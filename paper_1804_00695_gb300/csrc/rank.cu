@@ -23,9 +23,11 @@
 // 320 products; DRAM 9%, L1 48%), about 2,400 warp instructions a row of
 // which some 60% do not depend on the products.  Measured (one GB300):
 // 294 M products of 921,066 rows of 4-32 by 4-32 uniform entries (FP32) 9.65
-// -> 3.50 ms against a warp per row with two passes over B, 13 warps an SM
+// -> 3.47 ms (3.00 since two warps take the shorter ones, see below) against a
+// warp per row with two passes over B, 13 warps an SM
 // and stores scattered by word; 41,472 rows of about 4,500 outputs over
-// 41,472 columns (FP64) 9.56 -> 1.90 ms against a block's hash map with its
+// 41,472 columns (FP64) 9.56 -> 1.79 ms (1.87 while a product that is added
+// looked its rank up a second time) against a block's hash map with its
 // ordering (bin 5) and the window kernel (bin 6).  Blocks of 64 and 32
 // threads took 4.1 and 8.7 ms on the first (shared memory then holds too few
 // warps), 256 took 5.9; on the second 1024 x 8 took 2.9, 512 x 8 (a second
@@ -274,17 +276,21 @@ __global__ void __launch_bounds__(T, MINB) k_num_rank_block(RankP<V> a, int *err
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     if (u >= per) break;
-                    if (!((first >> u) & 1u)) continue;
+                    if (!((mine >> u) & 1u)) continue;
                     const int r = rank_of(c[u]);
-                    acc[r] = p[u];
-                    cols[r] = c[u];
+                    if ((first >> u) & 1u) {
+                        acc[r] = p[u];
+                        cols[r] = c[u];
+                    } else {
+                        c[u] = r;   // only the place is needed from here on
+                    }
                 }
                 mine &= ~first;
                 if (__syncthreads_or(mine != 0)) {
 #pragma unroll
                     for (int u = 0; u < U; u++) {
                         if (u >= per) break;
-                        if ((mine >> u) & 1u) atomicAdd(&acc[rank_of(c[u])], p[u]);
+                        if ((mine >> u) & 1u) atomicAdd(&acc[c[u]], p[u]);
                     }
                     __syncthreads();
                 }
@@ -571,14 +577,13 @@ __global__ void __launch_bounds__(T, MINB) k_num_rank_short(RankP<V> a, int *err
                     acc[r] = p[u];
                     cols[r] = col0 + (int)(in >> 16) * 32 + b;
                 }
+                c[u] = r;
             }
             if (__syncthreads_or(more != 0)) {
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     if (32 * (NW * u + w) >= total) break;
-                    if (!((more >> u) & 1u)) continue;
-                    const int k = c[u] >> 5;
-                    atomicAdd(&acc[(int)(info[k] & 0xffffu) + __popc(masks[k] & ((1u << (c[u] & 31)) - 1u))], p[u]);
+                    if ((more >> u) & 1u) atomicAdd(&acc[c[u]], p[u]);
                 }
                 __syncthreads();
             }
