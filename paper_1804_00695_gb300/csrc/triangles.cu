@@ -24,13 +24,15 @@
 // pairs only cost their construction and twice the bytes.
 //
 // Measured (one GB300, R-MAT scale 18, 16 edges a vertex, 0.65e9 lookups): 4.5
-// -> 1.55 ms.  Heavy rows 2.7 -> 1.21 ms (a warp took an entry k at a time, its
-// lanes the pairs of an L_k that mostly has fewer than 32), L 1.02 -> 0.16 ms
-// (counted, then filled, a hub's row by one warp 32 entries at a time), degrees
-// and labels 0.19 -> 0.06 ms (80,000 atomics on the bucket of degree 0).  Now
-// instruction issue bounds it, some 22 cycles an SM for 32 lookups.  A hub's
-// row as one block's work took 3.6 ms; tasks of 1024, 512 and 256 entries 1.65,
-// 1.25 and 1.21; blocks of 256 threads 1.29, of 1024 1.42.
+// -> 1.1 ms.  Heavy rows 2.7 -> 0.79 ms (a warp took an entry k at a time, its
+// lanes the pairs of an L_k that mostly has fewer than 32; 1.21 while a step
+// inside one row L_k looked its entry up like any other, 0.81 with four loads
+// of a lane in flight instead of six), L 1.02 -> 0.16 ms (counted, then filled,
+// a hub's row by one warp 32 entries at a time), degrees and labels 0.19 -> 0.06
+// ms (80,000 atomics on the bucket of degree 0).  Now instruction issue bounds
+// it, some 14 cycles an SM for 32 lookups.  A hub's row as one block's work took
+// 3.6 ms; tasks of 1024, 512 and 256 entries 1.65, 1.25 and 1.21; blocks of 256
+// threads 1.29, of 1024 1.42 (these before the steps inside one row).
 #include <climits>
 #include "internal.cuh"
 
@@ -44,7 +46,7 @@ constexpr int64_t TRI_SMEM_WORDS = 48 * 1024;   // 192 KB of bitmap in shared me
 constexpr int TRI_LONG = 1024;           // longer rows of the graph are taken by a block
 constexpr int TRI_TASK = 256;            // entries of a heavy row that a block takes at once
 constexpr int TRI_ROW_MAX = 1 << 20;     // 1024 rows of at most this many columns fit an int
-constexpr int TRI_U = 4;                 // loads of a lane in flight together
+constexpr int TRI_U = 6;                 // loads of a lane in flight together
 
 // deg[u] (clamped to n - 1 for rows with repeated columns) and its histogram
 // in hist[1 + deg] (hist[0] stays 0: the scan then gives bucket starts).
@@ -211,7 +213,9 @@ __global__ void k_tri_bins(int64_t n, const int32_t *__restrict__ lcol, const in
 // The columns of the rows L_k of a batch of entries k staged with the prefix
 // sums of their lengths (pre, padded with 33 INT_MAX; eq: start less the first
 // column's number), dealt out to a warp's share [tc, tend) of them, 32 a step:
-// hit(column) for each, by TRI_U steps whose loads are in flight together.
+// hit(column) for each, by TRI_U steps whose loads are in flight together.  Most
+// rows of a hub's entries are longer than a step: a step that ends before the
+// next row starts reads on in its row without looking anything up.
 template <typename Hit>
 __device__ __forceinline__ void tri_walk(const int *pre, const long long *eq, int ne, int tc, int tend, int total,
                                          const int32_t *__restrict__ lcol, int lane, Hit hit) {
@@ -223,6 +227,9 @@ __device__ __forceinline__ void tri_walk(const int *pre, const long long *eq, in
         e0 += __popc(m);
         if (m != 0xffffffffu) break;
     }
+    // the entry of the step's first column, and where the next one starts
+    const int32_t *row = lcol + eq[e0];
+    int next = pre[e0 + 1];
     for (; tc < tend; tc += 32 * TRI_U) {
         int c[TRI_U];
 #pragma unroll
@@ -230,11 +237,17 @@ __device__ __forceinline__ void tri_walk(const int *pre, const long long *eq, in
             const int tu = tc + 32 * u;
             c[u] = -1;
             if (tu >= tend) continue;   // uniform in the warp
+            if (tu + 32 < next) {   // (uniform) the step lies in one row, and so does the next one's start
+                if (tu + lane < total) c[u] = row[tu + lane];
+                continue;
+            }
             const int b = pre[e0 + 1 + lane] - tu;
             const unsigned m = __reduce_or_sync(0xffffffffu, b < 32 ? 1u << b : 0u);
             const int e = e0 + __popc(m & (2u * below + 1u));
             e0 += __popc(__ballot_sync(0xffffffffu, b <= 32));
             if (tu + lane < total) c[u] = lcol[eq[e] + (tu + lane)];
+            row = lcol + eq[e0];
+            next = pre[e0 + 1];
         }
 #pragma unroll
         for (int u = 0; u < TRI_U; u++)
