@@ -578,17 +578,20 @@ int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *
 // products are in rank.cu: the entries of A are staged with the prefix sums of
 // pairs(B_k), the entries that start within a step set a bit each, and a
 // pair's entry is the number of bits up to its lane; BM_U steps' loads are in
-// flight together.  Then the bitmap is counted and cleared 16 bytes at a time.
+// flight together.  A block's row meets long rows of B, so there a step that
+// ends before the next entry starts reads on without looking anything up (in a
+// warp's rows, of 18 pairs an entry, that cost 0.97 -> 1.10 ms).  Then the bitmap is counted and cleared 16 bytes at a time.
 // What bounds it: instruction issue and, in rows of a few hundred pairs, the
 // chain of loads A -> descriptors -> pairs.  Measured (one GB300, symbolic
 // second pass and the first pass whose rows mostly failed it, before -> now):
 // batch of 64 products of uniform rows (921,066 rows, 294 M products) 2.9 ->
-// 1.0 ms; A*A of an R-MAT graph, scale 17 8.8 -> 3.0 ms (block hash maps of
-// 8192 slots before), scale 13 1.2 -> 0.12 ms (a warp walked rows of up to
-// half a million pairs); 41,472 rows of 5,000 pairs 0.78 -> 0.35 ms.  The rows
+// 0.94 ms; A*A of an R-MAT graph, scale 17 8.8 -> 2.15 ms (block hash maps of
+// 8192 slots before; 2.8 without reading on, 2.2 with four loads in flight),
+// scale 13 1.2 -> 0.11 ms (a warp walked rows of up to half a million pairs);
+// 41,472 rows of 5,000 pairs 0.78 -> 0.35 ms.  The rows
 // are listed and counted without a list length on the host, so the call waits
 // for the device once instead of twice.
-constexpr int BM_U = 4, BM_WPB = 8;
+constexpr int BM_U = 8, BM_WPB = 8;
 
 struct BitmapP {
     const int64_t *arp; const int32_t *acol;
@@ -609,6 +612,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(BitmapP a, DevState *st) {
     constexpr bool WARP = NT == 32;
     constexpr int NW = NT / 32;
+    constexpr bool RUNS = !WARP;
     extern __shared__ __align__(16) unsigned bm_smem[];
     __shared__ int wsum[NW], wcnt[NW];
     __shared__ long long row_s;
@@ -686,6 +690,13 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
                     e0 += __popc(m);
                     if (m != 0xffffffffu) break;
                 }
+            // the entry of the step's first pair, and where the next one starts
+            const int2 *row = a.pairs;
+            int next = 0;
+            if (RUNS && tc < tend) {
+                row = a.pairs + eq[e0];
+                next = pre[e0 + 1];
+            }
             for (; tc < tend; tc += 32 * BM_U) {
                 int2 pr[BM_U];
 #pragma unroll
@@ -693,11 +704,19 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
                     const int tu = tc + 32 * u;
                     pr[u] = make_int2(lo, 0);
                     if (tu >= tend) continue;   // uniform in the warp
+                    if (RUNS && tu + 32 < next) {   // (uniform) one row of B, and it goes on
+                        if (tu + lane < total) pr[u] = row[tu + lane];
+                        continue;
+                    }
                     const int b = pre[e0 + 1 + lane] - tu;
                     const unsigned m = __reduce_or_sync(0xffffffffu, b < 32 ? 1u << b : 0u);
                     const int e = e0 + __popc(m & (2u * below + 1u));
                     e0 += __popc(__ballot_sync(0xffffffffu, b <= 32));
                     if (tu + lane < total) pr[u] = a.pairs[eq[e] + (tu + lane)];
+                    if (RUNS) {
+                        row = a.pairs + eq[e0];
+                        next = pre[e0 + 1];
+                    }
                 }
 #pragma unroll
                 for (int u = 0; u < BM_U; u++) {
