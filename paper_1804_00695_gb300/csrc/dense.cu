@@ -17,14 +17,17 @@
 //
 // What bounds it: shared-memory updates and the loads that feed them, about
 // 27 cycles an SM for 32 products where the update alone takes 9.4 (random
-// words), and 5 of the 14.4 ms below for staging and writing out windows.
+// words), and 5 of the 13.9 ms below for staging and writing out windows.
 // Measured (one GB300, FP32, A*A of an R-MAT graph of scale 17: 3.3e9
-// products in 39,071 rows of 8192 to 131,072 outputs): 40.8 -> 14.4 ms
+// products in 39,071 rows of 8192 to 131,072 outputs): 40.8 -> 13.9 ms
 // against a window kernel in which one lane walked each short part (loads of
 // a warp on 32 lines) and every product marked a bitmap. Of that: even dealing
 // 19.4, permuted slots 16.7, rows handed out one at a time 14.7, two blocks
-// of 512 threads an SM and strips of 64 14.4. Blocks of 256 threads over 44
-// KB took 19.4 before the last two.
+// of 512 threads an SM and strips of 64 14.4, the flat products loaded in
+// place 13.9. Blocks of 256 threads over 44 KB took 19.4 before the last
+// three. Everything flat, steps inside one part read on without a lookup,
+// takes 15.1 (and 5.8 for 6.3 ms on 41,448 FP64 rows of 16,000 products whose
+// parts have about 50), strips of 128 14.0 (6.7).
 #include <climits>
 #include "internal.cuh"
 
@@ -205,8 +208,11 @@ __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
                 for (int x = tid; x < 33; x += T) pre[ne + x] = INT_MAX;   // a step looks 32 parts ahead
                 if (tid == 0) str[ne] = strips;
                 __syncthreads();
-                // Both loops load one step ahead of the updates: a warp would
-                // otherwise wait for its loads, then for its updates, in turn.
+                // The strips are loaded one ahead of the updates: a warp would
+                // otherwise wait for its loads, then for its updates, in turn
+                // (few rows show it: 2148 of them 0.23 against 0.27 ms).  The
+                // flat products are not: what they find their parts with and
+                // hold a step ahead costs more than the wait.
                 auto add = [&](const int (&cc)[U], const V (&vv)[U], V av1) {
 #pragma unroll
                     for (int u = 0; u < U; u++) {
@@ -262,12 +268,20 @@ __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
                     int tc = w * pw * 32;
                     const int tend = min(total, tc + pw * 32);
                     int e0 = -1;
-                    // products tc + lane, tc + 32 + lane, ...: columns, values of B and parts (-1: none)
-                    auto load = [&](int t0, int (&cc)[F], V (&vv)[F], int (&ee)[F]) {
+                    if (tc < tend) {
+                        for (int x = 0; x < ne; x += 32) {
+                            const unsigned m = __ballot_sync(0xffffffffu, x + lane < ne && pre[x + lane] <= tc);
+                            e0 += __popc(m);
+                            if (m != 0xffffffffu) break;
+                        }
+                    }
+                    for (; tc < tend; tc += 32 * F) {
+                        int c[F];
+                        V v[F], av1[F];
 #pragma unroll
                         for (int u = 0; u < F; u++) {
-                            const int tu = t0 + 32 * u;
-                            ee[u] = -1;
+                            const int tu = tc + 32 * u;
+                            c[u] = -1;
                             if (tu >= tend) continue;   // uniform in the warp
                             const int b = pre[e0 + 1 + lane] - tu;
                             const unsigned m = __reduce_or_sync(0xffffffffu, b < 32 ? 1u << b : 0u);
@@ -275,35 +289,17 @@ __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
                             e0 += __popc(__ballot_sync(0xffffffffu, b <= 32));
                             if (tu + lane < total) {
                                 const long long q = eq[e] + (tu + lane);
-                                ee[u] = e;
-                                cc[u] = bcol[q];
-                                vv[u] = bval[q];
+                                c[u] = bcol[q];
+                                v[u] = bval[q];
+                                av1[u] = ea[e];
                             }
                         }
-                    };
-                    auto add1 = [&](const int (&cc)[F], const V (&vv)[F], const int (&ee)[F]) {
 #pragma unroll
                         for (int u = 0; u < F; u++) {
-                            if (ee[u] < 0) continue;
-                            const unsigned at = (unsigned)cc[u] - (unsigned)w0;
-                            if (at < (unsigned)W) atomicAdd(&acc[dense_slot(at)], dense_prod(ea[ee[u]], vv[u]));
+                            if (c[u] < 0) continue;
+                            const unsigned at = (unsigned)c[u] - (unsigned)w0;
+                            if (at < (unsigned)W) atomicAdd(&acc[dense_slot(at)], dense_prod(av1[u], v[u]));
                             else flag |= DERR_COUNT;
-                        }
-                    };
-                    if (tc < tend) {
-                        for (int x = 0; x < ne; x += 32) {
-                            const unsigned m = __ballot_sync(0xffffffffu, x + lane < ne && pre[x + lane] <= tc);
-                            e0 += __popc(m);
-                            if (m != 0xffffffffu) break;
-                        }
-                        int c0[F], c1[F], k0[F], k1[F];
-                        V v0[F], v1[F];
-                        load(tc, c0, v0, k0);
-                        for (; tc < tend; tc += 64 * F) {
-                            load(tc + 32 * F, c1, v1, k1);
-                            add1(c0, v0, k0);
-                            load(tc + 64 * F, c0, v0, k0);
-                            add1(c1, v1, k1);
                         }
                     }
                 }
