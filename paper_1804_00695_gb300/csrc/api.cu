@@ -377,7 +377,7 @@ static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     L.ccnt = L.flops + align_up((size_t)n * 8);
     L.longs = L.ccnt + align_up((size_t)nb * 4);
     L.tmp = L.longs + align_up((size_t)nb * 4);
-    L.gws = L.tmp + align_up(scan_tmp_bytes(n));
+    L.gws = L.tmp + align_up(scan_binning_tmp_bytes(n));
     return L;
 }
 

@@ -286,6 +286,7 @@ __device__ __forceinline__ int64_t desc_start(int4 d) {
     return (int64_t)(((uint64_t)(unsigned)d.y << 32) | (uint64_t)(unsigned)d.x);
 }
 size_t scan_tmp_bytes(int64_t n);
+size_t scan_binning_tmp_bytes(int64_t n);   // launch_scan_binning
 // x[0..n] holds counts in x[1..n]; on return x is the exclusive prefix
 // (x[0] = 0); *total (device) = x[n].
 int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &c);
