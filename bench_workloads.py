@@ -176,6 +176,21 @@ def _oracle_rows_sample(a, b, fl, start, tol_tag, device_rows, label, seconds=CP
              "sample": f"{label}: rows [{r0}, {r1}) of C ({m} multiplications), {dt:.2f} s"}, par)
 
 
+def dense_numeric_rows(g, c_rp, flops):
+    """Rows of g*g that the dense windows take (g's rows sorted): bins 5 and 6
+    with more than 8192 outputs, or with more than 6144 products and one per 8
+    columns of the row's span of 32-column blocks (num_cls)."""
+    rp, col = np.asarray(g.row_ptr, dtype=np.int64), g.col.astype(np.int64)
+    some = np.diff(rp) > 0
+    lo, hi = np.full(g.nrows, 1 << 40), np.full(g.nrows, -1)
+    lo[some], hi[some] = col[rp[:-1][some]] >> 5, col[rp[1:][some] - 1] >> 5
+    lo = bench._seg_reduce(np.minimum, lo[col], rp, 1 << 40)
+    words = np.maximum(bench._seg_reduce(np.maximum, hi[col], rp, -1) - lo + 1, 0)
+    nn = np.diff(c_rp)
+    return ((bench.bins_of(nn, flops) >= 5) & (words > 0) & (flops < 1 << 31)
+            & ((nn > 8192) | ((flops > 6144) & (flops * 8 >= words * 32))))
+
+
 # ---------------------------------------------------------------- R-MAT
 def measure_rmat(args, g, local):
     """C = A*A on the R-MAT graph: GFLOP/s, % of the HBM-byte roofline, the
@@ -234,9 +249,13 @@ def measure_rmat(args, g, local):
             mask = nar
         elif lab == "small":
             mask = (bb == 1) | (bb == 2)
+        elif lab == "dense":
+            mask = dense_numeric_rows(g, crp, fl)
         elif lab.startswith("bin"):
             mask = bb == int(lab[3:4])
         else:
+            continue
+        if lab == "dense" and mask.sum() * nl != nrows:
             continue
         kern.append((tms / nl, key, bench.kernel_bytes(g, g.row_ptr, crp, mask, 4, True), nl))
     roof = None

@@ -310,8 +310,7 @@ SPGEMM_API int spgemm_managed_free(void *ptr);
  * triangle-counting experiment of Section 4.1, after Wolf et al.): the
  * vertices are relabelled in order of non-decreasing degree, L is the
  * strictly lower triangle of the relabelled pattern, and the number of
- * triangles is the sum of (L*L) masked by L, computed as L x compressed(L)
- * (Section 2.1's column compression of the right-hand operand).
+ * triangles is the sum of (L*L) masked by L.
  * A: device CSR, the symmetric pattern of the graph without self loops
  * (values unused; a self loop is ignored).  *total (host): the number of
  * triangles.  perm (device, nrows int64, may be NULL): the label of every
