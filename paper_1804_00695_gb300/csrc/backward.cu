@@ -12,6 +12,7 @@
 // Rows of C with at most BWD_CAP entries are searched in a copy of their
 // columns in shared memory (a warp per row, products dealt out over the
 // lanes); longer rows are searched in global memory.
+#include <climits>
 #include "internal.cuh"
 
 namespace sg {
@@ -30,10 +31,16 @@ __device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int
 // A warp per row of A whose row of C has at most BWD_CAP entries: the
 // columns of C_i are copied to shared memory, the products a_ik * b_kj of
 // the row are dealt out over the lanes through prefix sums of nnz(B_k)
-// (stored a_ik staged BWD_E at a time), each lane finds dC_ij by binary
-// search in the copy, adds its dA term into the staged entry's accumulator
-// and its dB term atomically into db.
-constexpr int BWD_CAP = 1024, BWD_WPB = 8, BWD_E = 32;
+// (stored a_ik staged BWD_E at a time; a step's entries from the starts
+// within it, as in rank.cu), each lane finds dC_ij by binary search in the
+// copy, adds its dA term into the staged entry's accumulator and its dB term
+// atomically into db.
+// What bounds it: the chain B's column -> search -> dC.  BWD_U steps go
+// through it together: their loads of B, then their searches (as many halvings
+// for every lane), then their loads of dC.  Measured (one GB300, FP32): 20,001
+// rows of about 320 products 101 -> 80 us (two steps together 87, six 95).
+constexpr int BWD_CAP = 1024, BWD_WPB = 8, BWD_E = 32, BWD_U = 4;
+constexpr int BWD_ROW_MAX = 1 << 20;   // entries of a row of B taken (32 of them fit an int; a row of C holds fewer)
 
 template <typename V>
 __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
@@ -45,13 +52,14 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
     __shared__ long long eq0_all[BWD_WPB * BWD_E];
     __shared__ V ea_all[BWD_WPB * BWD_E];
     __shared__ V dacc_all[BWD_WPB * BWD_E];
-    __shared__ int pre_all[BWD_WPB * (BWD_E + 1)];
+    __shared__ int pre_all[BWD_WPB * BWD_E];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int *cs = cs_all + w * BWD_CAP;
     long long *eq0 = eq0_all + w * BWD_E;
     V *ea = ea_all + w * BWD_E;
     V *dacc = dacc_all + w * BWD_E;
-    int *pre = pre_all + w * (BWD_E + 1);
+    int *pre = pre_all + w * BWD_E;
+    const unsigned below = (1u << lane) - 1u, upto = 2u * below + 1u;
     bool missing = false;
     for (int64_t i = (int64_t)blockIdx.x * BWD_WPB + w; i < nrows; i += (int64_t)gridDim.x * BWD_WPB) {
         const int64_t c0 = crp[i];
@@ -65,12 +73,11 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
         __syncwarp();
         for (int pb = 0; pb < plen; pb += BWD_E) {
             int len = 0;
+            int64_t q0 = 0;
             if (pb + lane < plen) {
                 const int k = acol[p0 + pb + lane];
-                const int64_t q0 = brp[k];
-                eq0[lane] = q0;
-                len = (int)(brp[k + 1] - q0);
-                ea[lane] = aval ? aval[p0 + pb + lane] : V(0);
+                q0 = brp[k];
+                len = (int)min(brp[k + 1] - q0, (int64_t)BWD_ROW_MAX);
             }
             dacc[lane] = V(0);
             int incl = len;
@@ -78,49 +85,81 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
                 const int y = __shfl_up_sync(0xffffffffu, incl, d);
                 if (lane >= d) incl += y;
             }
-            pre[lane] = incl - len;
-            if (lane == 31) pre[BWD_E] = incl;
+            // the entries with a row of B, in order
+            const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+            const int pos = __popc(some & below), ne = __popc(some);
+            if (len > 0) {
+                pre[pos] = incl - len;
+                eq0[pos] = q0 - (incl - len);
+                ea[pos] = aval ? aval[p0 + pb + lane] : V(0);
+            }
             const int total = __shfl_sync(0xffffffffu, incl, 31);
             __syncwarp();
-            int e = 0;
-            for (int t0 = 0; t0 < total; t0 += 32) {
-                const int t = t0 + lane;
-                V term = V(0);
-                const bool live = t < total;
-                if (live) {
-                    while (pre[e + 1] <= t) e++;
-                    const int64_t q = eq0[e] + (t - pre[e]);
-                    const int j = bcol[q];
-                    int lo = 0, hi = nc;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (cs[mid] < j) lo = mid + 1;
-                        else hi = mid;
-                    }
-                    if (lo < nc && cs[lo] == j) {
-                        const V g = dc[c0 + lo];
-                        if (bval) term = g * bval[q];
-                        if (db) atomicAdd(&db[q], ea[e] * g);
-                    } else {
-                        missing = true;
+            const int at = lane < ne ? pre[lane] : INT_MAX;   // first product of entry `lane`
+            for (int t0 = 0; t0 < total; t0 += 32 * BWD_U) {
+                long long q[BWD_U];
+                int e[BWD_U], j[BWD_U], lo[BWD_U];
+                unsigned m[BWD_U];
+                V bv[BWD_U], g[BWD_U];
+#pragma unroll
+                for (int u = 0; u < BWD_U; u++) {
+                    const int tc = t0 + 32 * u;
+                    e[u] = -1;
+                    j[u] = lo[u] = 0;
+                    bv[u] = V(0);
+                    if (tc >= total) continue;   // uniform in the warp
+                    const int b = at - tc;
+                    m[u] = __reduce_or_sync(0xffffffffu, (unsigned)b < 32u ? 1u << b : 0u);
+                    const int ee = __popc(__ballot_sync(0xffffffffu, b < 0)) + __popc(m[u] & upto) - 1;
+                    if (tc + lane < total) {
+                        e[u] = ee;
+                        q[u] = eq0[ee] + (tc + lane);
+                        j[u] = bcol[q[u]];
+                        if (bval) bv[u] = bval[q[u]];
                     }
                 }
-                if (bval) {
-                    // the lanes of one staged a_ik are consecutive: a segmented
-                    // sum over them leaves its dA term in the segment's first
-                    // lane, which alone updates the entry's accumulator
-                    const unsigned grp = __match_any_sync(0xffffffffu, live ? e : -1 - lane);
-                    const int last = 31 - __clz(grp);
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const V y = __shfl_down_sync(0xffffffffu, term, d);
-                        if (lane + d <= last) term += y;
+                for (int n = nc; n > 1;) {
+                    const int half = n >> 1;
+#pragma unroll
+                    for (int u = 0; u < BWD_U; u++) lo[u] += cs[lo[u] + half - 1] < j[u] ? half : 0;
+                    n -= half;
+                }
+#pragma unroll
+                for (int u = 0; u < BWD_U; u++) {
+                    g[u] = V(0);
+                    if (e[u] < 0) continue;
+                    if (lo[u] < nc && cs[lo[u]] < j[u]) lo[u]++;
+                    if (lo[u] < nc && cs[lo[u]] == j[u]) {
+                        g[u] = dc[c0 + lo[u]];
+                    } else {
+                        missing = true;
+                        e[u] = -1 - e[u] - 1;   // (no term, but still of its entry)
                     }
-                    if (live && lane == __ffs(grp) - 1) dacc[e] += term;
-                    __syncwarp();
+                }
+#pragma unroll
+                for (int u = 0; u < BWD_U; u++) {
+                    const int tc = t0 + 32 * u;
+                    if (tc >= total) break;
+                    if (db && e[u] >= 0) atomicAdd(&db[q[u]], ea[e[u]] * g[u]);
+                    if (bval) {
+                        // the lanes of one staged a_ik are consecutive: a segmented
+                        // sum over them leaves its dA term in the segment's first
+                        // lane, which alone updates the entry's accumulator
+                        V term = e[u] >= 0 ? g[u] * bv[u] : V(0);
+                        const unsigned after = m[u] & ~upto;
+                        const int last = after ? __ffs(after) - 2 : min(31, total - 1 - tc);
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const V y = __shfl_down_sync(0xffffffffu, term, d);
+                            if (lane + d <= last) term += y;
+                        }
+                        const int ee = e[u] >= 0 ? e[u] : -2 - e[u];
+                        if (tc + lane < total && (lane == 0 || (m[u] >> lane & 1u))) dacc[ee] += term;
+                        __syncwarp();
+                    }
                 }
             }
             __syncwarp();
-            if (da && pb + lane < plen) da[p0 + pb + lane] = dacc[lane];
+            if (da && pb + lane < plen) da[p0 + pb + lane] = len > 0 ? dacc[pos] : V(0);
             __syncwarp();
         }
     }
