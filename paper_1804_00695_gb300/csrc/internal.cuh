@@ -34,6 +34,8 @@ enum : int {
     DERR_WINDOW = 8,      // chunked: a column of A outside the rows of B copied for its part
 };
 
+constexpr int CLS_SLOTS = 24;   // classes the device state has room for
+
 struct DevState {          // lives in device memory, one per handle
     int err;
     int b_out_of_range;    // B holds values outside the double-word range
@@ -49,9 +51,9 @@ struct DevState {          // lives in device memory, one per handle
     unsigned long long triangles;   // spgemm_triangles: the count
     // numeric rows by class (NumCls): rows, list cursors, largest row of C,
     // largest column span in 32-column blocks
-    long long cls_count[16];
-    long long cls_cursor[16];
-    int cls_nnz[16], cls_words[16];
+    long long cls_count[CLS_SLOTS];
+    long long cls_cursor[CLS_SLOTS];
+    int cls_nnz[CLS_SLOTS], cls_words[CLS_SLOTS];
     unsigned long long next_row;   // rows a kernel has handed out (cleared before it)
     // symbolic phase: whether the 32-slot maps have rows, whether rows are
     // marked for bitmaps; rows of a warp's bitmap, rows of a block's bitmap
@@ -127,7 +129,9 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //   CLS_NARROW  BIN_NARROW (a list only when other rows lie between them)
 //   CLS_RANK_W  at most RANK_W_FLOPS products over at most RANK_M_WORDS blocks
 //   CLS_RANK_S  at most RANK_S_NNZ outputs over at most RANK_S_WORDS blocks
-//   CLS_RANK_M4, CLS_RANK_M5  wider spans up to RANK_M_WORDS blocks: rows
+//   CLS_RANK_V  at most RANK_V_FLOPS products over wider spans up to
+//               RANK_M_WORDS blocks
+//   CLS_RANK_M4, CLS_RANK_M5  other rows over spans up to RANK_M_WORDS blocks: rows
 //               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
 //   CLS_WIDE3 .. CLS_WIDE4C   other rows of bins 3 and 4 by outputs
 //   CLS_BLOCK, CLS_HUGE       other rows of bins 5 and 6
@@ -135,17 +139,21 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //               accumulators hold, or many products over their span
 // Why the lines lie there: 512 products are eight a lane for the two warps of
 // a short row (rank.cu has both sides; 8192 blocks keep its first bitmap
-// within 1.5 KB); 2048 blocks are the bitmap that 128 threads scan in
+// within 1.5 KB), 1024 eight for four warps (13,774 rows of 513 to 1024 FP32
+// products over 3125 blocks 228 -> 89 us against CLS_RANK_M4; within 2048
+// blocks CLS_RANK_S is the faster, 0.66 against 0.73 ms for 124,998 rows);
+// 2048 blocks are the bitmap that 128 threads scan in
 // one step of 16 words, 8192 the one that 512 threads do; a row of 8192 FP64
 // outputs over 8192 blocks takes 167 KB of shared memory, the next power of
 // two would not fit.  Below them the rank accumulators measured 2.6-5x
 // faster than the maps and windows (rank.cu has the figures).
 enum NumCls {
-    CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_W, CLS_RANK_S, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
+    CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_W, CLS_RANK_S, CLS_RANK_V, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
     CLS_BLOCK, CLS_DENSE, CLS_HUGE, CLS_NARROW, NCLS
 };
+static_assert(NCLS <= CLS_SLOTS, "DevState keeps the classes' counts");
 constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
-constexpr int RANK_W_FLOPS = 512;
+constexpr int RANK_W_FLOPS = 512, RANK_V_FLOPS = 1024;
 constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit 32 bits)
 // Dense windows from one product per 8 columns of the span on (their cost per
 // row is the span written out plus the products, the rank accumulators' the
@@ -167,6 +175,7 @@ __host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, 
     if (words > 0 && flops <= RANK_FLOPS) {
         if (flops <= RANK_W_FLOPS && words <= RANK_M_WORDS) return CLS_RANK_W;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_S_WORDS) return CLS_RANK_S;
+        if (flops <= RANK_V_FLOPS && words <= RANK_M_WORDS) return CLS_RANK_V;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_M_WORDS) return CLS_RANK_M4;
         if (nnz <= RANK_M_NNZ && words <= RANK_M_WORDS) return CLS_RANK_M5;
     }
@@ -391,9 +400,9 @@ size_t window_global_ws(int64_t max_alen, int nsm);
 
 // rank.cu: listed rows with a dense rank accumulator (a block each), in FP32
 // or native FP64; rows wider than max_words blocks or with more than max_nnz
-// outputs are skipped.  RANK_SHORT: rows of CLS_RANK_W; RANK_ROW: of
+// outputs are skipped.  RANK_SHORT: rows of CLS_RANK_W; RANK_MID: of CLS_RANK_V; RANK_ROW: of
 // CLS_RANK_S (or CLS_B2).
-enum RankSize { RANK_SHORT, RANK_ROW, RANK_LONG };
+enum RankSize { RANK_SHORT, RANK_MID, RANK_ROW, RANK_LONG };
 int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
                     const int2 *rspan, const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz,
                     int64_t max_words, int *err, Ctx &c);

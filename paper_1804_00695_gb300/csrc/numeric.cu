@@ -1682,15 +1682,18 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                                              k == CLS_WINDOW_B ? "numeric.window_block" : "numeric.window_warp", err, c));
                 break;
             case CLS_RANK_W:
-                if (short_with_rows) break;   // one launch with the next list
+            case CLS_RANK_V:
+                if (k == CLS_RANK_W && short_with_rows) break;   // one launch with the next list
                 if (MODE != MODE_DW) {
-                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, RANK_SHORT, cls.nnz[k], cls.words[k], err, c));
+                    SG_TRY(launch_num_rank(DT, A, B, C, bdesc, rspan, r, cnt, k == CLS_RANK_W ? RANK_SHORT : RANK_MID,
+                                           cls.nnz[k], cls.words[k], err, c));
                     break;
                 }
-                SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
+                if (k == CLS_RANK_W) SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
                 if (cls.words[k] > RANK_S_WORDS) {
                     SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
                     SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
+                    SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
                 }
                 break;
             case CLS_B2:

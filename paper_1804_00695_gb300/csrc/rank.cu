@@ -348,8 +348,8 @@ static int run_rank_block(const RankP<V> &p, int *err, const char *label, Ctx &c
 }
 
 // ---------------------------------------------------------------- short rows
-// Rows of at most RANK_W_FLOPS products: T threads per row, the products in
-// their registers, and the bitmap of the span in two levels.  A first bitmap
+// Rows of at most F products: T threads per row (RANK_W_FLOPS with two warps,
+// RANK_V_FLOPS with four), the products in their registers, and the bitmap of the span in two levels.  A first bitmap
 // holds a bit per 32-column block of the span; its prefix counts number the
 // row's non-empty blocks, and only these get a word of the second bitmap.  So
 // what is cleared and scanned is a word per 1024 columns and a word per
@@ -370,7 +370,8 @@ static int run_rank_block(const RankP<V> &p, int *err, const char *label, Ctx &c
 // loads and barriers behind it.  Measured (one GB300, FP32): 795,129 rows of
 // 64 products of up to 65,536 columns, with the block kernel's 124,998 longer
 // ones, 3.47 -> 3.00 ms; 86,197 such rows over 100,000 columns (spans that the
-// 128-thread block's bitmap does not hold) 1.36 -> 0.50 ms; FP64, 299,537
+// 128-thread block's bitmap does not hold) 1.36 -> 0.36 ms with the 13,774 of
+// 513 to 1024 products beside them; FP64, 299,537
 // rows with 48,168 longer ones, 1.45 -> 1.22 ms.  Two warps a row: a warp
 // with 16 products a lane takes 3.04 ms for the first (its code no longer
 // fits the instruction cache), 128 threads with four a lane 2.83; 96 threads
@@ -401,10 +402,10 @@ struct RankWSmem {
 };
 
 // bw, nmax of the parameters: words of the first bitmap, outputs.
-template <typename V, typename Q, int T, int MINB>
+template <typename V, typename Q, int T, int F, int MINB>
 __global__ void __launch_bounds__(T, MINB) k_num_rank_short(RankP<V> a, int *err) {
-    constexpr int NW = T / 32, U = RANK_W_FLOPS / T, UB = U < 8 ? U : 8;
-    static_assert(U * T == RANK_W_FLOPS && U % UB == 0, "whole slots");
+    constexpr int NW = T / 32, U = F / T, UB = 8;
+    static_assert(U * T == F && U % UB == 0, "whole slots");
     extern __shared__ __align__(16) unsigned char mem[];
     __shared__ int s_nz, s_done;
     const RankWSmem<V> L(a.bw, a.nmax);
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(T, MINB) k_num_rank_short(RankP<V> a, int *err
             }
             const int incl = scan(len), tot = __shfl_sync(0xffffffffu, incl, 31);
             const unsigned some = __ballot_sync(0xffffffffu, len > 0);
-            fits = tot <= RANK_W_FLOPS - total && __all_sync(0xffffffffu, len <= RANK_W_FLOPS);
+            fits = tot <= F - total && __all_sync(0xffffffffu, len <= F);
             if (!fits) break;   // A or B changed since the symbolic phase
             if (pb > 0) __syncthreads();
             if (w == 0 && len > 0) {
@@ -602,25 +603,30 @@ __global__ void __launch_bounds__(T, MINB) k_num_rank_short(RankP<V> a, int *err
     if (flag) atomicOr(err, flag);
 }
 
+template <typename V, typename Q, int T, int F, int MINB>
+static int run_rank_short(const RankP<V> &p, int *err, const char *label, Ctx &c) {
+    auto kern = k_num_rank_short<V, Q, T, F, MINB>;
+    const size_t smem = RankWSmem<V>(p.bw, p.nmax).bytes;
+    int per_sm = 0;
+    SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
+    const int64_t blocks = std::min<int64_t>(p.count, (int64_t)per_sm * c.nsm);
+    c.begin(label, p.count);
+    kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);
+    c.end();
+    SG_CUDA(cudaGetLastError());
+    return SPGEMM_OK;
+}
+
 template <typename V, typename Q>
 static int num_rank(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc, const int2 *rspan,
                     const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz, int64_t max_words, int *err,
                     Ctx &c) {
-    if (size == RANK_SHORT) {
-        constexpr int T = 64;
+    if (size == RANK_SHORT || size == RANK_MID) {
         RankP<V> p{A.row_ptr, A.col_idx, (const V *)A.values, B.col_idx, (const V *)B.values,
                    C.row_ptr, C.col_idx, (V *)C.values, bdesc, rspan, rows, count,
                    (int)((max_words + 31) / 32), (int)max_nnz};
-        auto kern = k_num_rank_short<V, Q, T, 16>;
-        const size_t smem = RankWSmem<V>(p.bw, p.nmax).bytes;
-        int per_sm = 0;
-        SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
-        const int64_t blocks = std::min<int64_t>(count, (int64_t)per_sm * c.nsm);
-        c.begin("numeric.rank_short", count);
-        kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);
-        c.end();
-        SG_CUDA(cudaGetLastError());
-        return SPGEMM_OK;
+        if (size == RANK_SHORT) return run_rank_short<V, Q, 64, RANK_W_FLOPS, 16>(p, err, "numeric.rank_short", c);
+        return run_rank_short<V, Q, 128, RANK_V_FLOPS, 8>(p, err, "numeric.rank_mid", c);
     }
     const int bw = (int)((max_words + 15) & ~(int64_t)15);
     RankP<V> p{A.row_ptr, A.col_idx, (const V *)A.values, B.col_idx, (const V *)B.values,
