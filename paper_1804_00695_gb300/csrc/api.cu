@@ -484,7 +484,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
                          ? std::max(numeric_global_ws(h->max_row_nnz, B->ncols, h->nsm, SPGEMM_F64),
                                     window_global_ws(h->max_alen, h->nsm))
                          : 0;
-        if (h->cls.count[CLS_DENSE]) h->num_gws = std::max(h->num_gws, dense_bytes);
+        if (h->cls.count[CLS_DENSE]) h->num_gws = std::max(h->num_gws, dense_bytes + dense_fold_ws(h->max_alen, h->nsm));
         h->num_lists = 0;
         // numeric scratch: B split into double-words, then the second-level maps
         SG_TRY(ws_reserve(h, L.persist + align_up((size_t)B->nnz * 8) + h->num_gws, s, L.persist));

@@ -81,7 +81,17 @@ struct DenseP {
     int64_t count;
     int W, nwin;
     unsigned long long *next;   // rows handed out so far
+    V *fold;                    // W sums for every block (null: none)
 };
+
+// In FP32 a slot takes the terms of at most DENSE_FOLD batches of a row's
+// entries before the window is added to sums of its own in global memory (L2):
+// a hub's entries are sums of tens of thousands of terms, and the rounding of
+// one long chain of additions grows with its length.  A*A of an R-MAT graph of
+// scale 17 against 64 bits (2-norms): 3.6e-7 to 1.2e-6 -> 1.6e-7, for 13.9 ->
+// 14.2 ms.  FP64 goes without: its registers would spill (6.3 -> 7.1 ms at
+// scale 16), and its chains keep far more digits than the result needs.
+constexpr int DENSE_FOLD = 4;
 
 template <typename V, int T>
 struct DenseSmem {
@@ -103,6 +113,7 @@ constexpr int DENSE_STRIP_L = 6, DENSE_STRIP = 1 << DENSE_STRIP_L;   // entries 
 template <typename V, int T, int MINB>
 __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
     constexpr int NW = T / 32, U = DENSE_STRIP / 32, F = 2, VW = 16 / (int)sizeof(V);   // values per 16 bytes
+    constexpr bool FOLDS = sizeof(V) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int wsum[NW], wcnt[NW], wstr[NW];
     __shared__ long long row_s;
@@ -165,6 +176,8 @@ __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
         if (single) entry(tid, j0);
         for (int j = j0; j <= j1 && j < a.nwin; j++) {
             const int64_t w0 = (int64_t)j * W;
+            bool folded = false;
+            V *sums = FOLDS && a.fold ? a.fold + (int64_t)blockIdx.x * W : nullptr;
             for (int pb = 0; pb < plen; pb += T) {
                 // stage the parts of up to T rows of B inside the window (empty ones left out)
                 if (!single) entry(pb + tid, j);
@@ -304,6 +317,19 @@ __global__ void __launch_bounds__(T, MINB) k_num_dense(DenseP<V> a, int *err) {
                     }
                 }
                 __syncthreads();
+                // (an empty slot is -0.0, which an addition leaves as it is)
+                if (FOLDS && sums && pb + T < plen && (pb / T + 1) % DENSE_FOLD == 0) {
+                    for (int x = tid; x < W; x += T) {
+                        sums[x] = folded ? sums[x] + acc[x] : acc[x];
+                        acc[x] = dense_empty(V(0));
+                    }
+                    folded = true;
+                    __syncthreads();
+                }
+            }
+            if (FOLDS && folded) {
+                for (int x = tid; x < W; x += T) acc[x] = sums[x] + acc[x];
+                __syncthreads();
             }
             // entries of each warp's runs, then their places
             int n = 0;
@@ -361,8 +387,11 @@ constexpr int64_t dense_most() { return 88 * 1024 / (int64_t)sizeof(V); }
 size_t dense_ws(int64_t nrows_b, int64_t ncols_b) {
     int W, nwin;
     dense_windows(ncols_b, dense_most<double>(), W, nwin);
-    return (size_t)nrows_b * (size_t)(nwin - 1) * 4;
+    return ((size_t)nrows_b * (size_t)(nwin - 1) * 4 + 255) & ~(size_t)255;
 }
+// The windows' sums of all blocks that fit the chip (no more than its shared
+// memory), when a row of A has more than the batches of one fold.
+size_t dense_fold_ws(int64_t max_alen, int nsm) { return max_alen > 256 * DENSE_FOLD ? (size_t)nsm * (228 << 10) : 0; }
 
 template <typename V>
 static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc, const int2 *rspan,
@@ -383,13 +412,16 @@ static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, co
         SG_CUDA(cudaGetLastError());
     }
     DenseP<V> p{A.row_ptr, A.col_idx, (const V *)A.values, B.col_idx, (const V *)B.values, C.row_ptr, C.col_idx,
-                (V *)C.values, bdesc, rspan, rows, split, count, W, nwin, next};
+                (V *)C.values, bdesc, rspan, rows, split, count, W, nwin, next, nullptr};
+    const size_t used = ((size_t)cells * 4 + 255) & ~(size_t)255;
     SG_CUDA(cudaMemsetAsync(next, 0, sizeof(*next), c.s));
     auto go = [&](auto kern, int T, size_t smem) -> int {
         int per_sm = 0;
         SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
+        const int64_t blocks = std::min<int64_t>(count, (int64_t)per_sm * c.nsm);
+        if (sizeof(V) == 4 && used + (size_t)blocks * W * sizeof(V) <= ws_bytes) p.fold = (V *)((char *)ws + used);
         c.begin("numeric.dense", count);
-        kern<<<(unsigned)std::min<int64_t>(count, (int64_t)per_sm * c.nsm), T, smem, c.s>>>(p, err);
+        kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);
         c.end();
         SG_CUDA(cudaGetLastError());
         return SPGEMM_OK;

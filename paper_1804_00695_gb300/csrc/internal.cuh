@@ -410,6 +410,7 @@ int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_
 // dense.cu: listed rows over windows of a dense accumulator (rows of B
 // sorted); dense_ws: bytes of the split table (either type); next: device counter.
 size_t dense_ws(int64_t nrows_b, int64_t ncols_b);
+size_t dense_fold_ws(int64_t max_alen, int nsm);   // behind the table
 int launch_num_dense(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
                      const int2 *rspan, const int32_t *rows, int64_t count, void *ws, size_t ws_bytes,
                      unsigned long long *next, int *err, Ctx &c);
