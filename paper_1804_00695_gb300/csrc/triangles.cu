@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(T) k_tri_heavy(
                         rc += (bm[c >> 5] >> (c & 31)) & 1u;
                     }
                 }
+                __syncthreads();   // the bits are cleared once every warp has looked its columns up
                 continue;
             }
             int incl = d.z;
