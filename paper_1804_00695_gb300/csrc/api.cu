@@ -357,7 +357,7 @@ static int widen(int lanes, int64_t rows, double work, int nsm) {
 // overlap it.
 struct WsLayout {
     size_t bins, cls, rows, desc, mm, spans, nlo, nwords, ulist, persist;   // persistent
-    size_t ana, flops, pairs, ccnt, longs, tmp, gws;                   // symbolic scratch
+    size_t ana, flops, pairs, ccnt, longs, maps, tmp, gws;             // symbolic scratch
 };
 static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     WsLayout L;
@@ -376,7 +376,8 @@ static WsLayout ws_layout(int64_t n, int64_t nb, int64_t nnzb) {
     L.flops = L.pairs + align_up((size_t)nnzb * 8);
     L.ccnt = L.flops + align_up((size_t)n * 8);
     L.longs = L.ccnt + align_up((size_t)nb * 4);
-    L.tmp = L.longs + align_up((size_t)nb * 4);
+    L.maps = L.longs + align_up((size_t)nb * 4);
+    L.tmp = L.maps + align_up((size_t)n * 4);
     L.gws = L.tmp + align_up(scan_binning_tmp_bytes(n));
     return L;
 }
@@ -441,9 +442,11 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         } else {
             SG_TRY(launch_analyze(*A, *B, ana, minmax, flops, bins, C_row_ptr, rspan, h->dstate, bitmaps, c));
         }
-        SG_TRY(launch_symbolic_first(*A, bins, desc, pairs, C_row_ptr, rows, h->dstate, bitmaps, gs, c));
+        SG_TRY(launch_symbolic_first(*A, bins, desc, pairs, C_row_ptr, rows, (int32_t *)(w + L.maps), h->dstate, bitmaps,
+                                     gs, c));
         if (bitmaps) {
-            SG_TRY(launch_symbolic_bitmaps(*A, *B, desc, pairs, rspan, rows, C_row_ptr, h->dstate, c));
+            SG_TRY(launch_symbolic_bitmaps(*A, *B, desc, pairs, rspan, rows, (int32_t *)(w + L.maps), bins, C_row_ptr,
+                                           h->dstate, c));
         } else {
             SG_TRY(fetch_state(h, s));
             SG_TRY(device_errors(h->hstate->err));

@@ -56,9 +56,10 @@ struct DevState {          // lives in device memory, one per handle
     int cls_nnz[CLS_SLOTS], cls_words[CLS_SLOTS];
     unsigned long long next_row;   // rows a kernel has handed out (cleared before it)
     // symbolic phase: whether the 32-slot maps have rows, whether rows are
-    // marked for bitmaps; rows of a warp's bitmap, rows of a block's bitmap
+    // marked; rows of the warps, of the blocks' bitmaps and of the blocks' maps
     int sym_first, sym_marked;
-    unsigned long long sym_warp, sym_block;
+    unsigned long long sym_warp, sym_block, sym_map;   // sym_map: rows of a block's map
+    unsigned long long next_map;   // rows of those handed out
 };
 
 // ---------------------------------------------------------------- bins
@@ -70,20 +71,38 @@ constexpr int BIN_HUGE = 6;     // widest bin: unbounded accumulator
 constexpr int NBINS = SPGEMM_NBINS;
 
 // Symbolic phase of a B of at most SYM_BITMAP_WORDS blocks of 32 columns (its
-// bitmap fits a block's shared memory), rows that are not narrow: at most
-// SYM_FIRST_PAIRS compressed pairs: a 32-slot map, which holds them whatever
-// their blocks; more pairs over at most SYM_WARP_WORDS blocks and at most
-// SYM_WARP_PAIRS of them: a warp and a bitmap of the row's span (marked
-// SYM_MARK_WARP in crp[i+1] until counted); the others: a block and a bitmap
-// (SYM_MARK_BLOCK).  A wider B goes through the optimistic first pass and the
-// lists by bin.
+// bitmap fits a block's shared memory), rows that are not narrow, by their
+// compressed pairs and the blocks they span (sym_mark; the mark is kept in
+// crp[i+1] until the row is counted):
+//   at most SYM_FIRST_PAIRS pairs: a 32-slot map, which holds them whatever
+//     their blocks (no mark);
+//   SYM_MARK_WARP: up to SYM_WARP_PAIRS pairs over at most SYM_WARP_WORDS
+//     blocks: a warp and a bitmap of the span; up to SYM_MAP_PAIRS over more: a
+//     warp and a map;
+//   SYM_MARK_MAP: up to SYM_MAP_BLOCK_PAIRS pairs, and one for 12 blocks of the
+//     span, over more than SYM_MAP_BLOCK_WORDS: a block and a map;
+//   SYM_MARK_BLOCK: the others: a block and a bitmap.
+// Why the lines lie there (one GB300, whole symbolic call): a block's bitmap is
+// cleared and counted over the whole span, and from 24,576 blocks on one fills
+// an SM, so that rows go through it one at a time.  Bitmap -> map, rows over
+// 3000 / 12,000 / 50,000 blocks: 200,000 of 40 pairs 784 -> 373, 1613 -> 377,
+// 5509 -> 372 us; 78,125 of 256 417 -> 320, 738 -> 340, 2295 -> 350; 33,333 of
+// 600 265 (bitmap kept), 412 -> 376, 1082 -> 379; 20,000 of 1000 214 and 305
+// (kept), 729 -> 324; 10,000 of 2000 185, 232 (kept), 442 -> 308.
+// A wider B goes through the optimistic first pass and the lists by bin.
 constexpr int64_t SYM_BITMAP_WORDS = 53248;   // 208 KB
 constexpr int SYM_WARP_WORDS = 2048;
 constexpr long long SYM_FIRST_PAIRS = 32, SYM_WARP_PAIRS = 4096;
-constexpr int SYM_MARK_WARP = -1, SYM_MARK_BLOCK = -2;
+constexpr long long SYM_MAP_PAIRS = 256, SYM_MAP_BLOCK_PAIRS = 2048;
+constexpr int SYM_MAP_L = 9, SYM_MAP_BLOCK_L = 12;   // slots of their maps (log2): two for every pair
+constexpr int SYM_MAP_BLOCK_WORDS = 8192;
+static_assert((2 << SYM_MAP_L) <= SYM_WARP_WORDS, "a warp's map lies where its bitmap does");
+constexpr int SYM_MARK_WARP = -1, SYM_MARK_BLOCK = -2, SYM_MARK_MAP = -3;
 __host__ __device__ inline int sym_mark(long long cpairs, int words) {
     if (cpairs <= SYM_FIRST_PAIRS) return 0;
-    return cpairs <= SYM_WARP_PAIRS && words <= SYM_WARP_WORDS ? SYM_MARK_WARP : SYM_MARK_BLOCK;
+    if (words <= SYM_WARP_WORDS) return cpairs <= SYM_WARP_PAIRS ? SYM_MARK_WARP : SYM_MARK_BLOCK;
+    if (cpairs <= SYM_MAP_PAIRS) return SYM_MARK_WARP;
+    return words > SYM_MAP_BLOCK_WORDS && cpairs <= SYM_MAP_BLOCK_PAIRS && cpairs * 12 <= words ? SYM_MARK_MAP : SYM_MARK_BLOCK;
 }
 
 // Numeric bins by exact output count (and product count):
@@ -350,14 +369,17 @@ int launch_num_window(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgem
 // symbolic.cu
 // First pass over all rows with a 32-slot map and G lanes per row (rows of
 // bins EMPTY, HUGE and NARROW are skipped).  With bitmaps, marked rows are
-// skipped too and listed instead (room for all rows): those for a warp from
-// rows[0] on, those for a block from rows[nrows(A) - 1] downwards.
+// skipped too and listed instead (room for all rows in both lists): those for a
+// warp from rows[0] on, those for a block from rows[nrows(A) - 1] downwards,
+// those for a block's map in maps.
 int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
-                          int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, int G, Ctx &c);
-// The listed rows, counted over bitmaps of their span; no list length is
-// needed on the host.
+                          int64_t *crp, int32_t *rows, int32_t *maps, DevState *st, bool bitmaps, int G, Ctx &c);
+// The listed rows (the warps' and blocks' lists in rows, those of SYM_MARK_MAP in
+// maps), counted over bitmaps of their span or maps; no list length is needed
+// on the host.
 int launch_symbolic_bitmaps(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *pairs,
-                            const int2 *rspan, const int32_t *rows, int64_t *crp, DevState *st, Ctx &c);
+                            const int2 *rspan, const int32_t *rows, const int32_t *maps, const uint8_t *bins,
+                            int64_t *crp, DevState *st, Ctx &c);
 // Second pass: kernels of bins 2..6; counts[b] = rows in bin b (host),
 // rows = concatenated bin lists, rspan[i] = column-block span of row i.
 // Writes nnz(C_i) to crp[i+1].

@@ -7,7 +7,7 @@
 // When a bitmap of all column blocks of B fits shared memory (up to 1.7 M
 // columns), rows with at most 32 pairs take a 32-slot map, G lanes sharing the
 // row's stored a_ik, and the others a bitmap of their span, by a warp or a
-// block (k_sym_rows).
+// block, or, with few pairs over a wide span, a map of their blocks (k_sym_rows).
 //
 // With a wider B, rows are sized by an upper bound on their distinct blocks.
 // A first pass takes every row with bound <= 4096 in row order with the
@@ -60,7 +60,7 @@ __device__ __forceinline__ bool first_pass_empty(const DevState *st, bool bitmap
 // The marked rows' lists: a warp takes 32 rows at a time and reserves their
 // places with one atomic per list.
 __device__ __forceinline__ void list_marked(int64_t n, const int64_t *__restrict__ crp, int32_t *__restrict__ rows,
-                                            DevState *st) {
+                                            int32_t *__restrict__ maps, DevState *st) {
     if (*(volatile int *)&st->sym_marked == 0) return;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
@@ -68,13 +68,17 @@ __device__ __forceinline__ void list_marked(int64_t n, const int64_t *__restrict
          i0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = i0 + lane;
         const int64_t m = i < n ? crp[i + 1] : 0;
-        const unsigned mw = __ballot_sync(0xffffffffu, m == SYM_MARK_WARP), mb = __ballot_sync(0xffffffffu, m == SYM_MARK_BLOCK);
+        const unsigned mw = __ballot_sync(0xffffffffu, m == SYM_MARK_WARP), mb = __ballot_sync(0xffffffffu, m == SYM_MARK_BLOCK),
+                       mm = __ballot_sync(0xffffffffu, m == SYM_MARK_MAP);
         long long at = 0;
         if (lane == 0 && mw) at = (long long)atomicAdd(&st->sym_warp, (unsigned long long)__popc(mw));
         if (lane == 1 && mb) at = (long long)atomicAdd(&st->sym_block, (unsigned long long)__popc(mb));
-        const long long aw = __shfl_sync(0xffffffffu, at, 0), ab = __shfl_sync(0xffffffffu, at, 1);
+        if (lane == 2 && mm) at = (long long)atomicAdd(&st->sym_map, (unsigned long long)__popc(mm));
+        const long long aw = __shfl_sync(0xffffffffu, at, 0), ab = __shfl_sync(0xffffffffu, at, 1),
+                        am = __shfl_sync(0xffffffffu, at, 2);
         if (m == SYM_MARK_WARP) rows[aw + __popc(mw & below)] = (int32_t)i;
         if (m == SYM_MARK_BLOCK) rows[n - 1 - (ab + __popc(mb & below))] = (int32_t)i;
+        if (m == SYM_MARK_MAP) maps[am + __popc(mm & below)] = (int32_t)i;
     }
 }
 
@@ -82,7 +86,8 @@ template <int G>
 __global__ void __launch_bounds__(256) k_sym_first(
     int64_t n, const uint8_t *__restrict__ bins, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc,
-    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, DevState *st, bool bitmaps) {
+    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, int32_t *__restrict__ maps, DevState *st,
+    bool bitmaps) {
     using Lay = SymFirstLayout<G>;
     constexpr int S = Lay::S, L = 5, RPW = 32 / G, WPB = 8, PER = S / G;
     constexpr int E = Lay::E, EL = E / G, NR = WPB * RPW;
@@ -97,7 +102,7 @@ __global__ void __launch_bounds__(256) k_sym_first(
     int *pre = reg + Lay::o_pre;
     const unsigned lmask = (G == 32) ? 0xffffffffu : ((1u << G) - 1);
     const int64_t stride = (int64_t)gridDim.x * WPB * RPW;
-    if (bitmaps) list_marked(n, crp, rows, st);
+    if (bitmaps) list_marked(n, crp, rows, maps, st);
     if (first_pass_empty(st, bitmaps)) return;
     for (int64_t base = ((int64_t)blockIdx.x * WPB + w) * RPW; base < n; base += stride) {
         const int64_t i = base + g;
@@ -198,7 +203,8 @@ template <int G>
 __global__ void __launch_bounds__(256) k_sym_first_strided(
     int64_t n, const uint8_t *__restrict__ bins, const int64_t *__restrict__ arp,
     const int32_t *__restrict__ acol, const int4 *__restrict__ desc,
-    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, DevState *st, bool bitmaps) {
+    const int2 *__restrict__ pairs, int64_t *__restrict__ crp, int32_t *__restrict__ rows, int32_t *__restrict__ maps, DevState *st,
+    bool bitmaps) {
     using Lay = SymFirstLayout<G>;
     constexpr int S = Lay::S, L = 5, RPW = 32 / G, WPB = 8, PER = S / G;
     constexpr int E = Lay::E, EL = E / G, NR = WPB * RPW;
@@ -213,7 +219,7 @@ __global__ void __launch_bounds__(256) k_sym_first_strided(
     int *pre = reg + Lay::o_pre;
     const unsigned lmask = (G == 32) ? 0xffffffffu : ((1u << G) - 1);
     const int64_t stride = (int64_t)gridDim.x * WPB * RPW;
-    if (bitmaps) list_marked(n, crp, rows, st);
+    if (bitmaps) list_marked(n, crp, rows, maps, st);
     if (first_pass_empty(st, bitmaps)) return;
     for (int64_t base = ((int64_t)blockIdx.x * WPB + w) * RPW; base < n; base += stride) {
         const int64_t i = base + g;
@@ -539,7 +545,7 @@ static int prep(K kern, size_t smem) {
 
 template <int G>
 static int run_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
-                     int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, Ctx &c) {
+                     int64_t *crp, int32_t *rows, int32_t *maps, DevState *st, bool bitmaps, Ctx &c) {
     constexpr int GPB = 256 / G;   // rows per block: 8 warps x 32/G rows
     int64_t blocks = (A.nrows + GPB - 1) / GPB;
     // one resident wave striding over the rows: when the analysis left this
@@ -551,23 +557,23 @@ static int run_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc,
     c.begin("symbolic.first", A.nrows);
     if (G <= 8)
         k_sym_first_strided<G><<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, bins, A.row_ptr, A.col_idx, desc,
-                                                                  pairs, crp, rows, st, bitmaps);
+                                                                  pairs, crp, rows, maps, st, bitmaps);
     else
         k_sym_first<G><<<(unsigned)blocks, 256, 0, c.s>>>(A.nrows, bins, A.row_ptr, A.col_idx, desc,
-                                                       pairs, crp, rows, st, bitmaps);
+                                                       pairs, crp, rows, maps, st, bitmaps);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
 int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *desc, const int2 *pairs,
-                          int64_t *crp, int32_t *rows, DevState *st, bool bitmaps, int G, Ctx &c) {
+                          int64_t *crp, int32_t *rows, int32_t *maps, DevState *st, bool bitmaps, int G, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     switch (G) {
-        case 4: return run_first<4>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
-        case 8: return run_first<8>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
-        case 16: return run_first<16>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
-        default: return run_first<32>(A, bins, desc, pairs, crp, rows, st, bitmaps, c);
+        case 4: return run_first<4>(A, bins, desc, pairs, crp, rows, maps, st, bitmaps, c);
+        case 8: return run_first<8>(A, bins, desc, pairs, crp, rows, maps, st, bitmaps, c);
+        case 16: return run_first<16>(A, bins, desc, pairs, crp, rows, maps, st, bitmaps, c);
+        default: return run_first<32>(A, bins, desc, pairs, crp, rows, maps, st, bitmaps, c);
     }
 }
 
@@ -591,16 +597,38 @@ int launch_symbolic_first(const spgemm_csr &A, const uint8_t *bins, const int4 *
 // 41,472 rows of 5,000 pairs 0.78 -> 0.35 ms.  The rows
 // are listed and counted without a list length on the host, so the call waits
 // for the device once instead of twice.
+// MAP: rows over more blocks than the bitmap has (bw) put their pairs into a map
+// in its place: what is cleared and counted is then two slots for every pair and
+// not the span (internal.cuh has the rule and both sides).
 constexpr int BM_U = 8, BM_WPB = 8;
 
 struct BitmapP {
     const int64_t *arp; const int32_t *acol;
     const int4 *desc; const int2 *pairs; const int2 *rspan;
-    const int32_t *rows;
+    const int32_t *rows, *maps;
+    const uint8_t *bins;
     int64_t n;
     int64_t *crp;
     int bw;   // bitmap words (a multiple of 4)
 };
+
+// Adds a block's mask to a map of 2^L slots that is empty where all is zero
+// (keys are the blocks plus one); false if full.
+__device__ __forceinline__ bool sym_map_add(unsigned *keys, unsigned *masks, int L, int blk, unsigned m) {
+    const unsigned key = (unsigned)blk + 1u, msk = (1u << L) - 1u;
+    unsigned h = hash_slot(blk, L);
+#pragma unroll 1
+    for (unsigned probe = 0; probe <= msk; probe++) {
+        unsigned k = ((volatile unsigned *)keys)[h];
+        if (k == 0u) k = atomicCAS(&keys[h], 0u, key);
+        if (k == 0u || k == key) {
+            atomicOr(&masks[h], m);
+            return true;
+        }
+        h = (h + 1u) & msk;
+    }
+    return false;
+}
 
 template <int NT>
 struct BitmapSmem {   // words per row in flight: bitmap, starts of the entries (8 bytes each), their first pairs
@@ -608,7 +636,7 @@ struct BitmapSmem {   // words per row in flight: bitmap, starts of the entries 
     static size_t bytes(int bw, int rows) { return (size_t)rows * (size_t)(bw + extra) * 4; }
 };
 
-template <int NT>
+template <int NT, bool MAP>
 __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(BitmapP a, DevState *st) {
     constexpr bool WARP = NT == 32;
     constexpr int NW = NT / 32;
@@ -626,22 +654,29 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
         if (WARP) __syncwarp();
         else __syncthreads();
     };
-    const int64_t count = (int64_t) * (volatile unsigned long long *)(WARP ? &st->sym_warp : &st->sym_block);
+    const int64_t count = (int64_t) * (volatile unsigned long long *)(WARP ? &st->sym_warp : MAP ? &st->sym_map : &st->sym_block);
     if (count == 0) return;
     for (int x = tid; x < a.bw / 4; x += NT) ((uint4 *)bits)[x] = make_uint4(0u, 0u, 0u, 0u);
     int64_t t = WARP ? (int64_t)blockIdx.x * BM_WPB + wid : 0;
+    bool fail = false;
     while (true) {
         if (!WARP) {   // rows of very different work: handed out one at a time
-            if (tid == 0) row_s = (long long)atomicAdd(&st->next_row, 1ull);
+            if (tid == 0) row_s = (long long)atomicAdd(MAP ? &st->next_map : &st->next_row, 1ull);
             __syncthreads();
             t = row_s;
         }
         if (t >= count) break;
-        const int i = WARP ? a.rows[t] : a.rows[a.n - 1 - t];
+        const int i = WARP ? a.rows[t] : MAP ? a.maps[t] : a.rows[a.n - 1 - t];
         const int2 sp = a.rspan[i];
         const int lo = sp.x, nw = sp.y;
         const int64_t p0 = a.arp[i];
         const int64_t plen = a.arp[i + 1] - p0;
+        // a row over more blocks than the bitmap has: a map by the bound on its blocks
+        int L = 0;
+        if (MAP && nw > a.bw) {
+            const int b = a.bins[i];
+            L = !WARP ? SYM_MAP_BLOCK_L : b <= 2 ? 7 : SYM_MAP_L;
+        }
         sync();
         for (int64_t pb = 0; pb < plen; pb += NT) {
             int len = 0;
@@ -718,6 +753,16 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
                         next = pre[e0 + 1];
                     }
                 }
+                if (MAP && L) {
+#pragma unroll 1
+                    for (int u = 0; u < BM_U; u++) {
+                        int2 x = pr[0];
+#pragma unroll
+                        for (int y = 1; y < BM_U; y++) if (u == y) x = pr[y];
+                        if (x.y != 0 && !sym_map_add(bits + (1 << L), bits, L, x.x, (unsigned)x.y)) fail = true;
+                    }
+                    continue;
+                }
 #pragma unroll
                 for (int u = 0; u < BM_U; u++) {
                     const unsigned wd = (unsigned)(pr[u].x - lo);
@@ -727,10 +772,12 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
             sync();
         }
         int c = 0;
-        for (int x = tid * 4; x < nw; x += NT * 4) {
+        const int used = MAP && L ? 1 << L : nw;   // words that hold bits
+        for (int x = tid * 4; x < used; x += NT * 4) {
             const uint4 v = *(const uint4 *)&bits[x];
             c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
             *(uint4 *)&bits[x] = make_uint4(0u, 0u, 0u, 0u);
+            if (MAP && L) *(uint4 *)&bits[used + x] = make_uint4(0u, 0u, 0u, 0u);
         }
         c = __reduce_add_sync(0xffffffffu, c);
         if (WARP) {
@@ -747,33 +794,40 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
         }
         sync();
     }
+    if (MAP && fail) atomicOr(&st->err, DERR_PROBE);
 }
 
-template <int NT>
+template <int NT, bool MAP>
 static int run_bitmap(const BitmapP &p, DevState *st, const char *label, Ctx &c) {
     const int threads = NT == 32 ? BM_WPB * 32 : NT;
     const size_t smem = BitmapSmem<NT>::bytes(p.bw, NT == 32 ? BM_WPB : 1);
     int per_sm = 0;
-    SG_TRY(kernel_blocks_per_sm((const void *)k_sym_rows<NT>, threads, smem, &per_sm));
+    SG_TRY(kernel_blocks_per_sm((const void *)k_sym_rows<NT, MAP>, threads, smem, &per_sm));
     const int64_t blocks = std::min<int64_t>((p.n * NT + threads - 1) / threads, (int64_t)per_sm * c.nsm);
     c.begin(label, p.n);
-    k_sym_rows<NT><<<(unsigned)blocks, threads, smem, c.s>>>(p, st);
+    k_sym_rows<NT, MAP><<<(unsigned)blocks, threads, smem, c.s>>>(p, st);
     c.end();
     SG_CUDA(cudaGetLastError());
     return SPGEMM_OK;
 }
 
 int launch_symbolic_bitmaps(const spgemm_csr &A, const spgemm_csr &B, const int4 *desc, const int2 *pairs,
-                            const int2 *rspan, const int32_t *rows, int64_t *crp, DevState *st, Ctx &c) {
+                            const int2 *rspan, const int32_t *rows, const int32_t *maps, const uint8_t *bins, int64_t *crp,
+                            DevState *st, Ctx &c) {
     if (A.nrows == 0) return SPGEMM_OK;
     const int nwords = (int)((B.ncols + 31) / 32);
-    BitmapP p{A.row_ptr, A.col_idx, desc, pairs, rspan, rows, A.nrows, crp, (std::min(nwords, SYM_WARP_WORDS) + 3) & ~3};
-    SG_TRY(run_bitmap<32>(p, st, "symbolic.warp_rows", c));
+    BitmapP p{A.row_ptr, A.col_idx, desc, pairs, rspan, rows, maps, bins, A.nrows, crp, (std::min(nwords, SYM_WARP_WORDS) + 3) & ~3};
+    if (nwords <= SYM_WARP_WORDS) SG_TRY((run_bitmap<32, false>(p, st, "symbolic.warp_rows", c)));
+    else SG_TRY((run_bitmap<32, true>(p, st, "symbolic.warp_rows", c)));
+    if (nwords > SYM_MAP_BLOCK_WORDS) {
+        p.bw = 2 << SYM_MAP_BLOCK_L;
+        SG_TRY((run_bitmap<256, true>(p, st, "symbolic.map_rows", c)));
+    }
     p.bw = (nwords + 3) & ~3;
     // a block's threads by the blocks that fit an SM beside its bitmap
-    if (nwords <= 8192) return run_bitmap<256>(p, st, "symbolic.block_rows", c);
-    if (nwords <= 24576) return run_bitmap<512>(p, st, "symbolic.block_rows", c);
-    return run_bitmap<1024>(p, st, "symbolic.block_rows", c);
+    if (nwords <= 8192) return run_bitmap<256, false>(p, st, "symbolic.block_rows", c);
+    if (nwords <= 24576) return run_bitmap<512, false>(p, st, "symbolic.block_rows", c);
+    return run_bitmap<1024, false>(p, st, "symbolic.block_rows", c);
 }
 
 static const char *SYM_LABEL[NBINS] = {"", "", "symbolic.bin2", "symbolic.bin3",
