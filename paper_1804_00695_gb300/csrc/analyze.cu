@@ -22,7 +22,8 @@ namespace sg {
 // addresses 32 rows apart from its neighbours' in one load instruction), and
 // every lane then reads its row from there; otherwise every lane loads its
 // own row.
-constexpr int64_t COMPRESS_LONG = 128;   // rows longer than this take a block each
+constexpr int64_t COMPRESS_LONG = 128;   // rows longer than this take a warp each
+constexpr int64_t COMPRESS_MID = 256;    // and longer than this a block
 constexpr int COMPRESS_STAGE = 1024;     // staged entries per warp
 constexpr int COMPRESS_WPB = 8;
 
@@ -55,12 +56,16 @@ __global__ void __launch_bounds__(COMPRESS_WPB * 32) k_compress(
     }
     __syncwarp();
     const bool lng = end - beg > COMPRESS_LONG;   // k_compress_long
-    const unsigned longs = __ballot_sync(0xffffffffu, lng);
-    if (longs) {
+    if (__any_sync(0xffffffffu, lng)) {   // the warps' rows from the front, the blocks' from the back
+        const bool blk = end - beg > COMPRESS_MID;
+        const unsigned mw = __ballot_sync(0xffffffffu, lng && !blk), mb = __ballot_sync(0xffffffffu, blk);
+        const unsigned below = (1u << lane) - 1u;
         int at = 0;
-        if (lane == 0) at = atomicAdd(long_count, __popc(longs));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (lng) long_list[at + __popc(longs & ((1u << lane) - 1u))] = (int32_t)r;
+        if (lane == 0 && mw) at = atomicAdd(&long_count[0], __popc(mw));
+        if (lane == 1 && mb) at = atomicAdd(&long_count[1], __popc(mb));
+        const int aw = __shfl_sync(0xffffffffu, at, 0), ab = __shfl_sync(0xffffffffu, at, 1);
+        if (blk) long_list[nrows - 1 - (ab + __popc(mb & below))] = (int32_t)r;
+        else if (lng) long_list[aw + __popc(mw & below)] = (int32_t)r;
     }
     if (!live || lng) return;
     const int *src = staged ? stage + (beg - wbeg) : col + beg;
@@ -105,28 +110,33 @@ __global__ void __launch_bounds__(COMPRESS_WPB * 32) k_compress(
     if (unsorted && unsorted_flag) atomicOr(unsorted_flag, 1);
 }
 
-// The same for the listed rows (longer than COMPRESS_LONG), a block per row,
-// COMPRESS_CHUNK entries at a time staged in shared memory: a pair starts
-// where an entry's block differs from the previous entry's (its place is the
-// number of starts before it, a block scan), and the thread at a start ORs the
-// bits of the run that follows.  A warp per row took 32 entries at a time with
-// a segmented scan of the masks and a carried run: a serial chain of 488
-// steps for the longest row of an R-MAT graph of scale 17, 1.5 ms for its 3.7 M
-// entries (0.074 now; scale 13 0.25 -> 0.015 ms).
+// The same for the listed rows, longer than COMPRESS_LONG.  Beyond COMPRESS_MID a
+// block per row, COMPRESS_CHUNK entries at a time staged in shared memory: a pair
+// starts where an entry's block differs from the previous entry's (its place is
+// the number of starts before it, a block scan), and the thread at a start ORs
+// the bits of the run that follows.  A warp per row of any length, 32 entries at a
+// time with a segmented scan of the masks and a carried run, was a serial chain
+// of 488 steps for the longest row of an R-MAT graph of scale 17, 1.5 ms for its
+// 3.7 M entries (0.07 now; scale 13 0.25 -> 0.016 ms).  Up to COMPRESS_MID a warp
+// per row, the whole row at once, the starts counted by ballots (296,296 rows of
+// 135 entries 194 us, 200,000 of 200 172; by a block each 971 and 670, since
+// most of a block's threads then only wait at its barriers).  Rows of 400
+// entries, 100,000 of them, take 385 us by blocks; a hundred of them alone 8.
 constexpr int COMPRESS_BS = 256, COMPRESS_PT = 4, COMPRESS_CHUNK = COMPRESS_BS * COMPRESS_PT;
+static_assert(COMPRESS_BS / 32 * COMPRESS_MID <= 2 * COMPRESS_CHUNK, "a warp's rows are staged where a block's are");
 
 __global__ void __launch_bounds__(COMPRESS_BS) k_compress_long(
-    int64_t ncols, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int2 *__restrict__ pairs,
+    int64_t nrows, int64_t ncols, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, int2 *__restrict__ pairs,
     int32_t *__restrict__ ccnt, int2 *__restrict__ minmax, int4 *__restrict__ desc, int2 *__restrict__ ana, int *err,
     int *unsorted_flag, const int *long_count, const int32_t *__restrict__ long_list) {
     constexpr int NW = COMPRESS_BS / 32;
-    __shared__ __align__(16) int st[COMPRESS_CHUNK];
+    __shared__ __align__(16) int st[2 * COMPRESS_CHUNK];
     __shared__ int wsum[NW], wmin[NW], wmax[NW];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int nlong = *(volatile const int *)long_count;
+    const int nmid = ((volatile const int *)long_count)[0], nlong = ((volatile const int *)long_count)[1];
     bool bad = false, unsorted = false;
     for (int t = blockIdx.x; t < nlong; t += gridDim.x) {
-        const int64_t r = long_list[t];
+        const int64_t r = long_list[nrows - 1 - t];
         const int64_t beg = rp[r], end = rp[r + 1];
         int npairs = 0, bmin = INT_MAX, bmax = INT_MIN;
         for (int64_t base = beg; base < end; base += COMPRESS_CHUNK) {
@@ -209,6 +219,50 @@ __global__ void __launch_bounds__(COMPRESS_BS) k_compress_long(
             if (ana) ana[r] = make_int2(len, npairs);
         }
     }
+    if (nmid > 0) {
+        __syncthreads();
+        int *ws = st + w * COMPRESS_MID;
+        // from the last block on, a warp of each in turn: the first ones have the blocks' rows
+        for (int t = w * gridDim.x + gridDim.x - 1 - blockIdx.x; t < nmid; t += gridDim.x * NW) {
+            const int64_t r = long_list[t];
+            const int64_t beg = rp[r];
+            const int len = (int)(rp[r + 1] - beg);
+            int npairs = 0, bmin = INT_MAX, bmax = INT_MIN;
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < COMPRESS_MID / 32; u++) {
+                const int x = lane + 32 * u;
+                int c = x < len ? col[beg + x] : -1;
+                if (x < len && (c < 0 || (int64_t)c >= ncols)) { bad = true; c = -1; }
+                ws[x] = c;
+            }
+            __syncwarp();
+            for (int x = lane; x - lane < len; x += 32) {
+                const int c = ws[x], prev = x > 0 ? ws[x - 1] : -1;
+                const bool start = c >= 0 && (prev < 0 || (c >> 5) != (prev >> 5));
+                const unsigned m = __ballot_sync(0xffffffffu, start);
+                if (c >= 0) {
+                    unsorted |= c <= prev;
+                    bmin = min(bmin, c >> 5);
+                    bmax = max(bmax, c >> 5);
+                }
+                if (start && pairs) {
+                    unsigned bits = 0;
+                    for (int p = x; p < len && ws[p] >> 5 == c >> 5; p++) bits |= 1u << (ws[p] & 31);
+                    pairs[beg + npairs + __popc(m & ((1u << lane) - 1u))] = make_int2(c >> 5, (int)bits);
+                }
+                npairs += __popc(m);
+            }
+            bmin = __reduce_min_sync(0xffffffffu, bmin);
+            bmax = __reduce_max_sync(0xffffffffu, bmax);
+            if (lane == 0) {
+                if (ccnt) ccnt[r] = npairs;
+                if (minmax) minmax[r] = make_int2(bmin, bmax);
+                if (desc) desc[r] = make_int4((int)(unsigned)(uint64_t)beg, (int)((uint64_t)beg >> 32), len, npairs);
+                if (ana) ana[r] = make_int2(len, npairs);
+            }
+        }
+    }
     if (bad) atomicOr(err, DERR_COL_RANGE);
     if (unsorted && unsorted_flag) *unsorted_flag = 1;
 }
@@ -225,8 +279,9 @@ int launch_compress(const spgemm_csr &M, int2 *pairs, int32_t *ccnt, int2 *minma
         // one resident wave (it returns at once when no row is long)
         const int64_t wblocks = std::min<int64_t>(M.nnz / (COMPRESS_LONG + 1), resident_blocks(k_compress_long, COMPRESS_BS, c.nsm));
         c.begin("compress_long", M.nrows);
-        k_compress_long<<<(unsigned)wblocks, COMPRESS_BS, 0, c.s>>>(M.ncols, M.row_ptr, M.col_idx, pairs, ccnt, minmax,
-                                                                    desc, ana, err, unsorted, long_count, long_list);
+        k_compress_long<<<(unsigned)wblocks, COMPRESS_BS, 0, c.s>>>(M.nrows, M.ncols, M.row_ptr, M.col_idx, pairs,
+                                                                    ccnt, minmax, desc, ana, err, unsorted, long_count,
+                                                                    long_list);
         c.end();
     }
     SG_CUDA(cudaGetLastError());

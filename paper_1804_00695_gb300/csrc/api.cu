@@ -425,7 +425,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         const double mean_alen = (double)A->nnz / (double)n;
         const double mean_pairs = mean_alen * ((double)B->nnz / (double)(B->nrows > 0 ? B->nrows : 1)) * 0.6;
         const int gs = h->g_symbolic ? h->g_symbolic : lanes_for(mean_pairs / 64.0);
-        SG_TRY(launch_compress(*B, pairs, ccnt, minmax, desc, ana, &h->dstate->err, &h->dstate->long_rows,
+        SG_TRY(launch_compress(*B, pairs, ccnt, minmax, desc, ana, &h->dstate->err, h->dstate->long_rows,
                                (int32_t *)(w + L.longs), c, &h->dstate->b_unsorted));
         // B's column blocks fit a bitmap in shared memory: every row is counted
         // without a list length on the host, so the host waits once a call
@@ -1158,9 +1158,9 @@ int spgemm_compress(spgemm_handle h, const spgemm_csr *M, int32_t *count, uint32
     SG_TRY(ws_reserve(h, need + align_up((size_t)M->nrows * 4), s));
     h->sym_valid = false;
     Ctx c = h->ctx(s);
-    SG_CUDA(cudaMemsetAsync(&h->dstate->long_rows, 0, sizeof(int), s));
+    SG_CUDA(cudaMemsetAsync(h->dstate->long_rows, 0, sizeof(h->dstate->long_rows), s));
     SG_TRY(launch_compress(*M, (int2 *)pairs, count, (int2 *)h->ws, nullptr, nullptr, &h->dstate->err,
-                           &h->dstate->long_rows, (int32_t *)(h->ws + need), c));
+                           h->dstate->long_rows, (int32_t *)(h->ws + need), c));
     return SPGEMM_OK;
 }
 

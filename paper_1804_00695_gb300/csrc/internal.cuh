@@ -46,7 +46,7 @@ struct DevState {          // lives in device memory, one per handle
     long long max_row_nnz;   // largest row of C (numeric binning)
     long long flops_total;   // products of the whole product (analysis)
     int b_unsorted;          // some row of B has columns out of ascending order
-    int long_rows;           // rows the compression left to its block-per-row pass
+    int long_rows[2];        // rows the compression left to its second pass: to a warp each, to a block each
     long long max_alen;      // longest row of A (analysis)
     unsigned long long triangles;   // spgemm_triangles: the count
     // numeric rows by class (NumCls): rows, list cursors, largest row of C,
@@ -306,8 +306,8 @@ struct Ctx {
 // desc[k] = {row_ptr[k] low, high 32 bits, entries, pairs};
 // ana[k] = {entries, pairs}.  Any output may be NULL.
 // `unsorted` (may be null) is set to 1 if a row of M is not strictly ascending.
-// `long_count` (device, cleared by the caller before the call) and
-// `long_list` (room for M.nrows): the rows left to the block-per-row pass.
+// `long_count` (device, two, cleared by the caller before the call) and
+// `long_list` (room for M.nrows): the rows left to the second pass.
 int launch_compress(const spgemm_csr &M, int2 *pairs, int32_t *ccnt, int2 *minmax, int4 *desc,
                     int2 *ana, int *err, int *long_count, int32_t *long_list, Ctx &c, int *unsorted = nullptr);
 __device__ __forceinline__ int64_t desc_start(int4 d) {
