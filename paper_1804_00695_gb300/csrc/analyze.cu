@@ -133,7 +133,9 @@ __global__ void __launch_bounds__(COMPRESS_BS) k_compress_long(
     __shared__ __align__(16) int st[2 * COMPRESS_CHUNK];
     __shared__ int wsum[NW], wmin[NW], wmax[NW];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int nmid = ((volatile const int *)long_count)[0], nlong = ((volatile const int *)long_count)[1];
+    // (plain loads: k_compress is through, and the warps of an SM share the line; past the L1 every
+    // warp of the grid asks the L2 for it, 2.5 us a load when no row is long)
+    const int nmid = long_count[0], nlong = long_count[1];
     bool bad = false, unsorted = false;
     for (int t = blockIdx.x; t < nlong; t += gridDim.x) {
         const int64_t r = long_list[nrows - 1 - t];

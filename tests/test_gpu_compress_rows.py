@@ -65,3 +65,27 @@ def test_columns_out_of_range(cuda_lib, n, at):
         M = to_dev(m)
         with pytest.raises(sg.SpgemmError, match="out of range"):
             h.symbolic(to_dev(I.random_csr(10, m.nrows, 0.5, 1)), M)
+
+
+def test_rows_past_the_line_cost_their_entries(cuda_lib):
+    """Compression of 300,000 rows of 136 entries against as many entries in rows
+    of 600: a block for every row past 128 entries took over three times as long."""
+    import torch
+    h = sg.Handle()
+
+    def ms(n, per):
+        col = torch.randint(0, 3_000_000 // per, (n, per), device="cuda") + torch.arange(per, device="cuda") * (3_000_000 // per)
+        B = sg.Csr(n, 3_000_000, torch.arange(n + 1, device="cuda") * per, col.reshape(-1).int(),
+                   torch.ones(1, device="cuda").expand(n * per))
+        A = to_dev(I.random_csr(50, n, 2 / n, 1))
+        h.symbolic(A, B)
+        h.set_timing(True)
+        h.reset_timings()
+        for _ in range(5):
+            h.symbolic(A, B)
+        t = h.timings()
+        h.set_timing(False)
+        return t["compress"][2] + t["compress_long"][2]
+
+    short, long = ms(300_000, 136), ms(68_000, 600)
+    assert short < 1.8 * long, (short, long)
