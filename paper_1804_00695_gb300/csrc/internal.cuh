@@ -79,16 +79,16 @@ constexpr int NBINS = SPGEMM_NBINS;
 //   SYM_MARK_WARP: up to SYM_WARP_PAIRS pairs over at most SYM_WARP_WORDS
 //     blocks: a warp and a bitmap of the span; up to SYM_MAP_PAIRS over more: a
 //     warp and a map;
-//   SYM_MARK_MAP: up to SYM_MAP_BLOCK_PAIRS pairs, and one for 12 blocks of the
+//   SYM_MARK_MAP: up to SYM_MAP_BLOCK_PAIRS pairs, and one for 24 blocks of the
 //     span, over more than SYM_MAP_BLOCK_WORDS: a block and a map;
 //   SYM_MARK_BLOCK: the others: a block and a bitmap.
 // Why the lines lie there (one GB300, whole symbolic call): a block's bitmap is
 // cleared and counted over the whole span, and from 24,576 blocks on one fills
 // an SM, so that rows go through it one at a time.  Bitmap -> map, rows over
-// 3000 / 12,000 / 50,000 blocks: 200,000 of 40 pairs 784 -> 373, 1613 -> 377,
-// 5509 -> 372 us; 78,125 of 256 417 -> 320, 738 -> 340, 2295 -> 350; 33,333 of
-// 600 265 (bitmap kept), 412 -> 376, 1082 -> 379; 20,000 of 1000 214 and 305
-// (kept), 729 -> 324; 10,000 of 2000 185, 232 (kept), 442 -> 308.
+// 3000 / 12,000 / 50,000 blocks: 200,000 of 40 pairs 784 -> 346, 1613 -> 349,
+// 5509 -> 346 us; 78,125 of 256 417 -> 321, 738 -> 339, 2295 -> 340; 33,333 of
+// 600 265 and 412 (bitmap kept), 1082 -> 483; 20,000 of 1000 214 and 305 (kept),
+// 729 -> 401; 10,000 of 2000 185 and 232 (kept), 442 -> 373.
 // A wider B goes through the optimistic first pass and the lists by bin.
 constexpr int64_t SYM_BITMAP_WORDS = 53248;   // 208 KB
 constexpr int SYM_WARP_WORDS = 2048;
@@ -102,7 +102,7 @@ __host__ __device__ inline int sym_mark(long long cpairs, int words) {
     if (cpairs <= SYM_FIRST_PAIRS) return 0;
     if (words <= SYM_WARP_WORDS) return cpairs <= SYM_WARP_PAIRS ? SYM_MARK_WARP : SYM_MARK_BLOCK;
     if (cpairs <= SYM_MAP_PAIRS) return SYM_MARK_WARP;
-    return words > SYM_MAP_BLOCK_WORDS && cpairs <= SYM_MAP_BLOCK_PAIRS && cpairs * 12 <= words ? SYM_MARK_MAP : SYM_MARK_BLOCK;
+    return words > SYM_MAP_BLOCK_WORDS && cpairs <= SYM_MAP_BLOCK_PAIRS && cpairs * 24 <= words ? SYM_MARK_MAP : SYM_MARK_BLOCK;
 }
 
 // Numeric bins by exact output count (and product count):

@@ -637,13 +637,11 @@ struct BitmapSmem {   // words per row in flight: bitmap, starts of the entries 
 };
 
 template <int NT, bool MAP>
-__global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(BitmapP a, DevState *st) {
+__device__ __forceinline__ void sym_rows(const BitmapP &a, DevState *st, unsigned *bm_smem, int *wsum, int *wcnt,
+                                         long long &row_s) {
     constexpr bool WARP = NT == 32;
     constexpr int NW = NT / 32;
     constexpr bool RUNS = !WARP;
-    extern __shared__ __align__(16) unsigned bm_smem[];
-    __shared__ int wsum[NW], wcnt[NW];
-    __shared__ long long row_s;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tid = WARP ? lane : (int)threadIdx.x, w = WARP ? 0 : wid;
     const unsigned below = (1u << lane) - 1u;
@@ -797,13 +795,32 @@ __global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(Bitmap
     if (MAP && fail) atomicOr(&st->err, DERR_PROBE);
 }
 
+// The blocks' maps follow the warps' rows in the same launch (a launch of their
+// own cost 5 us where B has no such row).
+template <int NT, bool MAP>
+__global__ void __launch_bounds__(NT == 32 ? BM_WPB * 32 : NT) k_sym_rows(BitmapP a, DevState *st) {
+    constexpr int NW = NT == 32 ? BM_WPB : NT / 32;
+    extern __shared__ __align__(16) unsigned bm_smem[];
+    __shared__ int wsum[NW], wcnt[NW];
+    __shared__ long long row_s;
+    sym_rows<NT, MAP>(a, st, bm_smem, wsum, wcnt, row_s);
+    if (MAP) {
+        __syncthreads();
+        a.bw = 2 << SYM_MAP_BLOCK_L;
+        sym_rows<BM_WPB * 32, true>(a, st, bm_smem, wsum, wcnt, row_s);
+    }
+}
+
 template <int NT, bool MAP>
 static int run_bitmap(const BitmapP &p, DevState *st, const char *label, Ctx &c) {
     const int threads = NT == 32 ? BM_WPB * 32 : NT;
     const size_t smem = BitmapSmem<NT>::bytes(p.bw, NT == 32 ? BM_WPB : 1);
+    static_assert(!MAP || BM_WPB * (SYM_WARP_WORDS + BitmapSmem<32>::extra) >= (2 << SYM_MAP_BLOCK_L) + BitmapSmem<BM_WPB * 32>::extra,
+                  "a block's map fits where its warps' bitmaps do");
     int per_sm = 0;
     SG_TRY(kernel_blocks_per_sm((const void *)k_sym_rows<NT, MAP>, threads, smem, &per_sm));
-    const int64_t blocks = std::min<int64_t>((p.n * NT + threads - 1) / threads, (int64_t)per_sm * c.nsm);
+    // (with maps a block takes a row too)
+    const int64_t blocks = std::min<int64_t>(MAP ? p.n : (p.n * NT + threads - 1) / threads, (int64_t)per_sm * c.nsm);
     c.begin(label, p.n);
     k_sym_rows<NT, MAP><<<(unsigned)blocks, threads, smem, c.s>>>(p, st);
     c.end();
@@ -819,10 +836,6 @@ int launch_symbolic_bitmaps(const spgemm_csr &A, const spgemm_csr &B, const int4
     BitmapP p{A.row_ptr, A.col_idx, desc, pairs, rspan, rows, maps, bins, A.nrows, crp, (std::min(nwords, SYM_WARP_WORDS) + 3) & ~3};
     if (nwords <= SYM_WARP_WORDS) SG_TRY((run_bitmap<32, false>(p, st, "symbolic.warp_rows", c)));
     else SG_TRY((run_bitmap<32, true>(p, st, "symbolic.warp_rows", c)));
-    if (nwords > SYM_MAP_BLOCK_WORDS) {
-        p.bw = 2 << SYM_MAP_BLOCK_L;
-        SG_TRY((run_bitmap<256, true>(p, st, "symbolic.map_rows", c)));
-    }
     p.bw = (nwords + 3) & ~3;
     // a block's threads by the blocks that fit an SM beside its bitmap
     if (nwords <= 8192) return run_bitmap<256, false>(p, st, "symbolic.block_rows", c);

@@ -1,6 +1,6 @@
 """Symbolic phase of rows with few compressed pairs over wide spans: a map of the
 row's blocks in place of a bitmap of its span, by a warp (up to 256 pairs) or by
-a block (up to 2048, one for 12 blocks).  Rows around every line of the rule and
+a block (up to 2048, one for 24 blocks).  Rows around every line of the rule and
 of the maps' sizes, spans around 2048, 8192 and 24,576 blocks and up to the widest
 bitmap, counts and columns against the CPU oracle; and such rows must not cost a
 pass over their span each."""
