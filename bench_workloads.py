@@ -176,19 +176,35 @@ def _oracle_rows_sample(a, b, fl, start, tol_tag, device_rows, label, seconds=CP
              "sample": f"{label}: rows [{r0}, {r1}) of C ({m} multiplications), {dt:.2f} s"}, par)
 
 
-def dense_numeric_rows(g, c_rp, flops):
-    """Rows of g*g that the dense windows take (g's rows sorted): bins 5 and 6
-    with more than 8192 outputs, or with more than 6144 products and one per 8
-    columns of the row's span of 32-column blocks (num_cls)."""
+def dense_numeric_rows(g, c_rp, flops, nsm):
+    """Rows of g*g that the dense windows take in FP32 (g's rows sorted): bins 5
+    and 6 by num_cls and dense_by_window."""
     rp, col = np.asarray(g.row_ptr, dtype=np.int64), g.col.astype(np.int64)
     some = np.diff(rp) > 0
     lo, hi = np.full(g.nrows, 1 << 40), np.full(g.nrows, -1)
     lo[some], hi[some] = col[rp[:-1][some]] >> 5, col[rp[1:][some] - 1] >> 5
     lo = bench._seg_reduce(np.minimum, lo[col], rp, 1 << 40)
-    words = np.maximum(bench._seg_reduce(np.maximum, hi[col], rp, -1) - lo + 1, 0)
-    nn = np.diff(c_rp)
-    return ((bench.bins_of(nn, flops) >= 5) & (words > 0) & (flops < 1 << 31)
-            & ((nn > 8192) | ((flops > 6144) & (flops * 8 >= words * 32))))
+    span = 32 * np.maximum(bench._seg_reduce(np.maximum, hi[col], rp, -1) - lo + 1, 0)
+    nn, alen, fl = np.diff(c_rp), np.diff(rp), np.asarray(flops, dtype=np.int64)
+
+    def dense(vb):
+        n = -(-span // (90112 // vb))
+        return 13 * span + 281 * alen * n + 38 * fl if vb == 4 else 17 * span + (152 + 26 * np.minimum(n, 32) // 10) * alen * n + 63 * fl
+
+    def cursors(vb):
+        n, warps = -(-span // (32768 // vb)), fl > 256 * alen
+        w = ((63, 2200), (184, 147), 2) if vb == 4 else ((62, 2700), (214, 160), 5)
+        return w[2] * span + np.where(warps, w[0][1], w[0][0]) * alen * n + np.where(warps, w[1][1], w[1][0]) * fl
+
+    both = (bench.bins_of(nn, flops) >= 5) & (span > 0) & (fl < 1 << 31)
+    folds = (alen > 1024) & (fl - nn >= 2048)
+    few = (fl < 6 * alen) & (span <= 8192 * 32) & ~folds
+    small = np.where(few, dense(4) <= 98 * fl + 370 * alen, (fl > 6144) & (fl * 8 >= span))
+    large = folds | (dense(4) <= cursors(4))
+    by_cursors = both & (nn > 8192) & ~large
+    if by_cursors.sum() <= 2 * nsm:
+        large = np.ones_like(large)
+    return both & np.where(nn > 8192, large, small)
 
 
 # ---------------------------------------------------------------- R-MAT
@@ -250,12 +266,12 @@ def measure_rmat(args, g, local):
         elif lab == "small":
             mask = (bb == 1) | (bb == 2)
         elif lab == "dense":
-            mask = dense_numeric_rows(g, crp, fl)
+            mask = dense_numeric_rows(g, crp, fl, torch.cuda.get_device_properties(0).multi_processor_count)
         elif lab.startswith("bin"):
             mask = bb == int(lab[3:4])
         else:
             continue
-        if lab == "dense" and mask.sum() * nl != nrows:
+        if lab.startswith(("dense", "bin")) and mask.sum() * nl != nrows:   # not the rows of one launch
             continue
         kern.append((tms / nl, key, bench.kernel_bytes(g, g.row_ptr, crp, mask, 4, True), nl))
     roof = None

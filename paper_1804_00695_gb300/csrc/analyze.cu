@@ -575,7 +575,7 @@ __global__ void k_scan_sums(long long *tile_sums, int64_t tiles, long long *tota
 // same pass (k_scan_apply<true>): the counts are in registers there, and a
 // pass of its own read the offsets again and cost a launch.
 struct ScanBins {
-    const int64_t *flops;
+    const int64_t *arp, *flops;
     uint8_t *bins, *cls;
     const int2 *rspan;
     const int32_t *nlo;   // may be null
@@ -643,7 +643,8 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
             if (bin >= 2 && bin <= BIN_HUGE) {
                 const int words = b.rspan[i].y;
                 const bool listed = b.nlo && b.nlo[i] >= 0 && b.nwords[i] <= NARROW_NMAX;
-                k = num_cls(bin, c, f, words, listed, b.dense_ok && b.st->b_unsorted == 0);
+                k = num_cls(bin, c, f, words, listed, b.dense_ok && b.st->b_unsorted == 0,
+                            bin >= 5 ? b.arp[i + 1] - b.arp[i] : 0);
                 atomicAdd(&ccnt[k], 1);
                 if (c > cnnz[k]) atomicMax(&cnnz[k], (int)min(c, (long long)INT_MAX));
                 if (words > cwords[k]) atomicMax(&cwords[k], words);
@@ -696,11 +697,11 @@ int launch_scan_counts(int64_t *x, int64_t n, long long *total, void *tmp, Ctx &
     return run_scan<false, SCAN_PT>(x, n, total, tmp, ScanBins{}, c);
 }
 
-int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                        const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
+int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *arp, const int64_t *flops, uint8_t *bins,
+                        uint8_t *cls, const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
                         Ctx &c) {
     if (n == 0) return launch_scan_counts(crp, n, &st->nnz, tmp, c);
-    const ScanBins b{flops, bins, cls, rspan, nlo, nwords, st, dense_ok};
+    const ScanBins b{arp, flops, bins, cls, rspan, nlo, nwords, st, dense_ok};
     return n <= SCAN_FEW ? run_scan<true, 1>(crp, n, &st->nnz, tmp, b, c) : run_scan<true, SCAN_BIN_PT>(crp, n, &st->nnz, tmp, b, c);
 }
 

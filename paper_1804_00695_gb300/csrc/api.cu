@@ -465,9 +465,10 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         }
         // the split table of the dense rows stays within B's own size (and 64 MB)
         const size_t dense_bytes = dense_ws(B->nrows, B->ncols);
-        const bool dense_ok = dense_bytes <= (size_t)B->nnz * 12 + ((size_t)64 << 20);
-        SG_TRY(launch_scan_binning(C_row_ptr, n, w + L.tmp, flops, bins, cls, rspan, h->narrow ? nlo : nullptr,
-                                   nwords, h->dstate, dense_ok, c));
+        const size_t ws_most = (size_t)B->nnz * 12 + ((size_t)64 << 20);
+        const bool dense_ok = dense_bytes <= ws_most;
+        SG_TRY(launch_scan_binning(C_row_ptr, n, w + L.tmp, A->row_ptr, flops, bins, cls, rspan,
+                                   h->narrow ? nlo : nullptr, nwords, h->dstate, dense_ok, c));
         SG_TRY(fetch_state(h, s));
         SG_TRY(device_errors(h->hstate->err));
         *nnz_C = h->hstate->nnz;
@@ -487,10 +488,19 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
                          ? std::max(numeric_global_ws(h->max_row_nnz, B->ncols, h->nsm, SPGEMM_F64),
                                     window_global_ws(h->max_alen, h->nsm))
                          : 0;
-        if (h->cls.count[CLS_DENSE]) h->num_gws = std::max(h->num_gws, dense_bytes + dense_fold_ws(h->max_alen, h->nsm));
+        const long long *cc = h->cls.count;
+        const long long sparse = cc[CLS_DENSE_S] + std::max(cc[CLS_DENSE_D], cc[CLS_DENSE_F]);   // in either type
+        if (cc[CLS_DENSE] + sparse > 0)
+            h->num_gws = std::max(h->num_gws, dense_bytes + dense_fold_ws(h->max_alen, h->nsm));
+        // the cursors' workspace, if there is room: dense windows take those rows too
+        const size_t must = h->num_gws;
+        if (dense_by_window(sparse, h->nsm, h->max_alen, std::max(ws_most, (size_t)1 << 30)))
+            h->num_gws = std::max(h->num_gws, window_global_ws(h->max_alen, h->nsm));
         h->num_lists = 0;
         // numeric scratch: B split into double-words, then the second-level maps
-        SG_TRY(ws_reserve(h, L.persist + align_up((size_t)B->nnz * 8) + h->num_gws, s, L.persist));
+        const size_t before = L.persist + align_up((size_t)B->nnz * 8);
+        if (h->num_gws > must && ws_reserve(h, before + h->num_gws, s, L.persist) != SPGEMM_OK) h->num_gws = must;
+        SG_TRY(ws_reserve(h, before + h->num_gws, s, L.persist));
     }
     h->a_rp = A->row_ptr; h->a_col = A->col_idx; h->a_n = A->nrows; h->a_m = A->ncols;
     h->a_nnz = A->nnz;

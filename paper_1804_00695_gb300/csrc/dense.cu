@@ -382,7 +382,7 @@ static void dense_windows(int64_t ncols, int64_t most, int &W, int &nwin) {
 // Columns that fit a window: 88 KB of accumulators (96 once rounded up)
 // beside 10-12 KB of staging, two blocks an SM.
 template <typename V>
-constexpr int64_t dense_most() { return 88 * 1024 / (int64_t)sizeof(V); }
+constexpr int64_t dense_most() { return DENSE_BYTES / (int64_t)sizeof(V); }
 
 size_t dense_ws(int64_t nrows_b, int64_t ncols_b) {
     int W, nwin;
@@ -391,7 +391,8 @@ size_t dense_ws(int64_t nrows_b, int64_t ncols_b) {
 }
 // The windows' sums of all blocks that fit the chip (no more than its shared
 // memory), when a row of A has more than the batches of one fold.
-size_t dense_fold_ws(int64_t max_alen, int nsm) { return max_alen > 256 * DENSE_FOLD ? (size_t)nsm * (228 << 10) : 0; }
+static_assert(DENSE_FOLD_ALEN == 256 * DENSE_FOLD, "the shortest row of A that is folded");
+size_t dense_fold_ws(int64_t max_alen, int nsm) { return max_alen > DENSE_FOLD_ALEN ? (size_t)nsm * (228 << 10) : 0; }
 
 template <typename V>
 static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc, const int2 *rspan,

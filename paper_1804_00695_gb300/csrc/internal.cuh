@@ -154,8 +154,11 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 //               of at most RANK_S_NNZ outputs, and of at most RANK_M_NNZ
 //   CLS_WIDE3 .. CLS_WIDE4C   other rows of bins 3 and 4 by outputs
 //   CLS_BLOCK, CLS_HUGE       other rows of bins 5 and 6
-//   CLS_DENSE   rows of B sorted: rows with more outputs than the rank
-//               accumulators hold, or many products over their span
+//   CLS_DENSE   rows of B sorted: rows with many products over their span
+//   CLS_DENSE_D, CLS_DENSE, CLS_DENSE_F, CLS_DENSE_S  rows of B sorted: rows with
+//               more outputs than the rank accumulators hold, by the types in which
+//               dense windows cost less than cursors: FP64 only, both, FP32
+//               only (or the row may need folds), neither; see dense_by_window
 // Why the lines lie there: 512 products are eight a lane for the two warps of
 // a short row (rank.cu has both sides; 8192 blocks keep its first bitmap
 // within 1.5 KB), 1024 eight for four warps (13,774 rows of 513 to 1024 FP32
@@ -168,7 +171,8 @@ __host__ __device__ inline int sym_bin(long long keys, long long cpairs) {
 // faster than the maps and windows (rank.cu has the figures).
 enum NumCls {
     CLS_NONE = 0, CLS_B2, CLS_WINDOW_W, CLS_WINDOW_B, CLS_RANK_W, CLS_RANK_S, CLS_RANK_V, CLS_RANK_M4, CLS_RANK_M5, CLS_WIDE3, CLS_WIDE4A, CLS_WIDE4B, CLS_WIDE4C,
-    CLS_BLOCK, CLS_DENSE, CLS_HUGE, CLS_NARROW, NCLS
+    CLS_BLOCK, CLS_DENSE_D, CLS_DENSE, CLS_DENSE_F, CLS_DENSE_S,
+    CLS_HUGE, CLS_NARROW, NCLS
 };
 static_assert(NCLS <= CLS_SLOTS, "DevState keeps the classes' counts");
 constexpr int RANK_S_NNZ = 1024, RANK_S_WORDS = 2048, RANK_M_NNZ = 8192, RANK_M_WORDS = 8192;
@@ -180,17 +184,67 @@ constexpr long long RANK_FLOPS = 1LL << 24;   // products (their prefix sums fit
 // registers: A*A of R-MAT graphs, FP64, scale 16 with 12 edges a vertex 11.9
 // ms (one per 4 columns 12.4), scale 15 with 5 2.91 (2.94, one per 2 3.02).
 constexpr long long DENSE_FLOPS = 6144;
+// Rows with more outputs than the rank accumulators hold choose between the dense
+// windows and the windows walked by cursors (k_num_window) by what either costs:
+// its columns written out, every entry of the row of A staged (or its cursor
+// looked at) in every window, and the products; the cursors' entries more where
+// rows of B of over 256 entries go to a warp each.  The weights (0.1 ps of the chip
+// for a row, rows enough to fill it) are least-squares fits to 84 measured products
+// a kernel and type, spans of 9000 to 4 M columns, rows of B of 2 to 5000, 1 to 64
+// columns a product: two of three within 13%, all within 45%; the choice costs 1%
+// over the better kernel in the mean, 24% at worst.  Cursors -> dense, 2000 rows
+// over rows of B of 64, a product per c columns (ms): 262,144
+// columns FP32 c 6 2.00 -> 1.42, 12 1.08 -> 1.02, 16 0.77 -> 0.95, 24 0.60 -> 0.88
+// (FP64 2.59 -> 2.30, 1.54 -> 1.36, 1.09 -> 1.25, 0.93 -> 1.15); 1,048,576 columns,
+// c 10 4.5 -> 5.3 (6.7 -> 9.5), with rows of B of 1000 4.7 -> 2.0 (9.5 -> 2.7);
+// 10,000,000 columns, 10,000 products a row 7.2 -> 22.8 (14.2 -> 30.9).
+// Rows that fit the chip at once in dense windows (DENSE_FEW for each SM) take them
+// all the same: 40 rows over 524,288 columns, c 16 0.38 -> 0.23 ms, over 4,194,304,
+// c 64 3.0 -> 1.9; and so do all where the cursors' workspace has no room.  In FP32
+// a row that may hold sums long enough for folds (dense.cu) keeps them.
+// Rows of at most RANK_M_NNZ outputs over rows of B of a few entries choose between
+// dense windows and the rank accumulators in the same way (2000 rows of 3250
+// entries of two products, FP32, rank 351 us over 9000 and 356 over 60,000 columns;
+// 4000 entries of two over 40,000 columns, dense 574).
+constexpr int DENSE_BYTES = 88 * 1024;   // a window's accumulators
+constexpr int DENSE_FEW = 2;
+constexpr int DENSE_FOLD_ALEN = 1024;    // entries of a row of A from which on folds begin
+constexpr int DENSE_FOLD_TERMS = 2048;   // a sum of so many terms is folded whatever the window
 constexpr int WINDOW_NNZ = 256;
 constexpr long long WINDOW_FLOPS = 4096;
-// listed: the row is narrow and its words are all in its list.
-__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words, bool listed, bool dense_ok) {
+__host__ __device__ inline long long dense_cost(int vb, long long span, long long alen, long long flops) {
+    const long long w = DENSE_BYTES / vb, n = (span + w - 1) / w;
+    return vb == 4 ? 13 * span + 281 * alen * n + 38 * flops
+                   : 17 * span + (152 + 26 * (n < 32 ? n : 32) / 10) * alen * n + 63 * flops;
+}
+__host__ __device__ inline long long cursor_cost(int vb, long long span, long long alen, long long flops) {
+    const long long w = 32768 / vb, n = (span + w - 1) / w;
+    const bool warps = flops > 256 * alen;
+    return vb == 4 ? 2 * span + (warps ? 2200 : 63) * alen * n + (warps ? 147 : 184) * flops
+                   : 5 * span + (warps ? 2700 : 62) * alen * n + (warps ? 160 : 214) * flops;
+}
+// listed: the row is narrow and its words are all in its list; alen: entries of
+// the row of A (read for bins 5 and 6 only).
+__host__ __device__ inline int num_cls(int bin, long long nnz, long long flops, int words, bool listed, bool dense_ok,
+                                       long long alen) {
     if (bin < 2) return CLS_NONE;
     if (bin == 7) return CLS_NARROW;
     if (bin == 2) return CLS_B2;
     if (listed && nnz <= WINDOW_NNZ) return flops < WINDOW_FLOPS ? CLS_WINDOW_W : CLS_WINDOW_B;
-    if (dense_ok && bin >= 5 && words > 0 && flops < (1LL << 31) &&
-        (nnz > RANK_M_NNZ || (flops > DENSE_FLOPS && flops * 8 >= (long long)words * 32)))
-        return CLS_DENSE;
+    if (dense_ok && bin >= 5 && words > 0 && flops < (1LL << 31)) {
+        const long long span = (long long)words * 32;
+        const bool folds = alen > DENSE_FOLD_ALEN && flops - nnz >= DENSE_FOLD_TERMS;
+        if (nnz <= RANK_M_NNZ) {
+            bool dense = flops > DENSE_FLOPS && flops * 8 >= span;
+            if (flops < 6 * alen && words <= RANK_M_WORDS && !folds)   // short rows of B
+                dense = dense_cost(4, span, alen, flops) <= 98 * flops + 370 * alen;
+            if (dense) return CLS_DENSE;
+        } else {
+            const bool d = dense_cost(8, span, alen, flops) <= cursor_cost(8, span, alen, flops);
+            const bool f = folds || dense_cost(4, span, alen, flops) <= cursor_cost(4, span, alen, flops);
+            return f ? (d ? CLS_DENSE : CLS_DENSE_F) : d ? CLS_DENSE_D : CLS_DENSE_S;
+        }
+    }
     if (words > 0 && flops <= RANK_FLOPS) {
         if (flops <= RANK_W_FLOPS && words <= RANK_M_WORDS) return CLS_RANK_W;
         if (nnz <= RANK_S_NNZ && bin <= 4 && words <= RANK_S_WORDS) return CLS_RANK_S;
@@ -330,8 +384,8 @@ int launch_analyze(const spgemm_csr &A, const spgemm_csr &B, const int2 *ana, co
 // symbolic phase found narrow (nlo[i] >= 0; nlo may be null) that fit the
 // narrow numeric kernel get BIN_NARROW.  cls[i]: the row's class (num_cls);
 // rows, largest row and span per class in st.
-int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *flops, uint8_t *bins, uint8_t *cls,
-                        const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
+int launch_scan_binning(int64_t *crp, int64_t n, void *tmp, const int64_t *arp, const int64_t *flops, uint8_t *bins,
+                        uint8_t *cls, const int2 *rspan, const int32_t *nlo, const uint8_t *nwords, DevState *st, bool dense_ok,
                         Ctx &c);
 // Row lists of the symbolic second pass by bin: rows[offset(b) + t], offsets
 // from st->bin_count[0].
@@ -428,6 +482,12 @@ enum RankSize { RANK_SHORT, RANK_MID, RANK_ROW, RANK_LONG };
 int launch_num_rank(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
                     const int2 *rspan, const int32_t *rows, int64_t count, RankSize size, int64_t max_nnz,
                     int64_t max_words, int *err, Ctx &c);
+
+// Whether so many rows that cost less by cursors go to them, which need
+// window_global_ws(max_alen) bytes of ws_bytes.
+inline bool dense_by_window(long long count, int nsm, int64_t max_alen, size_t ws_bytes) {
+    return count > (long long)DENSE_FEW * nsm && window_global_ws(max_alen, nsm) <= ws_bytes;
+}
 
 // dense.cu: listed rows over windows of a dense accumulator (rows of B
 // sorted); dense_ws: bytes of the split table (either type); next: device counter.

@@ -1618,6 +1618,7 @@ static int run_huge(const NumP &a, const spgemm_csr &B, const int32_t *rows, int
 template <typename V>
 static int run_window(const NumP &a, const int32_t *rows, int64_t cnt, int *err, void *gws, size_t gws_bytes,
                       int64_t max_alen, Ctx &c) {
+    if (cnt <= 0) return SPGEMM_OK;
     constexpr int W = sizeof(V) == 8 ? 4096 : 8192;
     const int64_t cap = (int64_t)c.nsm * WIN_BPSM;
     const int64_t blocks = cnt < cap ? cnt : cap;
@@ -1664,6 +1665,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
     const bool short_with_rows = MODE != MODE_DW && cls.count[CLS_RANK_S] > 0 && cls.words[CLS_RANK_W] <= RANK_S_WORDS &&
                                  cls.count[CLS_RANK_W] < (int64_t)c.nsm * 96;
     int64_t off = 0;
+    bool dense_done = false;
     for (int k = first; k < NCLS; k++) {
         int64_t cnt = cls.count[k];
         const int32_t *r = rows + off;
@@ -1745,9 +1747,24 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                 SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
                 break;
             case CLS_BLOCK: SG_TRY((run_block<256, 8192, V>(a, r, cnt, err, BIN_HUGE - 1, c))); break;
+            case CLS_DENSE_D:
             case CLS_DENSE:
-                SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, r, cnt, gws, gws_bytes, &st->next_row, err, c));
+            case CLS_DENSE_F:
+            case CLS_DENSE_S: {   // lists one after another: all of them at the first that has rows
+                if (dense_done) break;
+                dense_done = true;
+                const int64_t nd = cls.count[CLS_DENSE_D], nb = cls.count[CLS_DENSE], nf = cls.count[CLS_DENSE_F], ns = cls.count[CLS_DENSE_S];
+                const bool f32 = MODE == MODE_F32;
+                const bool cursors = dense_by_window(ns + (f32 ? nd : nf), c.nsm, max_alen, gws_bytes);
+                const int32_t *d = cursors && f32 ? r + nd : r;
+                const int64_t dense = !cursors ? nd + nb + nf + ns : nb + (f32 ? nf : nd);
+                SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, d, dense, gws, gws_bytes, &st->next_row, err, c));
+                if (!cursors) break;
+                if (f32) SG_TRY(run_window<V>(a, r, nd, err, gws, gws_bytes, max_alen, c));
+                const int64_t rest = f32 ? ns : nf + ns;
+                SG_TRY(run_window<V>(a, d + dense, rest, err, gws, gws_bytes, max_alen, c));
                 break;
+            }
             case CLS_NARROW: break;   // launch_num_narrow
             default:
                 if (b_sorted) SG_TRY(run_window<V>(a, r, cnt, err, gws, gws_bytes, max_alen, c));
