@@ -1647,6 +1647,21 @@ static int run_warp_rank(const NumP &a, const int4 *bdesc, const int2 *rspan, co
     return run_rank<RANK_BW3, RANK_NMAX3, 4>(a, bdesc, rspan, r, cnt, 3, st, err, "numeric.rank2048", c);
 }
 
+// Rows of at most 1024 outputs over wider spans, a warp and a map each, four map
+// sizes by outputs; only the sizes that the list's largest row asks for (100,000
+// double-word rows of 64 outputs over 100,000 columns took 0.90 ms in the maps
+// of 512 slots and 0.55 in those of 256).
+template <int MODE>
+static int run_wide_rows(const NumP &a, const int4 *bdesc, const int2 *rspan, const int32_t *r, int64_t cnt, int max_nnz,
+                         DevState *st, Ctx &c) {
+    int *err = &st->err;
+    SG_TRY((run_wide<256, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide3", c)));
+    if (max_nnz > 128) SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 129, 1, st, err, "numeric.wide4a", c)));
+    if (max_nnz > 256) SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
+    if (max_nnz > 512) SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
+    return SPGEMM_OK;
+}
+
 template <int MODE>
 static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const uint8_t *bins,
                    const int4 *bdesc, const int2 *rspan, const int32_t *rows, const long long *counts,
@@ -1692,11 +1707,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                     break;
                 }
                 if (k == CLS_RANK_W) SG_TRY(run_warp_rank(a, bdesc, rspan, r, cnt, st, c));
-                if (cls.words[k] > RANK_S_WORDS) {
-                    SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
-                    SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
-                    SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
-                }
+                if (cls.words[k] > RANK_S_WORDS) SG_TRY(run_wide_rows<MODE>(a, bdesc, rspan, r, cnt, cls.nnz[k], st, c));
                 break;
             case CLS_B2:
             case CLS_RANK_S:
@@ -1715,9 +1726,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                 break;
             case CLS_RANK_M4:
                 if (MODE == MODE_DW) {
-                    SG_TRY((run_wide<512, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 0, 1, st, err, "numeric.wide4a", c)));
-                    SG_TRY((run_wide<1024, 64, 8, MODE>(a, bdesc, rspan, r, cnt, 257, 1, st, err, "numeric.wide4b", c)));
-                    SG_TRY((run_wide<2048, 64, 4, MODE>(a, bdesc, rspan, r, cnt, 513, 1, st, err, "numeric.wide4c", c)));
+                    SG_TRY(run_wide_rows<MODE>(a, bdesc, rspan, r, cnt, cls.nnz[k], st, c));
                     break;
                 }
                 if (cls.count[CLS_RANK_M5]) break;   // one launch with the next list
