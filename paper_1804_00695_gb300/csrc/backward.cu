@@ -35,14 +35,17 @@ __device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int
 // within it, as in rank.cu), each lane finds dC_ij by binary search in the
 // copy, adds its dA term into the staged entry's accumulator and its dB term
 // atomically into db.
-// What bounds it: the chain B's column -> search -> dC.  BWD_U steps go
-// through it together: their loads of B, then their searches (as many halvings
-// for every lane), then their loads of dC.  Measured (one GB300, FP32): 20,001
-// rows of about 320 products 101 -> 80 us (two steps together 87, six 95).
-constexpr int BWD_CAP = 1024, BWD_WPB = 8, BWD_E = 32, BWD_U = 4;
+// What bounds it: the chain B's column -> search -> dC.  U steps go through it
+// together: their loads of B, then their searches (as many halvings for every
+// lane), then their loads of dC.  Measured (one GB300, FP32): 20,001 rows of about
+// 320 products 101 -> 80 us with four steps together (two 87, six 95).  Where the
+// rows have 32 products or fewer in the mean, or 64, most have one step, or two,
+// and the others only cost: 200,000 rows of 9 products 153 us with four, 134 with
+// one, of 25 164 and 139; of 36 202 with four, 182 with two, of 64 227 and 215.
+constexpr int BWD_CAP = 1024, BWD_WPB = 8, BWD_E = 32;
 constexpr int BWD_ROW_MAX = 1 << 20;   // entries of a row of B taken (32 of them fit an int; a row of C holds fewer)
 
-template <typename V>
+template <typename V, int U>
 __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
     int64_t nrows, const int64_t *__restrict__ arp, const int32_t *__restrict__ acol,
     const V *__restrict__ aval, const int64_t *__restrict__ brp, const int32_t *__restrict__ bcol,
@@ -96,13 +99,13 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
             const int total = __shfl_sync(0xffffffffu, incl, 31);
             __syncwarp();
             const int at = lane < ne ? pre[lane] : INT_MAX;   // first product of entry `lane`
-            for (int t0 = 0; t0 < total; t0 += 32 * BWD_U) {
-                long long q[BWD_U];
-                int e[BWD_U], j[BWD_U], lo[BWD_U];
-                unsigned m[BWD_U];
-                V bv[BWD_U], g[BWD_U];
+            for (int t0 = 0; t0 < total; t0 += 32 * U) {
+                long long q[U];
+                int e[U], j[U], lo[U];
+                unsigned m[U];
+                V bv[U], g[U];
 #pragma unroll
-                for (int u = 0; u < BWD_U; u++) {
+                for (int u = 0; u < U; u++) {
                     const int tc = t0 + 32 * u;
                     e[u] = -1;
                     j[u] = lo[u] = 0;
@@ -121,11 +124,11 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
                 for (int n = nc; n > 1;) {
                     const int half = n >> 1;
 #pragma unroll
-                    for (int u = 0; u < BWD_U; u++) lo[u] += cs[lo[u] + half - 1] < j[u] ? half : 0;
+                    for (int u = 0; u < U; u++) lo[u] += cs[lo[u] + half - 1] < j[u] ? half : 0;
                     n -= half;
                 }
 #pragma unroll
-                for (int u = 0; u < BWD_U; u++) {
+                for (int u = 0; u < U; u++) {
                     g[u] = V(0);
                     if (e[u] < 0) continue;
                     if (lo[u] < nc && cs[lo[u]] < j[u]) lo[u]++;
@@ -137,7 +140,7 @@ __global__ void __launch_bounds__(BWD_WPB * 32) k_backward_rows(
                     }
                 }
 #pragma unroll
-                for (int u = 0; u < BWD_U; u++) {
+                for (int u = 0; u < U; u++) {
                     const int tc = t0 + 32 * u;
                     if (tc >= total) break;
                     if (db && e[u] >= 0) atomicAdd(&db[q[u]], ea[e[u]] * g[u]);
@@ -210,11 +213,17 @@ static int run_bwd(const spgemm_csr &A, const spgemm_csr &B, const spgemm_csr &C
     if (A.nrows == 0) return SPGEMM_OK;
     int64_t rblocks = (A.nrows + BWD_WPB - 1) / BWD_WPB;
     rblocks = rblocks < (int64_t)c.nsm * 16 ? rblocks : (int64_t)c.nsm * 16;
-    c.begin("backward", A.nrows);
-    k_backward_rows<V><<<(unsigned)rblocks, BWD_WPB * 32, 0, c.s>>>(
-        A.nrows, A.row_ptr, A.col_idx, (const V *)A.values, B.row_ptr, B.col_idx,
-        da ? (const V *)B.values : nullptr, C.row_ptr, C.col_idx, (const V *)C.values, (V *)da, (V *)db, err);
-    c.end();
+    auto rows = [&](auto kern) {
+        c.begin("backward", A.nrows);
+        kern<<<(unsigned)rblocks, BWD_WPB * 32, 0, c.s>>>(
+            A.nrows, A.row_ptr, A.col_idx, (const V *)A.values, B.row_ptr, B.col_idx,
+            da ? (const V *)B.values : nullptr, C.row_ptr, C.col_idx, (const V *)C.values, (V *)da, (V *)db, err);
+        c.end();
+    };
+    const double products = (double)A.nnz * (double)B.nnz / ((double)A.nrows * (double)std::max<int64_t>(B.nrows, 1));
+    if (products <= 32.0) rows(k_backward_rows<V, 1>);
+    else if (products <= 64.0) rows(k_backward_rows<V, 2>);
+    else rows(k_backward_rows<V, 4>);
     SG_CUDA(cudaGetLastError());
     int64_t blocks = (A.nrows * G + 255) / 256;
     blocks = blocks < (int64_t)c.nsm * 32 ? blocks : (int64_t)c.nsm * 32;
