@@ -115,6 +115,7 @@ struct spgemm_handle_s {
     ClsInfo cls;              // numeric rows by class (symbolic)
     size_t num_gws = 0;   // bytes of the second-level maps numeric needs
     int num_lists = 0;        // first class of the numeric row lists built (0 = none)
+    bool lists_in_graph = false;   // a captured call makes them when its graph runs
     bool b_sorted = false;    // every row of B strictly ascending (symbolic)
     int64_t max_alen = 0;     // longest row of A
     int small_cap = 32, slot_factor = 2;
@@ -497,6 +498,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         if (dense_by_window(sparse, h->nsm, h->max_alen, std::max(ws_most, (size_t)1 << 30)))
             h->num_gws = std::max(h->num_gws, window_global_ws(h->max_alen, h->nsm));
         h->num_lists = 0;
+        h->lists_in_graph = false;
         // numeric scratch: B split into double-words, then the second-level maps
         const size_t before = L.persist + align_up((size_t)B->nnz * 8);
         if (h->num_gws > must && ws_reserve(h, before + h->num_gws, s, L.persist) != SPGEMM_OK) h->num_gws = must;
@@ -559,7 +561,13 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
         if (k != CLS_NARROW || h->cls.count[k] < n) listed += h->cls.count[k];
     if (listed > 0 && h->num_lists != first_list) {
         SG_TRY(launch_scatter_cls(n, cls, rows, h->dstate, first_list, c));
-        h->num_lists = first_list;
+        // Under capture the lists are made whenever the graph runs, not by this
+        // call: a later call may come before it, or after it with other options,
+        // and makes its own.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        SG_CUDA(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) h->lists_in_graph = true;
+        h->num_lists = h->lists_in_graph ? 0 : first_list;
     }
     if (h->num_counts[BIN_NARROW] > 0) {
         // lanes per row: a chunk of G consecutive entries of a row of B per
