@@ -85,7 +85,7 @@ struct DenseP {
 };
 
 // In FP32 a slot takes the terms of at most DENSE_FOLD batches of a row's
-// entries before the window is added to sums of its own in global memory (L2):
+// entries (1024 with blocks of 256 threads, 2048 with 512) before the window is added to sums of its own in global memory (L2):
 // a hub's entries are sums of tens of thousands of terms, and the rounding of
 // one long chain of additions grows with its length.  A*A of an R-MAT graph of
 // scale 17 against 64 bits (2-norms): 3.6e-7 to 1.2e-6 -> 1.6e-7, for 13.9 ->
@@ -396,7 +396,8 @@ size_t dense_fold_ws(int64_t max_alen, int nsm) { return max_alen > DENSE_FOLD_A
 
 template <typename V>
 static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc, const int2 *rspan,
-                     const int32_t *rows, int64_t count, void *ws, size_t ws_bytes, unsigned long long *next, int *err, Ctx &c) {
+                     const int32_t *rows, int64_t count, int64_t max_alen, void *ws, size_t ws_bytes,
+                     unsigned long long *next, int *err, Ctx &c) {
     int W, nwin;
     dense_windows(B.ncols, dense_most<V>(), W, nwin);
     int32_t *split = (int32_t *)ws;
@@ -420,7 +421,13 @@ static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, co
         int per_sm = 0;
         SG_TRY(kernel_blocks_per_sm((const void *)kern, T, smem, &per_sm));
         const int64_t blocks = std::min<int64_t>(count, (int64_t)per_sm * c.nsm);
-        if (sizeof(V) == 4 && used + (size_t)blocks * W * sizeof(V) <= ws_bytes) p.fold = (V *)((char *)ws + used);
+        if (sizeof(V) == 4 && max_alen > (int64_t)T * DENSE_FOLD) {
+            if (used + (size_t)blocks * W * sizeof(V) > ws_bytes) {
+                set_error("numeric: workspace of the folded windows too small");
+                return SPGEMM_ERR_INTERNAL;
+            }
+            p.fold = (V *)((char *)ws + used);
+        }
         c.begin("numeric.dense", count);
         kern<<<(unsigned)blocks, T, smem, c.s>>>(p, err);
         c.end();
@@ -432,11 +439,11 @@ static int num_dense(const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, co
 }
 
 int launch_num_dense(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                     const int2 *rspan, const int32_t *rows, int64_t count, void *ws, size_t ws_bytes,
-                     unsigned long long *next, int *err, Ctx &c) {
+                     const int2 *rspan, const int32_t *rows, int64_t count, int64_t max_alen, void *ws,
+                     size_t ws_bytes, unsigned long long *next, int *err, Ctx &c) {
     if (count <= 0) return SPGEMM_OK;
-    return dtype == SPGEMM_F32 ? num_dense<float>(A, B, C, bdesc, rspan, rows, count, ws, ws_bytes, next, err, c)
-                               : num_dense<double>(A, B, C, bdesc, rspan, rows, count, ws, ws_bytes, next, err, c);
+    return dtype == SPGEMM_F32 ? num_dense<float>(A, B, C, bdesc, rspan, rows, count, max_alen, ws, ws_bytes, next, err, c)
+                               : num_dense<double>(A, B, C, bdesc, rspan, rows, count, max_alen, ws, ws_bytes, next, err, c);
 }
 
 }  // namespace sg

@@ -490,12 +490,13 @@ inline bool dense_by_window(long long count, int nsm, int64_t max_alen, size_t w
 }
 
 // dense.cu: listed rows over windows of a dense accumulator (rows of B
-// sorted); dense_ws: bytes of the split table (either type); next: device counter.
+// sorted); ws holds the split table (dense_ws, either type) and behind it, when a row of
+// A is long enough for folds, the folded windows (dense_fold_ws); next: device counter.
 size_t dense_ws(int64_t nrows_b, int64_t ncols_b);
-size_t dense_fold_ws(int64_t max_alen, int nsm);   // behind the table
+size_t dense_fold_ws(int64_t max_alen, int nsm);
 int launch_num_dense(int dtype, const spgemm_csr &A, const spgemm_csr &B, spgemm_csr &C, const int4 *bdesc,
-                     const int2 *rspan, const int32_t *rows, int64_t count, void *ws, size_t ws_bytes,
-                     unsigned long long *next, int *err, Ctx &c);
+                     const int2 *rspan, const int32_t *rows, int64_t count, int64_t max_alen, void *ws,
+                     size_t ws_bytes, unsigned long long *next, int *err, Ctx &c);
 
 // batched.cu: one instance of a batch, with its place in the stacked arrays.
 struct BatchInst {

@@ -1767,7 +1767,7 @@ static int run_all(const NumP &a, const spgemm_csr &A, const spgemm_csr &B, spge
                 const bool cursors = dense_by_window(ns + (f32 ? nd : nf), c.nsm, max_alen, gws_bytes);
                 const int32_t *d = cursors && f32 ? r + nd : r;
                 const int64_t dense = !cursors ? nd + nb + nf + ns : nb + (f32 ? nf : nd);
-                SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, d, dense, gws, gws_bytes, &st->next_row, err, c));
+                SG_TRY(launch_num_dense(DT, A, B, C, bdesc, rspan, d, dense, max_alen, gws, gws_bytes, &st->next_row, err, c));
                 if (!cursors) break;
                 if (f32) SG_TRY(run_window<V>(a, r, nd, err, gws, gws_bytes, max_alen, c));
                 const int64_t rest = f32 ? ns : nf + ns;
