@@ -502,7 +502,8 @@ int launch_scatter_cls(int64_t n, const uint8_t *cls, int32_t *rows, DevState *s
 // chain of loads, and with eight rows a thread a handful of blocks walked eight
 // such chains one after another).  Measured, k_scan_apply<true> with 8 -> these:
 // 4096 rows 12.3 -> 8.2 us, 8192 20.4 -> 10.2, 20,001 16.4 -> 8.9, 2.1 M and
-// 79,507 together 49 -> 37 (one a thread there 41).
+// 79,507 together 49 -> 37 (one a thread there 41; 39 since classing a row takes
+// divisions, at six blocks an SM: 43 with the 60 registers it takes unasked).
 constexpr int SCAN_BS = 256, SCAN_PT = 8, SCAN_BIN_PT = 4;
 constexpr int64_t SCAN_FEW = 131072;
 
@@ -591,14 +592,15 @@ struct ScanBins {
 constexpr int64_t SCAN_DIRECT = 4096;
 
 template <bool BINS, bool SUMMED, int PT>
-__global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x, int64_t n,
+__global__ void __launch_bounds__(SCAN_BS, PT == SCAN_BIN_PT ? 6 : 0) k_scan_apply(int64_t *__restrict__ x, int64_t n,
                                                         const long long *__restrict__ tile_sums, long long *total,
                                                         ScanBins b) {
     __shared__ long long sh[SCAN_BS / 32];
     __shared__ long long tot;
     __shared__ unsigned long long hist[NBINS];
-    __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS];
+    __shared__ int ccnt[NCLS], cnnz[NCLS], cwords[NCLS], narrow_flops;   // at most NARROW_FLOPS a row
     if (BINS) {
+        if (threadIdx.x == 0) narrow_flops = 0;
         if (threadIdx.x < NBINS) hist[threadIdx.x] = 0;
         if (threadIdx.x < NCLS) ccnt[threadIdx.x] = cnnz[threadIdx.x] = cwords[threadIdx.x] = 0;
     }
@@ -632,7 +634,7 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
 #pragma unroll
     for (int j = 0; j < PT; j++) {
         const int64_t i = base + j;
-        int bin = BIN_EMPTY;
+        int bin = BIN_EMPTY, nf = 0;
         if (i < n) {
             const long long c = v[j], f = b.flops[i];
             bin = c > 0 ? num_bin(c, f) : BIN_EMPTY;
@@ -640,6 +642,7 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
             b.bins[i] = (uint8_t)bin;
             if (bin == BIN_HUGE) atomicMax((unsigned long long *)&b.st->max_row_nnz, (unsigned long long)c);
             int k = bin == BIN_NARROW ? CLS_NARROW : CLS_NONE;
+            if (bin == BIN_NARROW) nf = (int)f;
             if (bin >= 2 && bin <= BIN_HUGE) {
                 const int words = b.rspan[i].y;
                 const bool listed = b.nlo && b.nlo[i] >= 0 && b.nwords[i] <= NARROW_NMAX;
@@ -652,9 +655,12 @@ __global__ void __launch_bounds__(SCAN_BS) k_scan_apply(int64_t *__restrict__ x,
             b.cls[i] = (uint8_t)k;
         }
         warp_hist(hist, i < n, bin);
+        nf = __reduce_add_sync(0xffffffffu, nf);
+        if ((threadIdx.x & 31) == 0 && nf) atomicAdd(&narrow_flops, nf);
     }
     __syncthreads();
     const int t = threadIdx.x;
+    if (t == 0 && narrow_flops) atomicAdd(&b.st->narrow_flops, (unsigned long long)narrow_flops);
     if (t < NBINS && hist[t]) atomicAdd((unsigned long long *)&b.st->bin_count[1][t], hist[t]);
     if (t == BIN_NARROW && hist[t]) atomicAdd((unsigned long long *)&b.st->cls_count[CLS_NARROW], hist[t]);
     if (t < NCLS && ccnt[t]) {

@@ -114,6 +114,7 @@ struct spgemm_handle_s {
     int64_t max_row_nnz = 0;
     ClsInfo cls;              // numeric rows by class (symbolic)
     size_t num_gws = 0;   // bytes of the second-level maps numeric needs
+    int64_t narrow_flops = 0;   // products of the rows of CLS_NARROW
     int num_lists = 0;        // first class of the numeric row lists built (0 = none)
     bool lists_in_graph = false;   // a captured call makes them when its graph runs
     bool b_sorted = false;    // every row of B strictly ascending (symbolic)
@@ -343,12 +344,30 @@ static int lanes_for(double x, int lo = 8) {
     return g;
 }
 
-// Lanes per row, doubled while all rows fit less than one wave of warps (32
-// an SM) and a row has work for them: a row's chain of steps is then the
-// whole kernel.
+// Lanes per row of the narrow symbolic kernel, doubled while all rows fit less than
+// one wave of warps (32 an SM) and a row has work for them: a row's chain of steps is
+// then the whole kernel.
 static int widen(int lanes, int64_t rows, double work, int nsm) {
     while (lanes < 32 && rows * lanes < (int64_t)nsm * 32 * 32 && work > 2.0 * lanes) lanes *= 2;
     return lanes;
+}
+
+// Lanes per row of the narrow numeric kernels: a chunk of so many consecutive entries
+// of a row of B a step, so they follow the mean length of the rows of B (4 to 8
+// entries, else 8), and more where the rows are too few to fill the chip and have
+// the products for them: 32 (the window kernel) while that fits one wave of warps, 8
+// for rows of B of 3 to 8 entries while 4 lanes fit one (of up to 4 entries, half of
+// one with 8), 16 for longer ones while that fits.  Rows of 3000 products, FP32, us with 4 / 8
+// / 16 lanes: rows of B of 8, 9700 rows 129 / 82 / 127, 38,000 433 / 287 / 478; of 24,
+// 6000 104 / 63 / 53, 13,000 115 / 90 / 101; of 3, 9700 184 / 178 / 291, 19,000 261 /
+// 317 / 608; 5000 rows of 4096 products over rows of B of 8 take 98 with 32 and 111
+// with 16.
+static int narrow_lanes(double blen, int64_t rows, double work, int nsm) {
+    const int64_t wave = (int64_t)nsm * 32 * 32;
+    auto fits = [&](int lanes) { return 10 * rows * lanes <= 11 * wave && work > lanes; };
+    if (fits(32)) return 32;
+    if (blen > 8.0) return fits(16) ? 16 : 8;
+    return work > 8.0 && (blen > 4.0 ? rows * 4 < wave : rows * 16 < wave + wave / 8) ? 8 : 4;
 }
 
 // Workspace offsets.  [bins | classes | rows | B descriptors | B block ranges |
@@ -476,6 +495,7 @@ int spgemm_symbolic(spgemm_handle h, const spgemm_csr *A, const spgemm_csr *B, i
         if (bitmaps)
             for (int b = 0; b < NBINS; b++) h->sym_counts[b] = h->hstate->sym_hist[b];
         h->mean_flops = (double)h->hstate->flops_total / (double)n;
+        h->narrow_flops = (int64_t)h->hstate->narrow_flops;
         memcpy(h->num_counts, h->hstate->bin_count[1], sizeof(h->num_counts));
         for (int k = 0; k < NCLS; k++) {
             h->cls.count[k] = h->hstate->cls_count[k];
@@ -570,19 +590,23 @@ int spgemm_numeric(spgemm_handle h, int dtype, const spgemm_csr *A, const spgemm
         h->num_lists = h->lists_in_graph ? 0 : first_list;
     }
     if (h->num_counts[BIN_NARROW] > 0) {
-        // lanes per row: a chunk of G consecutive entries of a row of B per
-        // step, so G follows the mean length of the rows of B
         const double mean_blen = (double)B->nnz / (double)(B->nrows > 0 ? B->nrows : 1);
-        int gn = h->g_narrow_num ? h->g_narrow_num : (mean_blen <= 8.0 ? 4 : 8);
         const int64_t count = h->cls.count[CLS_NARROW];
         const int32_t *list = count < n ? rows + (listed - count) : nullptr;
-        if (!h->g_narrow_num) gn = widen(gn, count, h->mean_flops, h->nsm);
+        // (the products of the narrow rows: those of other rows say nothing about them)
+        const double mean = (double)h->narrow_flops / (double)count;
+        const int gn = h->g_narrow_num ? h->g_narrow_num : narrow_lanes(mean_blen, count, mean, h->nsm);
         if (gn == 32) {
-            const bool block = count < (int64_t)h->nsm * 8 && h->mean_flops >= 512.0;
+            // a block a row while the rows are fewer than eight an SM and long enough
+            // to share out: FP64, 1200 rows of 256 products 12 us by warps, 15 by
+            // blocks, of 512 15 and 15, of 1024 21 and 18, of 8000 99 and 53; 150 of 512
+            // 15 and 9, of 8000 100 and 21; 2400 of 1024 24 and 29
+            const bool block = count < (int64_t)h->nsm * 8 && mean >= 512.0;
             SG_TRY(launch_num_window(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, list, count, block, NARROW_NMAX,
                                      "numeric.narrow", &h->dstate->err, c));
-        } else
-        SG_TRY(launch_num_narrow(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, list, count, &h->dstate->err, gn, c));
+        } else {
+            SG_TRY(launch_num_narrow(dtype, *A, *B, *C, bdesc, nlo, nwords, ulist, list, count, &h->dstate->err, gn, c));
+        }
     }
     return launch_numeric(dtype, h->f64_native, *A, *B, *C, bins, bdesc, rspan, rows, h->num_counts,
                           h->cls, NarrowInfo{nlo, nwords, ulist}, h->dstate, bsplit, gws, h->num_gws, h->max_row_nnz, tune, h->b_sorted,

@@ -54,6 +54,7 @@ struct DevState {          // lives in device memory, one per handle
     long long cls_count[CLS_SLOTS];
     long long cls_cursor[CLS_SLOTS];
     int cls_nnz[CLS_SLOTS], cls_words[CLS_SLOTS];
+    unsigned long long narrow_flops;   // products of the rows of CLS_NARROW
     unsigned long long next_row;   // rows a kernel has handed out (cleared before it)
     // symbolic phase: whether the 32-slot maps have rows, whether rows are
     // marked; rows of the warps, of the blocks' bitmaps and of the blocks' maps
