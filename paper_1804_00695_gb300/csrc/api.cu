@@ -344,11 +344,12 @@ static int lanes_for(double x, int lo = 8) {
     return g;
 }
 
-// Lanes per row of the narrow symbolic kernel, doubled while all rows fit less than
-// one wave of warps (32 an SM) and a row has work for them: a row's chain of steps is
-// then the whole kernel.
+// Lanes per row of the narrow symbolic kernel, doubled while all rows then fit one
+// wave of warps (32 an SM, a tenth over it) and a row has work for them: a row's chain
+// of steps is then the whole kernel.  9000 rows of 60 entries 38 us with 4 lanes, 29, 28,
+// 33 with 32 (two waves); 25,000 of 12 entries 23 with 4, 28 with 8.
 static int widen(int lanes, int64_t rows, double work, int nsm) {
-    while (lanes < 32 && rows * lanes < (int64_t)nsm * 32 * 32 && work > 2.0 * lanes) lanes *= 2;
+    while (lanes < 32 && 20 * rows * lanes <= 11 * (int64_t)nsm * 32 * 32 && work > 2.0 * lanes) lanes *= 2;
     return lanes;
 }
 

@@ -76,3 +76,30 @@ def test_around_the_lines(cuda_lib, dtype, tag, rows, blen):
     a, b = _csr([(rows, 7, 0, 500), (3, 1, 0, 500)], 500, t), _csr([(500, blen, 5, 24)], 40, t)
     c = sg.Handle().spgemm(a, b)
     assert_matches(c, oracle_product(host_csr(a), host_csr(b), dtype), tag)
+
+
+@pytest.mark.parametrize("rows,alen", [(5000, 60), (9000, 60), (9000, 200), (16000, 30), (25000, 12), (38000, 12)])
+def test_symbolic_lanes(cuda_lib, rows, alen):
+    """No number of lanes set by hand counts the rows much faster."""
+    h = sg.Handle()
+    a, b = _csr([(rows, alen, 0, 400)], 400, torch.float32), _csr([(400, 24, 0, 2000)], 2000, torch.float32)
+
+    def ms():
+        rp = h.symbolic(a, b)[0]
+        h.set_timing(True)
+        best = 1e9
+        for _ in range(5):
+            h.reset_timings()
+            h.symbolic(a, b)
+            best = min(best, h.timings()["symbolic.narrow"][2])
+        h.set_timing(False)
+        return best, rp
+
+    auto, rp = ms()
+    by_hand = []
+    for lanes in (4, 8, 16, 32):
+        h.set_option(sg.OPT_LANES_NARROW_SYMBOLIC, lanes)
+        t, rp2 = ms()
+        by_hand.append(t)
+        assert torch.equal(rp, rp2)
+    assert auto < 1.3 * min(by_hand), (auto, by_hand)
