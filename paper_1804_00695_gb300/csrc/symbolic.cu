@@ -673,7 +673,7 @@ __device__ __forceinline__ void sym_rows(const BitmapP &a, DevState *st, unsigne
         int L = 0;
         if (MAP && nw > a.bw) {
             const int b = a.bins[i];
-            L = !WARP ? SYM_MAP_BLOCK_L : b <= 2 ? 7 : SYM_MAP_L;
+            L = !WARP ? SYM_MAP_BLOCK_L : b <= 2 ? 7 : b == 3 ? 9 : SYM_MAP_L;
         }
         sync();
         for (int64_t pb = 0; pb < plen; pb += NT) {
