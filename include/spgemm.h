@@ -108,7 +108,9 @@ SPGEMM_API int spgemm_symbolic(spgemm_handle handle, const spgemm_csr *A, const 
  * from spgemm_symbolic on this handle for the same A and B (same arrays and
  * sizes), fills C->col_idx and C->values (device, C->nnz elements each) with
  * ascending columns per row.  Values of A, B, C have type dtype.  Does not
- * synchronise.  Errors: SPGEMM_ERR_NOT_SYMBOLIC, SPGEMM_ERR_ARG. */
+ * synchronise, and can be captured in a CUDA graph (the first call after
+ * spgemm_symbolic makes row lists, and puts that step into the graph).
+ * Errors: SPGEMM_ERR_NOT_SYMBOLIC, SPGEMM_ERR_ARG. */
 SPGEMM_API int spgemm_numeric(spgemm_handle handle, int dtype, const spgemm_csr *A,
                    const spgemm_csr *B, spgemm_csr *C, void *stream);
 
@@ -411,9 +413,15 @@ SPGEMM_API int spgemm_compress(spgemm_handle handle, const spgemm_csr *M, int32_
 
 /* Per-bin row counts of the last symbolic and numeric phases on this handle
  * (host array of at least SPGEMM_NBINS int64 each), for tests and tuning.
- * Index 7 counts the narrow rows (SPGEMM_OPT_NARROW): in the symbolic
- * array the rows counted over a window, in the numeric array the rows
- * multiplied over one. */
+ * Index 0 counts the empty rows, index 7 the narrow rows (SPGEMM_OPT_NARROW):
+ * in the symbolic array the rows counted over a window, in the numeric array
+ * the rows multiplied over one.  The other rows are counted in the symbolic
+ * array by an upper bound on their distinct blocks of 32 columns (1: <= 16, 2:
+ * <= 64, 3: <= 256, 4: <= 1024, 5: <= 4096, 6: more; rows with more than 64
+ * compressed pairs for each of these move to wider ones) when B has at most
+ * 1,703,936 columns; with a wider B by the pass that counted them: 1 the first
+ * pass, 2 to 5 the rows of that bound that did not fit it, 6 the bitmap of all
+ * blocks.  In the numeric array they are counted by spgemm_bin_of. */
 #define SPGEMM_NBINS 8
 SPGEMM_API int spgemm_bin_counts(spgemm_handle handle, int64_t *symbolic_bins, int64_t *numeric_bins);
 

@@ -205,9 +205,10 @@ constexpr long long DENSE_FLOPS = 6144;
 // c 64 3.0 -> 1.9; and so do all where the cursors' workspace has no room.  In FP32
 // a row that may hold sums long enough for folds (dense.cu) keeps them.
 // Rows of at most RANK_M_NNZ outputs over rows of B of a few entries choose between
-// dense windows and the rank accumulators in the same way (2000 rows of 3250
-// entries of two products, FP32, rank 351 us over 9000 and 356 over 60,000 columns;
-// 4000 entries of two over 40,000 columns, dense 574).
+// dense windows and the rank accumulators in the same way (2000 rows of 4000
+// entries of two products, FP32, over 40,000 columns 574 us by dense windows, 428 by
+// rank, over 20,000 331 by dense windows; of 3250 entries over 9000 351 by rank, over
+// 60,000 356).
 constexpr int DENSE_BYTES = 88 * 1024;   // a window's accumulators
 constexpr int DENSE_FEW = 2;
 constexpr int DENSE_FOLD_ALEN = 1024;    // entries of a row of A from which on folds begin

@@ -12,10 +12,10 @@
 //   map;
 // * bin 5 (<= 4096 outputs): a block per row, shared hash map;
 // * rows with many products over their span, or more outputs than the rank
-//   accumulators hold, when the rows of B are sorted: windows of a dense
-//   accumulator (dense.cu);
+//   accumulators hold and enough products in a window, when the rows of B are
+//   sorted: windows of a dense accumulator (dense.cu);
 // * the rest of bin 6: column windows walked by cursors when the rows of B
-//   are sorted (the split table of dense.cu would outgrow B), else a two-level hash map (shared, then global memory: Section
+//   are sorted, else a two-level hash map (shared, then global memory: Section
 //   3.3's multilevel memory).
 //
 // Output rows have ascending columns.  FP64 values are accumulated as

@@ -15,7 +15,7 @@
 // with a 256-slot map of row i's blocks (shared memory), the others to a block
 // each with a dense bitmap of all columns (shared memory up to TRI_SMEM_WORDS
 // words, else a bitmap per block in global memory), set from row i and cleared
-// again after it.  The columns of the rows L_k are dealt out flat, 32
+// when the block meets another row.  The columns of the rows L_k are dealt out flat, 32
 // consecutive ones a step, as the products are in rank.cu.
 //
 // The paper compresses the right-hand operand into (block, mask) pairs
