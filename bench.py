@@ -223,6 +223,51 @@ def measured_peaks():
         return None
 
 
+LINE_MAX = 2400   # characters of the bench line: what records it keeps the end of a program's output only
+
+
+def _all_ok(d):
+    """Whether every parity verdict in a workload's result holds."""
+    ok = True
+    for k, v in d.items():
+        if k == "parity":
+            ok &= all(x for x in v.values() if isinstance(x, bool))
+        elif isinstance(v, dict):
+            ok &= _all_ok(v)
+    return ok
+
+
+def short_line(line):
+    """The bench line proper: the keys of the contract, floats to six digits,
+    per-kernel times and the other workloads' details left out (of each of
+    those the value, and whether all its parity checks held)."""
+    def digits(x):
+        if isinstance(x, float):
+            return float(f"{x:.6g}")
+        return {k: digits(v) for k, v in x.items()} if isinstance(x, dict) else x
+
+    out = {k: v for k, v in line.items() if k not in ("kernels_ms_per_step", "kernels_ms_note", "secondary")}
+    if out.get("roofline"):
+        out["roofline"] = {k: ({q: w for q, w in v.items() if q != "peak_source"} if isinstance(v, dict) else v)
+                           for k, v in out["roofline"].items() if k != "peak_source"}
+    if "secondary" in line:
+        out["secondary"] = {
+            name: {"error": d["error"][:60]} if "error" in d
+            else {**({"value": d["metric_value"], "ms": d["ms_per_step"]} if "metric_value" in d else {}), "ok": _all_ok(d)}
+            for name, d in line["secondary"].items()}
+    return digits(out)
+
+
+def emit(line):
+    """Everything that was measured as one JSON object on standard error, then
+    the bench line on standard output."""
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    text = json.dumps(short_line(line))
+    if len(text) > LINE_MAX:   # never at the expense of the line itself
+        text = json.dumps({k: v for k, v in short_line(line).items() if k != "secondary"})
+    print(text, flush=True)
+
+
 def run_reference(args, rank, world):
     if rank != 0:
         return
@@ -506,7 +551,7 @@ def main():
                 "cpu_baseline": cpu}
         if secondary is not None:
             line["secondary"] = secondary
-        print(json.dumps(line), flush=True)
+        emit(line)
     if dist:
         dist.destroy_process_group()
 
