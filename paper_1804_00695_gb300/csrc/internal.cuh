@@ -80,7 +80,7 @@ constexpr int NBINS = SPGEMM_NBINS;
 //   SYM_MARK_WARP: up to SYM_WARP_PAIRS pairs over at most SYM_WARP_WORDS
 //     blocks: a warp and a bitmap of the span; over more, up to SYM_MAP_PAIRS, or
 //     SYM_MAP_WIDE_PAIRS over more than SYM_MAP_WIDE_WORDS: a warp and a map;
-//   SYM_MARK_MAP: up to SYM_MAP_BLOCK_PAIRS pairs, and one for 24 blocks of the
+//   SYM_MARK_MAP: up to SYM_MAP_BLOCK_PAIRS pairs, and one for 28 blocks of the
 //     span, over more than SYM_MAP_BLOCK_WORDS: a block and a map;
 //   SYM_MARK_BLOCK: the others: a block and a bitmap.
 // Why the lines lie there (one GB300, whole symbolic call): a block's bitmap is
@@ -88,14 +88,16 @@ constexpr int NBINS = SPGEMM_NBINS;
 // an SM, so that rows go through it one at a time.  Bitmap -> map, rows over
 // 3000 / 12,000 / 50,000 blocks: 200,000 of 40 pairs 784 -> 347, 1613 -> 353,
 // 5509 -> 355 us; 78,125 of 256 417 -> 323, 738 -> 336, 2295 -> 340; 66,666 of 300
-// 370 (bitmap kept), 650 -> 305, 1979 -> 316; 33,333 of 600 265 and 412 (kept),
-// 1082 -> 477; 20,000 of 1000 214 and 305 (kept), 729 -> 401; 10,000 of 2000 185 and
-// 232 (kept), 442 -> 377.  A hundred rows of 400 take 101 by bitmaps, 111 by maps.
+// 370 (bitmap kept), 650 -> 305, 1979 -> 316; 150,000 of 600 758 (kept), 1364 ->
+// 1195, 4409 -> 1267; 20,000 of 1000 214 and 305 (kept), 729 -> 401; 50,000 of 1500
+// 409 and 660 (kept), 1679 -> 1094.  (A hundred rows of 400 take 101 by bitmaps, 111
+// by maps, of 600 100 and 124; a warp's map of 700 pairs, 0.7 full, takes 1.69 ms for
+// 150,000 rows over 10,000 blocks where bitmaps take 1.40.)
 // A wider B goes through the optimistic first pass and the lists by bin.
 constexpr int64_t SYM_BITMAP_WORDS = 53248;   // 208 KB
 constexpr int SYM_WARP_WORDS = 2048;
 constexpr long long SYM_FIRST_PAIRS = 32, SYM_WARP_PAIRS = 4096;
-constexpr long long SYM_MAP_PAIRS = 256, SYM_MAP_WIDE_PAIRS = 512, SYM_MAP_BLOCK_PAIRS = 2048;
+constexpr long long SYM_MAP_PAIRS = 256, SYM_MAP_WIDE_PAIRS = 640, SYM_MAP_BLOCK_PAIRS = 2048;
 constexpr int SYM_MAP_L = 10, SYM_MAP_BLOCK_L = 12;   // slots of the largest maps (log2): two for every pair
 constexpr int SYM_MAP_WIDE_WORDS = 8192, SYM_MAP_BLOCK_WORDS = 12288;
 static_assert((2 << SYM_MAP_L) <= SYM_WARP_WORDS, "a warp's map lies where its bitmap does");
@@ -104,7 +106,7 @@ __host__ __device__ inline int sym_mark(long long cpairs, int words) {
     if (cpairs <= SYM_FIRST_PAIRS) return 0;
     if (words <= SYM_WARP_WORDS) return cpairs <= SYM_WARP_PAIRS ? SYM_MARK_WARP : SYM_MARK_BLOCK;
     if (cpairs <= (words > SYM_MAP_WIDE_WORDS ? SYM_MAP_WIDE_PAIRS : SYM_MAP_PAIRS)) return SYM_MARK_WARP;
-    return words > SYM_MAP_BLOCK_WORDS && cpairs <= SYM_MAP_BLOCK_PAIRS && cpairs * 24 <= words ? SYM_MARK_MAP : SYM_MARK_BLOCK;
+    return words > SYM_MAP_BLOCK_WORDS && cpairs <= SYM_MAP_BLOCK_PAIRS && cpairs * 28 <= words ? SYM_MARK_MAP : SYM_MARK_BLOCK;
 }
 
 // Numeric bins by exact output count (and product count):
